@@ -42,10 +42,10 @@ extern "C" {
  * x: BF16 [cin][D][H][W]; w: BF16 [cout][cin][27]; b: FP32 [cout] or null (zero);
  * y: BF16 [cout][D][H][W], rounded to nearest even from the FP32 sum.
  * Runs on the tensor cores (tcgen05 MMAs, BF16 operands, FP32 accumulation in tensor
- * memory) as an implicit GEMM over tiles of 8 x 16 voxels of one plane: a TMA box brings
- * the tile of x with its halo, and the 27 taps are shifted views of it. Two scratch copies
- * are allocated and freed in stream order (cudaMallocAsync): x with its channels padded to
- * a multiple of 32 (BF16, group-major) and the weights packed for the MMAs. A wait inside
+ * memory) as an implicit GEMM over tiles of 8 x 16 voxels of up to four planes: TMA boxes
+ * bring the tile of x with its halo, and the 27 taps are shifted views of it. The scratch is
+ * allocated and freed in stream order (cudaMallocAsync): x with its channels padded to
+ * a multiple of 16 (BF16, group-major) and the weights packed for the MMAs. A wait inside
  * the kernel that gives up (not expected in operation) writes NaN to the outputs of its
  * tile. FWI_E_INVAL for sizes the tiling cannot take (D > 65535); FWI_E_CUDA also when the
  * scratch cannot be allocated. */
@@ -66,10 +66,13 @@ int64_t fwi_nn_conv3d_backward_weight_work(int cin, int cout, int D, int H, int 
 
 /* dw[co][ci][t] = sum_p dy[co][p] x[ci][p + t - 1] and db[co] = sum_p dy[co][p]: the
  * gradients of sum(dy * y) with respect to the weights and biases. On the tensor cores:
- * per slice of 2048 voxels one GEMM of the im2col matrix of x (with a row of ones for db)
- * against dy taken as three BF16 parts per value (so the products keep FP32 accuracy),
- * FP32 partial sums into `work`, then the slices added in order. Copies of x
- * (channels-last) and of the split dy are allocated and freed in stream order.
+ * per slice of at most 6144 voxels the products of dy, taken as three BF16 parts per value
+ * (so they keep FP32 accuracy; each part has its own FP32 sum), with the shifted tiles of x,
+ * the parts' sums into `work`, then the slices added in order. Tiles that reach over the
+ * grid's edge add dy = 0 there, so a non-finite x at the edge can make more taps of its
+ * channel non-finite than the taps that use it. Copies of x (group-major) and of the split
+ * dy (tile-ordered), and on small grids the partial sums, are allocated and freed in stream
+ * order.
  * dy: FP32 [cout][D][H][W]; x: BF16 [cin][D][H][W]; dw: FP32 [cout][cin][27];
  * db: FP32 [cout] or null; work: FP32 scratch (fwi_nn_conv3d_backward_weight_work). */
 fwi_status fwi_nn_conv3d_backward_weight(const float *dy, const uint16_t *x, int cin, int cout, int D, int H, int W,

@@ -1,6 +1,6 @@
 // fwi_conv_tc.cu -- the 3x3x3 convolutions of the learned preconditioner on the
 // fifth-generation tensor cores (tcgen05, sm_103a), as implicit GEMMs with BF16 operands
-// in shared memory and FP32 accumulators in tensor memory (TMEM):
+// and FP32 accumulators in tensor memory (TMEM):
 //
 //   forward         y[co][p]  = act(b[co] + sum_t sum_ci w[co][ci][t] x[ci][p + off(t)])
 //   backward data   dx[ci][p] = sum_t sum_co w[co][ci][t] dy[co][p - off(t)]
@@ -9,14 +9,16 @@
 // t one of the 27 taps (kz, ky, kx; kx fastest), out-of-grid taps reading zero. Products
 // of BF16 values are exact; the FP32 gradients of the backward passes enter as three BF16
 // parts (hi, lo, lo2 with hi + lo + lo2 = dy to 2^-24), so their products stay exact too.
-// Operands use the no-swizzle canonical layouts: a core matrix is 8 rows of 16 bytes
-// stored contiguously; LBO is the byte stride between core matrices along K and SBO along
-// M (or N), in both K-major and MN-major operands. One thread issues the tcgen05.mma and
-// commits them to an mbarrier; the epilogue reads the accumulator with tcgen05.ld.
 //
-// The forward and backward-data passes use the tile form (tile_conv_kernel): a TMA box of
-// the input with its halo, and the 27 taps as shifted MMA views of it. The weight gradient
-// (wgrad_kernel) gathers im2col rows from a channels-last copy into an MN-major operand.
+// All three read their activations from a channel-group-major copy src[g][z][y][x][8]
+// (groups of 8 channels, zero past the real ones): a TMA box of a tile of 8 (x) x 16 (y)
+// voxels of a plane with its halo lands in shared memory as [g][18][10][8], zero outside
+// the grid, and the 8 x-voxels of a row at any tap shift are one 128-byte core matrix of
+// the no-swizzle canonical layouts (8 rows of 16 bytes stored contiguously; LBO is the
+// byte stride between core matrices along K and SBO along M or N, in K-major and MN-major
+// operands). So the taps are shifted views of the box: no thread gathers anything. One
+// thread issues the tcgen05.mma and commits them to mbarriers, one the copies; the
+// epilogue reads the accumulators with tcgen05.ld.
 //
 // Every mbarrier wait is bounded (about a second). A block whose wait gives up waits
 // (bounded) for what it issued, writes NaN to its outputs (so the caller's loss turns
@@ -26,38 +28,52 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 #include "fwi_conv_tc.h"
 
 namespace fwi_tc {
 namespace {
 
-constexpr int kM = 128;          // MMA M: voxels (forward, backward data) or tap-channel rows
-constexpr int kKC = 64;          // K per chunk of the weight gradient: 4 MMAs of K = 16
-constexpr int kThreads = 256;    // threads of a weight-gradient block
-constexpr int kMaxN = 256;       // output channels per block (MMA N <= 256)
+constexpr int kM = 128;           // MMA M: the voxels of a tile, or the gradient rows of the weight gradient
+constexpr int kMaxN = 256;        // output channels per block (MMA N <= 256)
+constexpr int kSms = 152;
 constexpr int kSmPerSM = 233472;  // shared memory of an SM (228 KB); 1 KB more is reserved per block
-constexpr int kMinBlocks = 4;     // blocks per SM the register budget allows (64 registers)
+constexpr int kSmBlock = 230400;  // dynamic shared memory a block can have beside 2 KB of static
+constexpr int kTmemCols = 512;    // TMEM columns of an SM
 constexpr long long kWaitCycles = 2000000000LL;  // about a second
+
+constexpr int kTX = 8, kTY = 16;              // tile of one plane (x, y)
+constexpr int kBX = kTX + 2, kBY = kTY + 2;   // staged box with the halo
+constexpr int kRowBytes = kBX * 16;           // one staged row of a group: 160 bytes
+constexpr int kGroupBytes = kRowBytes * kBY;  // one staged group of a plane: 2880 bytes
 
 __device__ __forceinline__ unsigned su32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 
 // shared-memory matrix descriptor, no swizzle: start, leading (K) and stride (M/N) byte
-// offsets in 16-byte units, descriptor version 1 (bit 46)
+// offsets in 16-byte units, descriptor version 1 (bit 46). Shared addresses fit the 14-bit
+// field, so a view at a byte offset is the descriptor plus offset / 16.
 __device__ __forceinline__ uint64_t smem_desc(unsigned addr, unsigned lbo, unsigned sbo) {
   return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
          ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
 }
 // instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), BF16 A and B
 // (bits 7-9, 10-12 = 1), N / 8 at bit 17, M / 16 at bit 24; both operands K-major (a caller
-// sets bit 15 for an MN-major A)
+// sets bit 15 for an MN-major A, bit 16 for an MN-major B)
 __host__ __device__ constexpr uint32_t instr_desc(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
 }
 
-__device__ __forceinline__ void bar_init(uint64_t *b) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(b)) : "memory");
+__device__ __forceinline__ void bar_init(uint64_t *b, int count = 1) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(b)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(uint64_t *b) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(b)) : "memory");
+}
+__device__ __forceinline__ void bar_expect(uint64_t *b, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(b)), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ bool bar_done(uint64_t *b, unsigned parity) {
   unsigned d;
@@ -75,510 +91,127 @@ __device__ __forceinline__ bool bar_wait(uint64_t *b, unsigned parity) {
     if (clock64() - t0 > kWaitCycles) return false;
   return true;
 }
-
-// xcl[p][c] = x[c][p] for c < cin, zero for cin <= c < cp: thread per voxel and 8 channels
-__global__ void to_channels_last(const uint16_t *__restrict__ x, int64_t nv, int cin, int cp, uint16_t *__restrict__ xcl) {
-  const int groups = cp / 8;
-  const int64_t total = nv * groups;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = i % nv;
-    const int c0 = (int)(i / nv) * 8;
-    uint32_t v[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int e = 0; e < 8; e++)
-      if (c0 + e < cin) v[e >> 1] |= (uint32_t)__ldg(x + (int64_t)(c0 + e) * nv + p) << (16 * (e & 1));
-    *reinterpret_cast<uint4 *>(xcl + p * cp + c0) = make_uint4(v[0], v[1], v[2], v[3]);
-  }
+// one thread of a converged warp, by a predicate the compiler knows to be single: MMAs issued
+// under it take their descriptors from uniform registers (issued under threadIdx.x == 0 they
+// cost about 45 clocks each, whatever their size)
+__device__ __forceinline__ bool elect_one() {
+  unsigned e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+  return e != 0;
+}
+// D (TMEM columns at d) (+)= A B, A in shared memory (descriptor) or TMEM (column address). A
+// descriptor comes as its two halves: a view at a byte offset differs in the low half only
+// (start address field), so the issuing thread's arithmetic stays 32-bit.
+__device__ __forceinline__ void mma_ss(unsigned d, unsigned alo, unsigned ahi, unsigned blo, unsigned bhi, uint32_t idesc,
+                                       unsigned acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %6, 0;\n\tmov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}" ::"r"(d),
+      "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc)
+      : "memory");
+}
+__device__ __forceinline__ void mma_ts(unsigned d, unsigned a, unsigned blo, unsigned bhi, uint32_t idesc, unsigned acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 b, {%2, %3};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, p;\n\t}" ::"r"(d),
+      "r"(a), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc)
+      : "memory");
+}
+// the barrier completes when every MMA this thread issued so far has
+__device__ __forceinline__ void mma_commit(uint64_t *b) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(b)) : "memory");
+}
+__device__ __forceinline__ void tmem_alloc(unsigned *slot, int cols) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(slot)), "r"(cols) : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_free(unsigned tmem, int cols) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
+}
+__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld16(uint32_t r[16], unsigned a) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(a));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+// 16 columns of this thread's TMEM lane
+__device__ __forceinline__ void tmem_st16(unsigned a, const uint4 v[4]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(a),
+      "r"(v[0].x), "r"(v[0].y), "r"(v[0].z), "r"(v[0].w), "r"(v[1].x), "r"(v[1].y), "r"(v[1].z), "r"(v[1].w),
+      "r"(v[2].x), "r"(v[2].y), "r"(v[2].z), "r"(v[2].w), "r"(v[3].x), "r"(v[3].y), "r"(v[3].z), "r"(v[3].w)
+      : "memory");
 }
 
-// ---- weight gradient: dW[m][co] = sum_p A[p][m] dy[co][p], m = t Cp + ci (tap t, input
-// channel ci) and one more row m = 27 Cp of ones (the bias gradient), over a slice of
-// kSlice voxels per block; then the slices summed in order.
-//   - A is the im2col matrix of x in MN-major layout: a core matrix is 8 voxels (along K)
-//     of 16 bytes along M (8 channels of one tap), so a row is one 16-byte load from the
-//     channels-last copy; core (mg, kg) at mg * 1024 + kg * 128 (LBO = 128 along K, SBO =
-//     1024 along M);
-//   - B is the gradient in K-major layout, three BF16 parts per channel: a core row is 8
-//     consecutive voxels of one channel and part (16 bytes of the split copy), core (kg, ng)
-//     at kg * (N / 8) * 128 + ng * 128; each chunk runs 3 x 4 MMAs into one accumulator.
-constexpr int kSlice = 2048;          // voxels per block (K per block before the split)
-constexpr int kWgSbo = 1024;          // A: bytes between cores along M (8 cores along K)
-constexpr int kWgABytes = 16 * kWgSbo;  // 128 rows x 64 voxels
-
-// dys[s][co][p] = part s of dy[co][p] (as split_channels_last), zero for co >= cout or
-// p >= nv: rows of nvp = nv rounded up to kSlice voxels
-__global__ void split_channels_first(const float *__restrict__ dy, int64_t nv, int64_t nvp, int cout, int cop,
-                                     uint16_t *__restrict__ dys) {
-  const int64_t total = (int64_t)cop * nvp;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = i % nvp;
-    const int co = (int)(i / nvp);
-    float r = (co < cout && p < nv) ? __ldg(dy + (int64_t)co * nv + p) : 0.f;
-#pragma unroll
-    for (int part = 0; part < 3; part++) {
-      const uint16_t h = __bfloat16_as_ushort(__float2bfloat16_rn(r));
-      dys[((int64_t)part * cop + co) * nvp + p] = h;
-      r -= __uint_as_float((uint32_t)h << 16);
-    }
-  }
-}
-
-__global__ void __launch_bounds__(kThreads, kMinBlocks)
-    wgrad_kernel(const uint16_t *__restrict__ xcl, const uint16_t *__restrict__ dys, int cp, int cop, int nt_n,
-                 int tmem_cols, int mrows, int D, int H, int W, int64_t nvp, float *__restrict__ part) {
-  extern __shared__ __align__(1024) unsigned char sm[];
-  const int bpart = nt_n * kKC * 2;  // one part's B chunk
-  const int bbuf = 3 * bpart;
-  uint64_t *done = reinterpret_cast<uint64_t *>(sm + 2 * kWgABytes + 2 * bbuf);  // [2]
-  unsigned *tslot = reinterpret_cast<unsigned *>(done + 2);
-  int *abort_flag = reinterpret_cast<int *>(tslot + 2);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t nv = (int64_t)D * H * W;
-  // the row tiles of a slice are neighbours in the grid, so they read its voxels while L2
-  // still holds them
-  const int mt = blockIdx.x, slice = blockIdx.y, nt = blockIdx.z;
-  const int64_t v0 = (int64_t)slice * kSlice;
-  const unsigned lbo_b = (unsigned)(nt_n / 8) * 128u;
-  const int nchunk = kSlice / kKC;
-  if (tid == 0) {
-    bar_init(&done[0]);
-    bar_init(&done[1]);
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)),
-                 "r"(tmem_cols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const unsigned tmem = *tslot;
-  const uint32_t idesc = instr_desc(nt_n) | (1u << 15);  // A MN-major
-
-  int issued = 0;
-  bool ok = true;
-  for (int c = 0; c < nchunk; c++) {
-    const int s = c & 1;
-    unsigned char *sa = sm + s * kWgABytes;
-    unsigned char *sb = sm + 2 * kWgABytes + s * bbuf;
-    if (c >= 2 && !bar_wait(&done[s], ((c - 2) >> 1) & 1)) atomicExch(abort_flag, 1);
-    const int64_t pc = v0 + (int64_t)c * kKC;  // first voxel of the chunk
-    // A: 16 x 8 cores of 8 rows (voxels): 1024 rows, 4 per thread
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      const int r = tid + j * kThreads;  // row id: (mg, kg, row)
-      const int mg = r >> 6, kg = (r >> 3) & 7, rw = r & 7;
-      const int m0 = mt * 128 + mg * 8;
-      const int t = m0 / cp, ci0 = m0 % cp;
-      const int64_t p = pc + kg * 8 + rw;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (p < nv && m0 < mrows) {
-        if (t < 27) {
-          const int vx = (int)(p % W), vy = (int)(p / W % H), vz = (int)(p / W / H);
-          const int qx = vx + t % 3 - 1, qy = vy + t / 3 % 3 - 1, qz = vz + t / 9 - 1;
-          if (qx >= 0 && qx < W && qy >= 0 && qy < H && qz >= 0 && qz < D)
-            v = __ldg(reinterpret_cast<const uint4 *>(xcl + (((int64_t)qz * H + qy) * W + qx) * cp + ci0));
-        } else {
-          v.x = 0x3F80u;  // the ones row: BF16 1.0 in its first element
-        }
-      }
-      *reinterpret_cast<uint4 *>(sa + mg * kWgSbo + kg * 128 + rw * 16) = v;
-    }
-    // B: three parts of nt_n channels x 8 cores of 8 voxels
-    for (int r = tid; r < 3 * nt_n * 8; r += kThreads) {
-      const int part_i = r / (nt_n * 8), rr = r % (nt_n * 8);
-      const int n = rr >> 3, kg = rr & 7;
-      const int co = nt * nt_n + n;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (co < cop)
-        v = __ldg(reinterpret_cast<const uint4 *>(dys + ((int64_t)part_i * cop + co) * nvp + pc + kg * 8));
-      *reinterpret_cast<uint4 *>(sb + part_i * bpart + kg * lbo_b + (n >> 3) * 128 + (n & 7) * 16) = v;
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (*(volatile int *)abort_flag != 0) {
-      ok = false;
-      break;
-    }
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-      for (int pi = 0; pi < 3; pi++)
-#pragma unroll
-        for (int ks = 0; ks < kKC / 16; ks++) {
-          const uint64_t da = smem_desc(su32(sa) + ks * 256, 128, kWgSbo);
-          const uint64_t db = smem_desc(su32(sb) + pi * bpart + 2 * ks * lbo_b, lbo_b, 128);
-          const unsigned acc = (c > 0 || pi > 0 || ks > 0) ? 1u : 0u;
-          asm volatile(
-              "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-              "l"(da), "l"(db), "r"(idesc), "r"(acc)
-              : "memory");
-        }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       su32(&done[s]))
-                   : "memory");
-    }
-    issued = c + 1;  // every thread counts the chunks thread 0 committed
-  }
-  if (*(volatile int *)abort_flag != 0) ok = false;
-  if (issued > 0 && !bar_wait(&done[(issued - 1) & 1], ((issued - 1) >> 1) & 1)) ok = false;
-  ok = __syncthreads_and(ok) != 0;
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  // partial sums of this slice: part[slice][co][m], lanes = consecutive m
-  const int q = warp & 3, chalf = warp >> 2;
-  const int m = mt * 128 + q * 32 + lane;
-  const int cols_half = nt_n / 2;
-  const int mpad = gridDim.x * 128;
-  for (int c0 = chalf * cols_half; c0 < (chalf + 1) * cols_half; c0 += 8) {
-    uint32_t r[8];
-    const unsigned ta = tmem + ((unsigned)(q * 32) << 16) + (unsigned)c0;
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(ta));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int j = 0; j < 8; j++) {
-      const int co = nt * nt_n + c0 + j;
-      part[((int64_t)slice * (gridDim.z * nt_n) + co) * mpad + m] = ok ? __uint_as_float(r[j]) : __uint_as_float(0x7FC00000u);
-    }
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
-}
-
-// dw[co][ci][t] and db[co]: the slices' partial sums added in slice order
-__global__ void wgrad_reduce_kernel(const float *__restrict__ part, int nslice, int ncol, int mpad, int cin, int cout,
-                                    int cp, float *__restrict__ dw, float *__restrict__ db) {
-  const int64_t total = (int64_t)cout * (cin * 27 + 1);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int co = (int)(i / (cin * 27 + 1)), j = (int)(i % (cin * 27 + 1));
-    const bool bias = j == cin * 27;
-    const int ci = bias ? 0 : j / 27, t = bias ? 0 : j % 27;
-    const int m = bias ? 27 * cp : t * cp + ci;
-    float acc = 0.f;
-    for (int sl = 0; sl < nslice; sl++) acc += part[((int64_t)sl * ncol + co) * mpad + m];
-    if (bias) {
-      if (db) db[co] = acc;
-    } else {
-      dw[((int64_t)co * cin + ci) * 27 + t] = acc;
-    }
-  }
-}
-
-}  // namespace
-
-// floats of partial sums conv3d_backward_weight_tc needs
-int64_t conv3d_backward_weight_tc_work(int cin, int cout, int D, int H, int W) {
-  const int cp = (cin + 7) / 8 * 8;
-  const int64_t nv = (int64_t)D * H * W;
-  const int64_t nslice = (nv + kSlice - 1) / kSlice;
-  const int64_t mpad = ((int64_t)27 * cp + 1 + 127) / 128 * 128;
-  const int n16 = (cout + 15) / 16 * 16;
-  const int nt_n = n16 < kMaxN ? n16 : kMaxN;
-  const int64_t ncol = (int64_t)((cout + nt_n - 1) / nt_n) * nt_n;
-  return nslice * ncol * mpad;
-}
-
-cudaError_t conv3d_backward_weight_tc(const float *dy, const uint16_t *x, int cin, int cout, int D, int H, int W,
-                                      float *dw, float *db, float *work, cudaStream_t s) {
-  const int cp = (cin + 7) / 8 * 8;
-  const int cop = (cout + 7) / 8 * 8;
-  const int64_t nv = (int64_t)D * H * W;
-  const int64_t nslice = (nv + kSlice - 1) / kSlice;
-  const int64_t nvp = nslice * kSlice;
-  const int mrows = 27 * cp + 1;
-  const int mtiles = (mrows + 127) / 128;
-  const int n16 = (cout + 15) / 16 * 16;
-  const int nt_n = n16 < kMaxN ? n16 : kMaxN;
-  const int ntiles = (cout + nt_n - 1) / nt_n;
-  if (nslice > 65535 || ntiles > 65535) return cudaErrorInvalidValue;
-  int tmem_cols = 32;
-  while (tmem_cols < nt_n) tmem_cols *= 2;
-  const int max_blocks = 512 / tmem_cols;
-  int smem = 2 * kWgABytes + 2 * 3 * nt_n * kKC * 2 + 64;
-  const int floor_smem = kSmPerSM / (max_blocks + 1) - 1024 + 16;
-  if (smem < floor_smem) smem = floor_smem;
-  if (smem > 232448) return cudaErrorInvalidValue;  // more than a block's shared memory
-  cudaError_t e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  uint16_t *xcl = nullptr, *dys = nullptr;
-  e = cudaMallocAsync(reinterpret_cast<void **>(&xcl), (size_t)nv * cp * sizeof(uint16_t), s);
-  if (e != cudaSuccess) return e;
-  e = cudaMallocAsync(reinterpret_cast<void **>(&dys), (size_t)3 * cop * nvp * sizeof(uint16_t), s);
-  if (e != cudaSuccess) {
-    cudaFreeAsync(xcl, s);
-    return e;
-  }
-  const int64_t xb = (nv * (cp / 8) + 255) / 256, yb = ((int64_t)cop * nvp + 255) / 256;
-  to_channels_last<<<(unsigned)(xb < 65536 ? xb : 65536), 256, 0, s>>>(x, nv, cin, cp, xcl);
-  split_channels_first<<<(unsigned)(yb < 65536 ? yb : 65536), 256, 0, s>>>(dy, nv, nvp, cout, cop, dys);
-  wgrad_kernel<<<dim3((unsigned)mtiles, (unsigned)nslice, (unsigned)ntiles), kThreads, smem, s>>>(
-      xcl, dys, cp, cop, nt_n, tmem_cols, mrows, D, H, W, nvp, work);
-  const int64_t nout = (int64_t)cout * (cin * 27 + 1);
-  wgrad_reduce_kernel<<<(unsigned)((nout + 255) / 256 < 65536 ? (nout + 255) / 256 : 65536), 256, 0, s>>>(
-      work, (int)nslice, ntiles * nt_n, mtiles * 128, cin, cout, cp, dw, db);
-  e = cudaGetLastError();
-  const cudaError_t f1 = cudaFreeAsync(dys, s), f2 = cudaFreeAsync(xcl, s);
-  return e != cudaSuccess ? e : (f1 != cudaSuccess ? f1 : f2);
-}
-
-namespace {
-
-// ---- tile form of the forward and backward-data convolutions. The source is a
-// channel-group-major copy src[g][z][y][x][8] (G groups of 8 channels, zero past the real
-// ones). A block owns an output tile of 8 (x) x 16 (y) voxels of one plane (MMA M = 128,
-// m = 8 y + x) and up to 256 GEMM output channels (N). Per pass of Gp groups one TMA box
-// (10 voxels x 8 channels as one 160-byte row, 18 rows, 3 planes, Gp groups) brings the tile with its halo into shared
-// memory as [g][z][y][x][8], zero outside the grid. The A operand of tap t and group pair
-// (2j, 2j + 1) is then a view of that box: core matrix y = the 8 x-voxels of row y (16 bytes
-// each, contiguous), start at the tap's shifted voxel, SBO = one staged row (160 bytes),
-// LBO = one staged group (8640 bytes). No thread gathers anything.
-// Weights stream per (pass, tap) chunk (N x Gp x 8 BF16, K-major, packed once per call by
-// tile_pack_kernel) through a ring of 4 buffers by bulk copies. One thread drives the copies
-// and the MMAs; all threads run the epilogue.
-constexpr int kTX = 8, kTY = 16;                // output tile (x, y)
-constexpr int kBX = kTX + 2, kBY = kTY + 2;     // staged box with the halo
-constexpr int kGroupBytes = kBX * kBY * 3 * 16;  // one staged group: 8640 bytes
-constexpr int kRowBytes = kBX * 16;             // one staged row: 160 bytes
-constexpr int kRingB = 4;                       // weight chunks in flight
-constexpr int kTileThreads = 128;
-
-// src[g][p][e] = x[8 g + e][p] (zero for channels >= cin)
-__global__ void to_group_major(const uint16_t *__restrict__ x, int64_t nv, int cin, int G, uint16_t *__restrict__ src) {
-  const int64_t total = nv * G;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = i % nv;
-    const int g = (int)(i / nv);
-    uint32_t v[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int e = 0; e < 8; e++)
-      if (8 * g + e < cin) v[e >> 1] |= (uint32_t)__ldg(x + (int64_t)(8 * g + e) * nv + p) << (16 * (e & 1));
-    *reinterpret_cast<uint4 *>(src + ((int64_t)g * nv + p) * 8) = make_uint4(v[0], v[1], v[2], v[3]);
-  }
-}
-
-// src[g][p][e] = part s of dy[co][p] for channel 8 g + e = s cop + co (three BF16 parts,
-// as split_channels_last), zero for co >= cout and for channels past 3 cop
-__global__ void split_group_major(const float *__restrict__ dy, int64_t nv, int cout, int cop, int G,
-                                  uint16_t *__restrict__ src) {
-  const int64_t total = nv * G;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = i % nv;
-    const int g = (int)(i / nv);
-    uint32_t v[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int e = 0; e < 8; e++) {
-      const int c = 8 * g + e, part = c / cop, co = c % cop;
-      if (part >= 3 || co >= cout) continue;
-      float r = __ldg(dy + (int64_t)co * nv + p);
-      uint16_t h = 0;
-      for (int q = 0; q <= part; q++) {
-        h = __bfloat16_as_ushort(__float2bfloat16_rn(r));
-        r -= __uint_as_float((uint32_t)h << 16);
-      }
-      v[e >> 1] |= (uint32_t)h << (16 * (e & 1));
-    }
-    *reinterpret_cast<uint4 *>(src + ((int64_t)g * nv + p) * 8) = make_uint4(v[0], v[1], v[2], v[3]);
-  }
-}
-
-// weight chunks: for N tile nt, pass ps, tap t: N x (Gp x 8) K-major, core (kg, ng) at
-// kg * (N / 8) * 128 + ng * 128. Source channel c = 8 (ps Gp + kg) + kk; forward: w[n][c][t];
-// backward: c = s cop + co, w[co][n][t]
-__global__ void tile_pack_kernel(const uint16_t *__restrict__ w, int n_rows, int n_red, int cop, bool bwd, int nt_n,
-                                 int gp, int npass, int ntiles, uint16_t *__restrict__ out) {
-  const int64_t chunk = (int64_t)nt_n * gp * 8;
-  const int64_t total = (int64_t)ntiles * npass * 27 * chunk;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int kk = (int)(i % 8), row = (int)(i / 8 % 8);
-    const int64_t r = i / 64;
-    const int ng = (int)(r % (nt_n / 8)), kg = (int)(r / (nt_n / 8) % gp);
-    const int64_t q = r / (nt_n / 8) / gp;  // (tile, pass, tap)
-    const int t = (int)(q % 27), ps = (int)(q / 27 % npass), nt = (int)(q / 27 / npass);
-    const int n = nt * nt_n + ng * 8 + row;
-    const int c = 8 * (ps * gp + kg) + kk;
-    uint16_t v = 0;
-    if (n < n_rows) {
-      if (!bwd) {
-        if (c < n_red) v = w[((int64_t)n * n_red + c) * 27 + t];
-      } else {
-        const int part = c / cop, co = c % cop;
-        if (part < 3 && co < n_red) v = w[((int64_t)co * n_rows + n) * 27 + t];
-      }
-    }
-    out[i] = v;
-  }
-}
-
-// the halo box of a tile: x and the 8 channels of a group form one row of 80 elements (the
-// inner coordinate 8 (x0 - 1) is a multiple of 16 bytes), then y, z and the groups
-__device__ __forceinline__ void tma_box(void *dst, const CUtensorMap *tm, int x0, int y0, int z0, int g0, uint64_t *b) {
+// a plane's halo box of a tile: x and the 8 channels of a group form one row of 80 elements
+// (the inner coordinate 8 (x0 - 1) is a multiple of 16 bytes), then y, z and the groups
+__device__ __forceinline__ void tma_box(void *dst, const CUtensorMap *tm, int x0, int y0, int z, int g0, uint64_t *b) {
   asm volatile(
       "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
       "[%6];" ::"r"(su32(dst)),
-      "l"(reinterpret_cast<uint64_t>(tm)), "r"(8 * (x0 - 1)), "r"(y0 - 1), "r"(z0 - 1), "r"(g0), "r"(su32(b))
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(8 * (x0 - 1)), "r"(y0 - 1), "r"(z), "r"(g0), "r"(su32(b))
       : "memory");
 }
 __device__ __forceinline__ void bulk_copy(void *dst, const void *src, unsigned bytes, uint64_t *b) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(b)), "r"(bytes) : "memory");
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                    su32(dst)),
                "l"(src), "r"(bytes), "r"(su32(b))
                : "memory");
 }
 
-template <bool BWD>
-__global__ void __launch_bounds__(kTileThreads)
-    tile_conv_kernel(const __grid_constant__ CUtensorMap tm, const uint16_t *__restrict__ wpack,
-                     const float *__restrict__ bias, int n_out, int nt_n, int tmem_cols, int gp, int npass, int D, int H,
-                     int W, int relu, void *__restrict__ yout) {
-  extern __shared__ __align__(1024) unsigned char sm[];
-  const int a_bytes = kGroupBytes * gp;
-  const int b_bytes = nt_n * gp * 16;  // one chunk
-  unsigned char *sa = sm;
-  unsigned char *sb = sm + (a_bytes + 127) / 128 * 128;
-  uint64_t *loaded = reinterpret_cast<uint64_t *>(sb + kRingB * b_bytes);  // [kRingB]
-  uint64_t *done = loaded + kRingB;                                        // [kRingB]
-  uint64_t *a_full = done + kRingB;
-  unsigned *tslot = reinterpret_cast<unsigned *>(a_full + 1);
-  int *okslot = reinterpret_cast<int *>(tslot + 1);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int ntx = (W + kTX - 1) / kTX;
-  const int x0 = (blockIdx.x % ntx) * kTX, y0 = (blockIdx.x / ntx) * kTY, z0 = blockIdx.y;
-  const int nt = blockIdx.z;
-  const unsigned lbo_b = (unsigned)(nt_n / 8) * 128u;
-  const int nch = npass * 27;
-  const uint16_t *wt = wpack + (int64_t)nt * nch * nt_n * gp * 8;
-
-  if (tid == 0) {
-    for (int i = 0; i < kRingB; i++) {
-      bar_init(&loaded[i]);
-      bar_init(&done[i]);
-    }
-    bar_init(a_full);
-    *okslot = 1;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)),
-                 "r"(tmem_cols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const unsigned tmem = *tslot;
-
-  if (tid == 0) {
-    const uint32_t idesc = instr_desc(nt_n);
-    bool ok = true;
-    int copies = 0, committed = 0;  // weight chunks issued / chunks whose MMAs are committed
-    int a_pending = -1;  // the pass whose box copy has not been waited for
-    auto chunk_src = [&](int c) { return wt + (int64_t)c * nt_n * gp * 8; };
-    for (; copies < kRingB && copies < nch; copies++) bulk_copy(sb + copies * b_bytes, chunk_src(copies), b_bytes, &loaded[copies]);
-    for (int c = 0; c < nch && ok; c++) {
-      const int ps = c / 27, t = c % 27, s = c % kRingB;
-      if (t == 0) {
-        // a new pass: the previous pass's MMAs read the box, so they finish first
-        if (c > 0 && !bar_wait(&done[(c - 1) % kRingB], ((c - 1) / kRingB) & 1)) {
-          ok = false;
-          break;
-        }
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(a_full)), "r"(a_bytes)
-                     : "memory");
-        tma_box(sa, &tm, x0, y0, z0, ps * gp, a_full);
-        a_pending = ps;
-        if (!bar_wait(a_full, ps & 1)) {
-          ok = false;
-          break;
-        }
-        a_pending = -1;
-      }
-      if (!bar_wait(&loaded[s], (c / kRingB) & 1)) {
-        ok = false;
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      // the tap's shift (mirrored for the backward pass), as a staged voxel offset
-      const int dx = t % 3 - 1, dy = t / 3 % 3 - 1, dz = t / 9 - 1;
-      const int sx = BWD ? 1 - dx : 1 + dx, sy = BWD ? 1 - dy : 1 + dy, sz = BWD ? 1 - dz : 1 + dz;
-      const unsigned a0 = su32(sa) + (unsigned)(((sz * kBY) + sy) * kBX + sx) * 16u;
-      const unsigned b0 = su32(sb + s * b_bytes);
-      for (int j = 0; j < gp / 2; j++) {
-        const uint64_t da = smem_desc(a0 + 2 * j * kGroupBytes, kGroupBytes, kRowBytes);
-        const uint64_t db = smem_desc(b0 + 2 * j * lbo_b, lbo_b, 128);
-        const unsigned acc = (c > 0 || j > 0) ? 1u : 0u;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-            "l"(da), "l"(db), "r"(idesc), "r"(acc)
-            : "memory");
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(&done[s]))
-                   : "memory");
-      committed = c + 1;
-      // refill the buffer of chunk c - 1 (its MMAs ran before this chunk's) with chunk c + 3
-      if (c >= 1 && copies < nch) {
-        const int sp = (c - 1) % kRingB;
-        if (!bar_wait(&done[sp], ((c - 1) / kRingB) & 1)) {
-          ok = false;
-          break;
-        }
-        bulk_copy(sb + sp * b_bytes, chunk_src(copies), b_bytes, &loaded[sp]);
-        copies++;
-      }
-    }
-    // copies still in flight land before the shared memory is released
-    if (a_pending >= 0) bar_wait(a_full, a_pending & 1);
-    for (int c = committed; c < copies; c++) bar_wait(&loaded[c % kRingB], (c / kRingB) & 1);
-    if (committed > 0 && !bar_wait(&done[(committed - 1) % kRingB], ((committed - 1) / kRingB) & 1)) ok = false;
-    if (committed < nch) ok = false;
-    *okslot = ok ? 1 : 0;
-  }
-  __syncthreads();
-  const bool ok = *(volatile int *)okslot != 0;
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  // epilogue: warp q reads TMEM lanes 32 q .. 32 q + 31 (tile rows 4 q .. 4 q + 3)
-  const int m = warp * 32 + lane;
-  const int ox = x0 + (m & 7), oy = y0 + (m >> 3);
-  const bool in = ox < W && oy < H;
-  const int64_t nv = (int64_t)D * H * W;
-  const int64_t pe = ((int64_t)z0 * H + oy) * W + ox;
-  for (int c0 = 0; c0 < nt_n; c0 += 8) {
-    uint32_t r[8];
-    const unsigned ta = tmem + ((unsigned)(warp * 32) << 16) + (unsigned)c0;
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(ta));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    if (in) {
+// the three BF16 parts of an FP32 value, and the pattern of its part s
+__device__ __forceinline__ void split3(float v, uint16_t h[3]) {
 #pragma unroll
-      for (int j = 0; j < 8; j++) {
-        const int co = nt * nt_n + c0 + j;
-        if (co >= n_out) continue;
-        if constexpr (BWD) {
-          static_cast<float *>(yout)[(int64_t)co * nv + pe] = ok ? __uint_as_float(r[j]) : __uint_as_float(0x7FC00000u);
-        } else {
-          float v = __uint_as_float(r[j]) + (bias ? __ldg(bias + co) : 0.f);
-          if (relu) v = fmaxf(v, 0.f);
-          static_cast<uint16_t *>(yout)[(int64_t)co * nv + pe] =
-              ok ? __bfloat16_as_ushort(__float2bfloat16_rn(v)) : (uint16_t)0x7FC0;
-        }
-      }
-    }
+  for (int s = 0; s < 3; s++) {
+    h[s] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
+    v -= __uint_as_float((uint32_t)h[s] << 16);
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
+}
+__device__ __forceinline__ uint4 pack8(const uint16_t h[8]) {
+  return make_uint4((uint32_t)h[0] | (uint32_t)h[1] << 16, (uint32_t)h[2] | (uint32_t)h[3] << 16,
+                    (uint32_t)h[4] | (uint32_t)h[5] << 16, (uint32_t)h[6] | (uint32_t)h[7] << 16);
+}
+
+// src[g][p][e] = x[8 g + e][p] (zero for channels >= cin)
+__global__ void __launch_bounds__(256) to_group_major(const uint16_t *__restrict__ x, int64_t nv, int cin,
+                                                      uint16_t *__restrict__ src) {
+  const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  const int g = blockIdx.y;
+  if (p >= nv) return;
+  const uint16_t *q = x + 8 * g * nv + p;
+  uint32_t v[4] = {0u, 0u, 0u, 0u};
+  const int n = cin - 8 * g;
+#pragma unroll
+  for (int e = 0; e < 8; e++)
+    if (e < n) v[e >> 1] |= (uint32_t)__ldg(q + e * nv) << (16 * (e & 1));
+  *reinterpret_cast<uint4 *>(src + ((int64_t)g * nv + p) * 8) = make_uint4(v[0], v[1], v[2], v[3]);
+}
+
+// the split gradient in group-major form: channel s cop + co of src is part s of dy[co], cop
+// the channels rounded up to 8; zero for co >= cout and for groups past 3 cop / 8. A thread
+// reads 8 channels of a voxel once and writes their three parts.
+__global__ void split_group_major(const float *__restrict__ dy, int64_t nv, int cout, int cop, int G,
+                                  uint16_t *__restrict__ src) {
+  const int gq = cop / 8;
+  for (int g = blockIdx.y; g < gq; g += gridDim.y)
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nv; p += (int64_t)gridDim.x * blockDim.x) {
+      uint16_t h[3][8];
+#pragma unroll
+      for (int e = 0; e < 8; e++) {
+        uint16_t t[3];
+        split3(8 * g + e < cout ? __ldg(dy + (int64_t)(8 * g + e) * nv + p) : 0.f, t);
+#pragma unroll
+        for (int s = 0; s < 3; s++) h[s][e] = t[s];
+      }
+#pragma unroll
+      for (int s = 0; s < 3; s++) *reinterpret_cast<uint4 *>(src + ((int64_t)(s * gq + g) * nv + p) * 8) = pack8(h[s]);
+      if (g == 0)
+        for (int z = 3 * gq; z < G; z++) *reinterpret_cast<uint4 *>(src + ((int64_t)z * nv + p) * 8) = make_uint4(0u, 0u, 0u, 0u);
+    }
 }
 
 // cuTensorMapEncodeTiled from the driver, looked up once through the runtime
@@ -597,96 +230,703 @@ EncodeTiled encode_tiled() {
   return fn;
 }
 
-// the tile form over a group-major source of G groups (G a multiple of 4) that `prepare`
-// fills; n_rows GEMM output channels, n_red real source channels (forward: cin; backward:
-// cout, with cop = the part stride)
-template <bool BWD, class Prepare>
-cudaError_t run_tile(const uint16_t *w, const float *b, int n_rows, int n_red, int cop, int G, int D, int H, int W,
-                     int relu, void *y, cudaStream_t s, Prepare prepare) {
+// tensor map of a group-major copy as (x and 8 channels: 8 W, H, D, G) BF16; boxes of one
+// plane, gbox groups: (80, 18, 1, gbox), zero outside the grid
+cudaError_t box_map(CUtensorMap *tm, uint16_t *src, int D, int H, int W, int G, int gbox) {
   const EncodeTiled enc = encode_tiled();
   if (!enc) return cudaErrorNotSupported;
-  const int n16 = (n_rows + 15) / 16 * 16;
-  const int nt_n = n16 < kMaxN ? n16 : kMaxN;
-  const int ntiles = (n_rows + nt_n - 1) / nt_n;
-  int tmem_cols = 32;
-  while (tmem_cols < nt_n) tmem_cols *= 2;
-  // groups per pass: the largest of 12, 8, 4 that divides G and fits shared memory
-  int gp = 0, smem = 0;
-  for (int cand : {12, 8, 4}) {
-    if (G % cand) continue;
-    const int need = (kGroupBytes * cand + 127) / 128 * 128 + kRingB * nt_n * cand * 16 + 2 * kRingB * 8 + 32;
-    if (need <= 200 * 1024) {
-      gp = cand;
-      smem = need;
-      break;
+  std::memset(tm, 0, sizeof(*tm));
+  const cuuint64_t dims[4] = {(cuuint64_t)W * 8, (cuuint64_t)H, (cuuint64_t)D, (cuuint64_t)G};
+  const cuuint64_t pitch[3] = {(cuuint64_t)W * 16, (cuuint64_t)W * H * 16, (cuuint64_t)W * H * D * 16};
+  const cuuint32_t box[4] = {kBX * 8, kBY, 1, (cuuint32_t)gbox};
+  const cuuint32_t step[4] = {1, 1, 1, 1};
+  return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, src, dims, pitch, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+             ? cudaSuccess
+             : cudaErrorInvalidValue;
+}
+
+// ---- forward and backward data. A block owns `planes` consecutive planes of an 8 x 16 tile
+// (one accumulator of M = 128 voxels x nt_n channels each) and up to 256 GEMM output channels.
+// The reduction runs pass by pass over gp channel groups and, in a pass, tap by tap: per
+// (pass, tap) the weights (nt_n x 8 gp BF16, K-major) stream, `taps` taps per copy, through a
+// ring of buffers, and each pair of groups is one MMA per plane, on views of the planes' boxes.
+//
+// Issuing an MMA costs its thread 50 to 150 clocks of descriptor arithmetic and moves to
+// uniform registers (measured), more than an MMA of N = 32 runs (40 clocks): so warp p issues
+// the MMAs of plane p, and the four chains keep the tensor pipe fed. Warp 4 copies.
+//
+// Bound: in the MMA phase the operands' shared-memory reads (M = 128, K = 16: 4 KB of A for
+// any N); the epilogue's stores (8 voxels of a row per channel) overlap it only across the
+// blocks of an SM. Several planes share each weight copy and two of three halo planes: with
+// one plane a block, 28 -> 28 channels moved 90 KB through L2 per 128 voxels, 27 KB now.
+// Measured at 65 x 129 x 129 voxels: forward 28 -> 28 226 -> 142 us, backward data 28 -> 84
+// 1359 -> 546 us (one thread issuing for one plane a block before).
+constexpr int kTileThreads = 160;
+constexpr int kRingB = 4;      // most weight copies in flight
+constexpr int kMaxPlanes = 4;  // output planes of a block
+constexpr int kMaxBox = 2;     // box buffers (passes in flight)
+
+struct TileShape {
+  int nt_n, ntiles;  // GEMM output channels per block, N tiles
+  int gp, npass, G;  // groups per pass, passes, groups of the source (even)
+  int planes, nbox;  // output planes per block, box buffers
+  int taps, ring;    // taps per weight copy (1, 3 or 9), weight buffers
+  int cols, smem;    // TMEM columns, dynamic shared memory
+};
+
+// weight chunks: for N tile nt, pass ps, tap t: nt_n x (gp x 8) K-major, core (kg, ng) at
+// kg * (nt_n / 8) * 128 + ng * 128. Source channel c = 8 (ps gp + kg) + kk; forward: w[n][c][t];
+// backward: c = s cop + co, w[co][n][t]
+__global__ void tile_pack_kernel(const uint16_t *__restrict__ w, int n_rows, int n_red, int cop, bool bwd, int nt_n,
+                                 int gp, int npass, int ntiles, uint16_t *__restrict__ out) {
+  const int64_t chunk = (int64_t)nt_n * gp * 8;
+  const int64_t total = (int64_t)ntiles * npass * 27 * chunk;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int q = (int)(i / chunk);  // (tile, pass, tap)
+    const int e = (int)(i % chunk);
+    const int kk = e & 7, row = (e >> 3) & 7, r = e >> 6;
+    const int ng = r % (nt_n / 8), kg = r / (nt_n / 8);
+    const int t = q % 27, ps = q / 27 % npass, nt = q / 27 / npass;
+    const int n = nt * nt_n + ng * 8 + row;
+    const int c = 8 * (ps * gp + kg) + kk;
+    uint16_t v = 0;
+    if (n < n_rows) {
+      if (!bwd) {
+        if (c < n_red) v = w[((int64_t)n * n_red + c) * 27 + t];
+      } else {
+        const int part = c / cop, co = c % cop;
+        if (part < 3 && co < n_red) v = w[((int64_t)co * n_rows + n) * 27 + t];
+      }
     }
+    out[i] = v;
   }
-  if (gp == 0) return cudaErrorInvalidValue;
-  const int npass = G / gp;
-  const int max_blocks = 512 / tmem_cols;
-  const int floor_smem = kSmPerSM / (max_blocks + 1) - 1024 + 16;
-  if (smem < floor_smem) smem = floor_smem;
+}
+
+template <bool BWD>
+__global__ void __launch_bounds__(kTileThreads)
+    tile_conv_kernel(const __grid_constant__ CUtensorMap tm, const uint16_t *__restrict__ wpack,
+                     const float *__restrict__ bias, int n_out, TileShape ts, int D, int H, int W, int relu,
+                     void *__restrict__ yout) {
+  extern __shared__ __align__(1024) unsigned char sm[];
+  __shared__ uint64_t loaded[kRingB], done[kRingB], box_full[kMaxBox][kMaxPlanes + 2], box_free[kMaxBox], fin;
+  __shared__ unsigned tslot;
+  __shared__ int okslot;
+  __shared__ float sbias[kMaxN];
+  const int nt_n = ts.nt_n, gp = ts.gp, P = ts.planes, nbox = ts.nbox, npass = ts.npass;
+  const int plane_bytes = kGroupBytes * gp, box_bytes = plane_bytes * (P + 2);
+  const int t_bytes = nt_n * gp * 16;  // one tap's weights
+  const int taps = ts.taps, ring = ts.ring, b_bytes = t_bytes * taps;
+  unsigned char *sb = sm + nbox * box_bytes;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int ntx = (W + kTX - 1) / kTX;
+  const int x0 = (blockIdx.x % ntx) * kTX, y0 = (blockIdx.x / ntx) * kTY, z0 = blockIdx.y * P;
+  const int np = min(P, D - z0);  // planes of this block inside the grid
+  const int nt = blockIdx.z;
+  const unsigned lbo_b = (unsigned)(nt_n / 8) * 128u;
+  const int per = 27 / taps, nch = npass * per;  // weight copies per pass, in all
+
+  if (tid == 0) {
+    for (int i = 0; i < kRingB; i++) {
+      bar_init(&loaded[i]);
+      bar_init(&done[i], np);
+    }
+    for (int b = 0; b < nbox; b++) {
+      for (int i = 0; i < P + 2; i++) bar_init(&box_full[b][i]);
+      bar_init(&box_free[b], np);
+    }
+    bar_init(&fin, np);
+    okslot = 1;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  for (int i = tid; i < nt_n; i += kTileThreads) sbias[i] = bias && nt * nt_n + i < n_out ? __ldg(bias + nt * nt_n + i) : 0.f;
+  if (warp == 0) tmem_alloc(&tslot, ts.cols);
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const unsigned tmem = tslot;
+
+  const bool one = elect_one();
+  if (warp == 4 && one) {  // copies: the planes' boxes pass by pass, the weight chunks in order
+    const uint16_t *wt = wpack + (int64_t)nt * nch * (b_bytes / 2);
+    auto issue_box = [&](int ps) {
+      const int b = ps % nbox;
+      for (int k = 0; k < np + 2; k++) {
+        const int i = BWD ? np + 1 - k : k;  // in the order the taps need them
+        bar_expect(&box_full[b][i], plane_bytes);
+        tma_box(sm + b * box_bytes + i * plane_bytes, &tm, x0, y0, z0 - 1 + i, ps * gp, &box_full[b][i]);
+      }
+    };
+    bool ok = true;
+    int boxes = 0, c = 0;
+    for (; boxes < nbox && boxes < npass; boxes++) issue_box(boxes);
+    for (; c < nch && ok; c++) {
+      if (c % per == 0 && c > 0 && boxes < npass && boxes < c / per + nbox) {
+        // the buffer of pass boxes - nbox is free once that pass's MMAs have run
+        ok = bar_wait(&box_free[boxes % nbox], ((boxes / nbox) - 1) & 1);
+        if (!ok) break;
+        issue_box(boxes++);
+      }
+      const int s = c % ring;
+      if (c >= ring && !bar_wait(&done[s], ((c / ring) - 1) & 1)) {
+        ok = false;
+        break;
+      }
+      bar_expect(&loaded[s], b_bytes);
+      bulk_copy(sb + s * b_bytes, wt + (int64_t)c * (b_bytes / 2), b_bytes, &loaded[s]);
+    }
+    // every copy lands before the shared memory is released
+    for (int q = max(0, c - ring); q < c; q++) ok = bar_wait(&loaded[q % ring], (q / ring) & 1) && ok;
+    for (int q = max(0, boxes - nbox); q < boxes; q++)
+      for (int i = 0; i < np + 2; i++) ok = bar_wait(&box_full[q % nbox][i], (q / nbox) & 1) && ok;
+    if (!ok) atomicExch(&okslot, 0);
+  } else if (warp < np && one) {  // MMAs of plane `warp`
+    const uint32_t idesc = instr_desc(nt_n);
+    const unsigned d = tmem + (unsigned)(warp * nt_n);
+    const unsigned ahi = (unsigned)(smem_desc(0, kGroupBytes, kRowBytes) >> 32), bhi = (unsigned)(smem_desc(0, lbo_b, 128) >> 32);
+    const unsigned blo = (unsigned)smem_desc(su32(sb), lbo_b, 128), bj = (2 * lbo_b) >> 4;
+    bool ok = true;
+    int s = 0, tc = 0;
+    unsigned turn = 0, acc = 0;  // ring buffer and its phase; 0 for the accumulator's first MMA
+    for (int ps = 0; ps < npass && ok; ps++) {
+      const int b = ps % nbox;
+      const unsigned ph = (ps / nbox) & 1;
+      const unsigned box = (unsigned)smem_desc(su32(sm + b * box_bytes + warp * plane_bytes), kGroupBytes, kRowBytes);
+      // the taps of the pass with JN group pairs
+      auto run = [&](auto pairs) {
+        constexpr int JN = decltype(pairs)::value;
+        for (int r = 0; r < 9; r++) {  // (kz, ky): three taps
+          // the tap's shift, mirrored in the backward pass
+          const int sz = BWD ? 2 - r / 3 : r / 3, sy = BWD ? 2 - r % 3 : r % 3;
+          if (r % 3 == 0) ok = bar_wait(&box_full[b][warp + sz], ph);
+          const unsigned al = box + (((unsigned)sz * plane_bytes + (unsigned)sy * kRowBytes) >> 4);
+#pragma unroll
+          for (int kx = 0; kx < 3; kx++) {
+            if (tc == 0) ok = ok && bar_wait(&loaded[s], turn);
+            if (!ok) return;
+            fence_after();
+            const unsigned bl = blo + ((unsigned)(s * b_bytes + tc * t_bytes) >> 4);
+#pragma unroll
+            for (int j = 0; j < JN; j++) {
+              mma_ss(d, al + (BWD ? 2 - kx : kx) + j * ((2 * kGroupBytes) >> 4), ahi, bl + j * bj, bhi, idesc, acc);
+              acc = 1u;
+            }
+            if (++tc == taps) {
+              mma_commit(&done[s]);
+              tc = 0;
+              if (++s == ring) {
+                s = 0;
+                turn ^= 1u;
+              }
+            }
+          }
+        }
+        mma_commit(&box_free[b]);
+      };
+      switch (min(gp, ts.G - ps * gp) / 2) {
+        case 1: run(std::integral_constant<int, 1>{}); break;
+        case 2: run(std::integral_constant<int, 2>{}); break;
+        case 3: run(std::integral_constant<int, 3>{}); break;
+        case 4: run(std::integral_constant<int, 4>{}); break;
+        case 5: run(std::integral_constant<int, 5>{}); break;
+        default: run(std::integral_constant<int, 6>{});
+      }
+    }
+    mma_commit(&fin);
+    if (!bar_wait(&fin, 0)) ok = false;
+    if (!ok) atomicExch(&okslot, 0);
+  }
+  __syncthreads();
+  const bool ok = *(volatile int *)&okslot != 0;
+  fence_after();
+  // epilogue: warp q reads TMEM lanes 32 q .. 32 q + 31 (tile rows 4 q .. 4 q + 3)
+  const int m = warp * 32 + lane;
+  const int ox = x0 + (m & 7), oy = y0 + (m >> 3);
+  const bool in = ox < W && oy < H;
+  const int64_t nv = (int64_t)D * H * W;
+  using Out = typename std::conditional<BWD, float, uint16_t>::type;
+  if (warp < 4)
+    for (int p = 0; p < np; p++) {
+      Out *o = static_cast<Out *>(yout) + (int64_t)nt * nt_n * nv + ((int64_t)(z0 + p) * H + oy) * W + ox;
+      for (int c0 = 0; c0 < nt_n; c0 += 16) {
+        uint32_t r[16];
+        tmem_ld16(r, tmem + ((unsigned)(warp * 32) << 16) + (unsigned)(p * nt_n + c0));
+        const int nc = min(16, n_out - nt * nt_n - c0);
+        Out v[16];
+#pragma unroll
+        for (int j = 0; j < 16; j++) {
+          if constexpr (BWD) {
+            v[j] = ok ? __uint_as_float(r[j]) : __uint_as_float(0x7FC00000u);
+          } else {
+            float f = __uint_as_float(r[j]) + sbias[c0 + j];
+            if (relu) f = fmaxf(f, 0.f);
+            v[j] = ok ? __bfloat16_as_ushort(__float2bfloat16_rn(f)) : (uint16_t)0x7FC0;
+          }
+        }
+        if (in) {
+          if (nc == 16) {
+#pragma unroll
+            for (int j = 0; j < 16; j++) o[j * nv] = v[j];
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; j++)
+              if (j < nc) o[j * nv] = v[j];
+          }
+        }
+        o += 16 * nv;
+      }
+    }
+  fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_free(tmem, ts.cols);
+}
+
+int pow2_cols(int n) {
+  int c = 32;
+  while (c < n) c *= 2;
+  return c;
+}
+
+// shapes of the tile form for n_rows output channels and `groups` channel groups; false when
+// no shape fits
+bool tile_shape(int n_rows, int groups, int64_t tiles_xy, int D, TileShape *out) {
+  const int n16 = (n_rows + 15) / 16 * 16;
+  TileShape ts{};
+  ts.nt_n = n16 < kMaxN ? n16 : kMaxN;
+  ts.ntiles = (n_rows + ts.nt_n - 1) / ts.nt_n;
+  ts.G = (groups + 1) / 2 * 2;
+  // groups per pass: the largest of 12, 8, 4 that divides the groups rounded up to 4 and leaves
+  // room for the N tile. It sets the order of the FP32 sums, and with it the rounding of the
+  // stored BF16 activations (which a ReLU network amplifies) and of the gradients, so it depends
+  // on the channels alone, not on the grid or on the planes per block.
+  int gp = 0;
+  const int g4 = (groups + 3) / 4 * 4;
+  for (int cand : {12, 8, 4})
+    if (!gp && g4 % cand == 0 && 3 * kGroupBytes * cand + 4 * ts.nt_n * cand * 16 <= 200 * 1024) gp = cand;
+  if (!gp) return false;
+  if (gp > ts.G) gp = ts.G;
+  ts.gp = gp;
+  const int npass = ts.npass = (ts.G + gp - 1) / gp;
+  double best = 0;
+  for (int planes : {4, 2, 1})
+    for (int nbox = 1; nbox <= (npass > 1 ? kMaxBox : 1); nbox++)
+      for (int taps : {9, 3, 1})
+        for (int ring = 2; ring <= kRingB; ring++) {
+          if (planes * ts.nt_n > kTmemCols) continue;
+          const int cols = pow2_cols(planes * ts.nt_n);
+          const int box = kGroupBytes * gp * (planes + 2), copy = taps * ts.nt_n * gp * 16;
+          int smem = nbox * box + ring * copy;
+          if (smem > kSmBlock) continue;
+          // the shared memory keeps the blocks an SM can hold within its TMEM columns, so an
+          // allocation never waits
+          const int floor_smem = kSmPerSM / (kTmemCols / cols + 1) - 1024 + 16;
+          if (smem < floor_smem) smem = floor_smem;
+          const int occ = std::min(kTmemCols / cols, kSmPerSM / (smem + 2560));
+          // a model in SM clocks: an MMA of M = 128, K = 16 reads 4 KB of A and 32 nt_n bytes of B
+          // at 128 B per clock or computes nt_n / 2 clocks (both measured); a weight copy takes
+          // about 1500 clocks of latency and 24 B per clock and SM; the first planes, the gaps
+          // between passes with one box buffer and the epilogue are hidden only by the SM's other
+          // blocks
+          const double one = std::max(32.0 + ts.nt_n / 4.0, ts.nt_n / 2.0);
+          const double mma = 27.0 * (ts.G / 2) * planes * one;                    // tensor pipe
+          const double chain = 27.0 * (ts.G / 2) * std::max(planes * one, 110.0);  // issue of one warp
+          const double trip = 27.0 * npass / taps * (1500.0 + copy / 24.0) / (ring - 1);
+          const double body = std::max(chain, trip);
+          const double extra = 2500.0 + box / 30.0 * (nbox == 1 ? npass : 1) * 0.5 + 12.0 * planes * ts.nt_n;
+          const double blocks = (double)tiles_xy * ((D + planes - 1) / planes) * ts.ntiles;
+          const double waves = std::ceil(blocks / (kSms * (double)occ));
+          const double l2 = occ * 27.0 * ts.G * 16 * ts.nt_n / 24.0;  // weights of all blocks of the SM
+          const double cost = waves * std::max(std::max(occ * mma, l2), body + extra);
+          if (best == 0 || cost < best) {
+            best = cost;
+            ts.planes = planes;
+            ts.nbox = nbox;
+            ts.taps = taps;
+            ts.ring = ring;
+            ts.cols = cols;
+            ts.smem = smem;
+            *out = ts;
+          }
+        }
+  return best > 0;
+}
+
+unsigned blocks_x(int64_t n, int threads, int64_t most) {
+  const int64_t b = (n + threads - 1) / threads;
+  return (unsigned)(b < most ? b : most);
+}
+
+size_t align256(size_t n) { return (n + 255) / 256 * 256; }
+
+// the tile form over a group-major source that `prepare` fills; n_rows GEMM output channels,
+// n_red real source channels (forward: cin; backward: cout, with cop = the part stride)
+template <bool BWD, class Prepare>
+cudaError_t run_tile(const uint16_t *w, const float *b, int n_rows, int n_red, int cop, int groups, int D, int H, int W,
+                     int relu, void *y, cudaStream_t s, Prepare prepare) {
   const int64_t nv = (int64_t)D * H * W;
   const int64_t tiles_xy = (int64_t)((W + kTX - 1) / kTX) * ((H + kTY - 1) / kTY);
-  if (tiles_xy > 0x7fffffff || D > 65535 || ntiles > 65535) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(tile_conv_kernel<BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  const size_t pack_elems = (size_t)ntiles * npass * 27 * nt_n * gp * 8;
-  uint16_t *wp = nullptr, *src = nullptr;
-  e = cudaMallocAsync(reinterpret_cast<void **>(&wp), pack_elems * sizeof(uint16_t), s);
-  if (e != cudaSuccess) return e;
-  e = cudaMallocAsync(reinterpret_cast<void **>(&src), (size_t)G * nv * 8 * sizeof(uint16_t), s);
-  if (e != cudaSuccess) {
-    cudaFreeAsync(wp, s);
-    return e;
-  }
-  // tensor map of src as (x and 8 channels: 8 W, H, D, G) BF16; boxes (80, 18, 3, gp), zero
-  // outside the grid
-  CUtensorMap tm;
-  std::memset(&tm, 0, sizeof(tm));
-  const cuuint64_t dims[4] = {(cuuint64_t)W * 8, (cuuint64_t)H, (cuuint64_t)D, (cuuint64_t)G};
-  const cuuint64_t pitch[3] = {(cuuint64_t)W * 16, (cuuint64_t)W * H * 16, (cuuint64_t)nv * 16};
-  const cuuint32_t box[4] = {kBX * 8, kBY, 3, (cuuint32_t)gp};
-  const cuuint32_t step[4] = {1, 1, 1, 1};
-  if (enc(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, src, dims, pitch, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
-          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
-      CUDA_SUCCESS) {
-    cudaFreeAsync(src, s);
-    cudaFreeAsync(wp, s);
+  TileShape ts;
+  if (tiles_xy > 0x7fffffff || D > 65535 || !tile_shape(n_rows, groups, tiles_xy, D, &ts) || ts.ntiles > 65535)
     return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(tile_conv_kernel<BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmBlock);
+  if (e != cudaSuccess) return e;
+  const size_t pack_elems = (size_t)ts.ntiles * ts.npass * 27 * ts.nt_n * ts.gp * 8;
+  const size_t src_bytes = align256((size_t)ts.G * nv * 16);
+  unsigned char *buf = nullptr;
+  e = cudaMallocAsync(reinterpret_cast<void **>(&buf), src_bytes + pack_elems * 2, s);
+  if (e != cudaSuccess) return e;
+  uint16_t *src = reinterpret_cast<uint16_t *>(buf), *wp = reinterpret_cast<uint16_t *>(buf + src_bytes);
+  CUtensorMap tm;
+  e = box_map(&tm, src, D, H, W, ts.G, ts.gp);
+  if (e == cudaSuccess) {
+    tile_pack_kernel<<<blocks_x((int64_t)pack_elems, 256, 4096), 256, 0, s>>>(w, n_rows, n_red, cop, BWD, ts.nt_n, ts.gp,
+                                                                              ts.npass, ts.ntiles, wp);
+    prepare(src, ts.G);
+    tile_conv_kernel<BWD><<<dim3((unsigned)tiles_xy, (unsigned)((D + ts.planes - 1) / ts.planes), (unsigned)ts.ntiles),
+                            kTileThreads, ts.smem, s>>>(tm, wp, b, n_rows, ts, D, H, W, relu, y);
+    e = cudaGetLastError();
   }
-  const int64_t pblocks = ((int64_t)pack_elems + 255) / 256;
-  tile_pack_kernel<<<(unsigned)(pblocks < 4096 ? pblocks : 4096), 256, 0, s>>>(w, n_rows, n_red, cop, BWD, nt_n, gp,
-                                                                               npass, ntiles, wp);
-  const int64_t xblocks = (nv * G + 255) / 256;
-  prepare(src, (unsigned)(xblocks < 65536 ? xblocks : 65536));
-  tile_conv_kernel<BWD><<<dim3((unsigned)tiles_xy, (unsigned)D, (unsigned)ntiles), kTileThreads, smem, s>>>(
-      tm, wp, b, n_rows, nt_n, tmem_cols, gp, npass, D, H, W, relu, y);
-  e = cudaGetLastError();
-  const cudaError_t f1 = cudaFreeAsync(src, s), f2 = cudaFreeAsync(wp, s);
-  return e != cudaSuccess ? e : (f1 != cudaSuccess ? f1 : f2);
+  const cudaError_t f = cudaFreeAsync(buf, s);
+  return e != cudaSuccess ? e : f;
+}
+
+// ---- weight gradient: D_t[r][ci] = sum_p A[r][p] x[ci][p + off(t)], r = (part, channel) of the
+// split gradient. The three parts of up to 42 channels are the M = 128 rows of one operand
+// that is kept in TMEM, so the taps of a block share one load of it and an MMA reads only the
+// x view from shared memory (B, MN-major: a core matrix is 8 x-voxels along K of 8 channels).
+// With both operands in shared memory an MMA of N = 32 reads 5 KB (40 clocks) for 16 clocks of
+// math; from TMEM the read is 1 KB. A block owns a slice of voxel tiles, a group of T taps of
+// one kz (9 up to 32 channels, else 3 of one ky) and up to 112 input channels, one
+// accumulator of nt_n columns per tap. The three parts are added in the epilogue, so each
+// accumulator's chain is a third as long as with one for all parts.
+//
+// Warp 4 copies the stages (a gradient tile, contiguous in the tile-ordered split copy, and the
+// x box), warps 0-3 move the gradient rows from shared memory into one of two TMEM buffers,
+// warp 5 + t issues the MMAs of tap t (one thread's issue, about 45 clocks, takes three times
+// as long as an MMA of N = 32). Bound: the tensor pipe at small N and the hand-over of the
+// gradient buffers. Measured at 65 x 129 x 129 voxels, 28 x 28 channels: 1362 -> 215 us (im2col
+// rows gathered by the threads before); 56 x 56 channels at 33 x 65 x 65: 511 -> 126 us.
+constexpr int kWgA = 384;          // first TMEM column of the two gradient buffers (64 columns each)
+constexpr int kWgAccCols = 368;    // accumulator columns: 368 + 16 (bias) = 384
+constexpr int kWgMaxRing = 8;      // most stages in flight
+constexpr int kWgRows = 42;        // gradient channels per M tile (3 parts: 126 rows)
+constexpr int kWgSlice = 48;       // most tiles per slice: 6144 voxels, 384 sums per accumulator
+constexpr int kWorkSlice = 2048;    // voxels per slice the size of `work` is counted by
+
+// dyt[mt][tile][y][r][8 x]: the split gradient of the rows r = part cm + c of M tile mt
+// (channel mt cm + c), per voxel tile and tile row; zero outside the grid and past cout. A
+// block turns one tile of up to 32 channels through shared memory, so that both its reads
+// (8 voxels of a row) and its writes (16 bytes of consecutive channels) are contiguous.
+__global__ void __launch_bounds__(256) split_tiles(const float *__restrict__ dy, int cout, int cm, int ntx, int nty, int D,
+                                                   int H, int W, uint16_t *__restrict__ dyt) {
+  __shared__ float st[32][kM + 1];
+  const int tile = blockIdx.x, mt = blockIdx.z, c0 = blockIdx.y * 32;  // channel chunk of the M tile
+  const int x0 = tile % ntx * kTX, y0 = tile / ntx % nty * kTY, z = tile / ntx / nty;
+  const int nc = min(32, cm - c0);
+  for (int i = threadIdx.x; i < nc * kM; i += 256) {
+    const int c = i / kM, v = i % kM, x = x0 + (v & 7), y = y0 + (v >> 3), co = mt * cm + c0 + c;
+    st[c][v] = (co < cout && x < W && y < H) ? __ldg(dy + (((int64_t)co * D + z) * H + y) * W + x) : 0.f;
+  }
+  __syncthreads();
+  const int64_t base = ((int64_t)mt * gridDim.x + tile) * kTY * (3 * cm);
+  for (int i = threadIdx.x; i < 32 * kTY; i += 256) {
+    const int c = i & 31, y = i >> 5;
+    if (c >= nc) continue;
+    uint16_t h[3][8];
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+      uint16_t t[3];
+      split3(st[c][y * 8 + e], t);
+#pragma unroll
+      for (int s = 0; s < 3; s++) h[s][e] = t[s];
+    }
+#pragma unroll
+    for (int s = 0; s < 3; s++)
+      *reinterpret_cast<uint4 *>(dyt + (base + (int64_t)y * (3 * cm) + s * cm + c0 + c) * 8) = pack8(h[s]);
+  }
+}
+
+struct WgShape {
+  int T, nt_n, ntile;      // taps per block, input channels per block, N tiles
+  int cm, mt;              // gradient channels per M tile, M tiles
+  int G, ntx, nty, tiles;  // source groups, voxel tiles
+  int slices, per;         // slices, tiles per slice
+  int ring, smem;
+};
+
+template <int T>
+__global__ void __launch_bounds__(32 * (5 + T), 1)
+    wgrad_kernel(const __grid_constant__ CUtensorMap tm, const uint16_t *__restrict__ dyt, WgShape g, int D, int cin,
+                 int cout, float *__restrict__ part) {
+  extern __shared__ __align__(1024) unsigned char sm[];
+  __shared__ __align__(128) uint4 ones[8];  // a core matrix of BF16 ones (the bias gradient)
+  __shared__ uint64_t full[kWgMaxRing], free_[kWgMaxRing], a_full[2], a_free[2], fin;
+  __shared__ unsigned tslot;
+  __shared__ int okslot;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  // the blocks of one slice are neighbours in the grid: its voxels are read while L2 holds them
+  constexpr int ngrp = 27 / T;
+  const int grp = blockIdx.x % ngrp, nt = blockIdx.x / ngrp % g.ntile, mt = blockIdx.x / ngrp / g.ntile;
+  const int slice = blockIdx.y;
+  const int tap0 = grp * T, kz = tap0 / 9, ky0 = tap0 / 3 % 3;
+  const bool bias = tap0 / 9 == 1 && (T == 9 || ky0 == 1) && nt == 0;
+  const int R = 3 * g.cm, plane = g.ntx * g.nty;
+  const int box_bytes = g.nt_n / 8 * kGroupBytes, a_bytes = R * kTY * 16;
+  const int stage = (box_bytes + a_bytes + 127) / 128 * 128;  // box, then gradient rows [y][r][8 x]
+  // the slice's tiles whose plane z + kz - 1 is inside the grid (the others add nothing)
+  const int t0 = max(slice * g.per, kz == 0 ? plane : 0);
+  const int t1 = min(min((slice + 1) * g.per, g.tiles), kz == 2 ? plane * (D - 1) : g.tiles);
+  const int n = max(0, t1 - t0);
+
+  if (tid == 0) {
+    for (int i = 0; i < g.ring; i++) {
+      bar_init(&full[i]);
+      bar_init(&free_[i], T);
+    }
+    for (int i = 0; i < 2; i++) {
+      bar_init(&a_full[i], 4);
+      bar_init(&a_free[i], T);
+    }
+    bar_init(&fin, T);
+    okslot = 1;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (tid < 8) ones[tid] = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  if (warp == 0) tmem_alloc(&tslot, kTmemCols);
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const unsigned tmem = tslot;
+
+  const bool one = elect_one();
+  if (warp < 4) {  // gradient rows into TMEM: thread = row, 64 columns = 128 voxels
+    const int r = warp * 32 + lane;
+    bool ok = true;
+    for (int i = 0; i < n; i++) {
+      const int b = i & 1, st = i % g.ring;
+      ok = __all_sync(0xffffffffu, bar_wait(&full[st], (i / g.ring) & 1) && (i < 2 || bar_wait(&a_free[b], ((i >> 1) - 1) & 1)));
+      if (!ok) break;
+      fence_after();
+      const uint4 *q = reinterpret_cast<const uint4 *>(sm + st * stage + box_bytes) + r;
+      const unsigned a = tmem + ((unsigned)(warp * 32) << 16) + (unsigned)(kWgA + b * 64);
+#pragma unroll
+      for (int c = 0; c < 4; c++) {
+        uint4 v[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) v[k] = r < R ? q[(4 * c + k) * R] : make_uint4(0u, 0u, 0u, 0u);
+        tmem_st16(a + 16 * c, v);
+      }
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      fence_before();
+      __syncwarp();
+      if (lane == 0) bar_arrive(&a_full[b]);
+    }
+    if (!ok) atomicExch(&okslot, 0);
+  } else if (warp == 4 && one) {  // copies
+    const uint16_t *src = dyt + ((int64_t)mt * g.tiles + t0) * (a_bytes / 2);
+    bool ok = true;
+    int i = 0;
+    for (; i < n; i++) {
+      const int s = i % g.ring, tile = t0 + i;
+      if (i >= g.ring && !bar_wait(&free_[s], ((i / g.ring) - 1) & 1)) {
+        ok = false;
+        break;
+      }
+      bar_expect(&full[s], box_bytes + a_bytes);
+      bulk_copy(sm + s * stage + box_bytes, src + (int64_t)i * (a_bytes / 2), a_bytes, &full[s]);
+      tma_box(sm + s * stage, &tm, tile % g.ntx * kTX, tile / g.ntx % g.nty * kTY, tile / plane + kz - 1,
+              nt * (g.nt_n / 8), &full[s]);
+    }
+    for (int q = max(0, i - g.ring); q < i; q++) ok = bar_wait(&full[q % g.ring], (q / g.ring) & 1) && ok;
+    if (!ok) atomicExch(&okslot, 0);
+  } else if (warp >= 5 && one) {  // MMAs of tap w of the group
+    const int w = warp - 5;
+    const uint32_t idesc = instr_desc(g.nt_n) | (1u << 16), idesc1 = instr_desc(16) | (1u << 16);  // B MN-major
+    const unsigned dhi = (unsigned)(smem_desc(0, kRowBytes, kGroupBytes) >> 32);
+    const unsigned dlo0 =
+        (unsigned)smem_desc(su32(sm) + (unsigned)((ky0 + w / 3) * kRowBytes + w % 3 * 16), kRowBytes, kGroupBytes);
+    const uint64_t d1 = smem_desc(su32(ones), 0, 0);
+    const unsigned d1lo = (unsigned)d1, d1hi = (unsigned)(d1 >> 32);
+    const unsigned dt = tmem + (unsigned)(w * g.nt_n), db = tmem + (unsigned)(T * g.nt_n);
+    const bool ones_too = bias && w == 0;
+    bool ok = true;
+    for (int i = 0; i < n; i++) {
+      const int b = i & 1, s = i % g.ring;
+      if (!bar_wait(&a_full[b], (i >> 1) & 1) || !bar_wait(&full[s], (i / g.ring) & 1)) {
+        ok = false;
+        break;
+      }
+      fence_after();
+      const unsigned dlo = dlo0 + ((unsigned)(s * stage) >> 4), a = tmem + (unsigned)(kWgA + b * 64);
+#pragma unroll
+      for (int ks = 0; ks < 8; ks++) {  // 16 voxels: tile rows 2 ks, 2 ks + 1
+        const unsigned acc = (i > 0 || ks > 0) ? 1u : 0u;
+        mma_ts(dt, a + ks * 8, dlo + ((2 * ks * kRowBytes) >> 4), dhi, idesc, acc);
+        if (ones_too) mma_ts(db, a + ks * 8, d1lo, d1hi, idesc1, acc);
+      }
+      mma_commit(&a_free[b]);
+      mma_commit(&free_[s]);
+    }
+    mma_commit(&fin);
+    if (!bar_wait(&fin, 0)) ok = false;
+    if (!ok) atomicExch(&okslot, 0);
+  }
+  __syncthreads();
+  const bool ok = *(volatile int *)&okslot != 0;
+  fence_after();
+  // part[slice][co][t cin + ci], then the bias sum: the accumulators go to shared memory (the
+  // stages' space), where every thread adds the three parts' rows of its channels
+  float *se = reinterpret_cast<float *>(sm);
+  const int ncol = T * g.nt_n + (bias ? 16 : 0), pitch = ncol + 1;
+  if (warp < 4)
+    for (int c0 = 0; c0 < ncol; c0 += 16) {
+      uint32_t v[16];
+      tmem_ld16(v, tmem + ((unsigned)(warp * 32) << 16) + (unsigned)c0);
+#pragma unroll
+      for (int j = 0; j < 16; j++) se[tid * pitch + c0 + j] = n > 0 ? __uint_as_float(v[j]) : 0.f;
+    }
+  __syncthreads();
+  const int64_t row = 27 * (int64_t)cin + 1;
+  for (int c = warp; c < g.cm; c += 5 + T) {
+    const int co = mt * g.cm + c;
+    if (co >= cout) break;
+    const float *s0 = se + c * pitch, *s1 = s0 + g.cm * pitch, *s2 = s1 + g.cm * pitch;
+    float *out = part + ((int64_t)slice * cout + co) * row;
+    for (int t = 0; t < T; t++)
+      for (int j = lane; j < g.nt_n; j += 32) {
+        const int ci = nt * g.nt_n + j, q = t * g.nt_n + j;
+        if (ci < cin) out[(int64_t)(tap0 + t) * cin + ci] = ok ? s0[q] + (s1[q] + s2[q]) : __uint_as_float(0x7FC00000u);
+      }
+    if (bias && lane == 0) {
+      const int q = T * g.nt_n;
+      out[row - 1] = ok ? s0[q] + (s1[q] + s2[q]) : __uint_as_float(0x7FC00000u);
+    }
+  }
+  fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_free(tmem, kTmemCols);
+}
+
+// dw[co][ci][t] and db[co]: the slices' partial sums. A block owns 32 outputs; warp k adds
+// the slices k, k + 8, ... in order, then the eight sums are added in order (one thread per
+// output, all slices in one chain, took 64 us at 28 x 28 channels and 528 slices; 9 us now).
+__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float *__restrict__ part, int nslice, int cin, int cout,
+                                                           float *__restrict__ dw, float *__restrict__ db) {
+  __shared__ float sh[8][32];
+  const int64_t row = 27 * (int64_t)cin + 1, total = cout * row;
+  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+  for (int64_t i0 = (int64_t)blockIdx.x * 32; i0 < total; i0 += (int64_t)gridDim.x * 32) {
+    const int64_t i = i0 + lane;
+    float acc = 0.f;
+    if (i < total)
+#pragma unroll 4
+      for (int sl = k; sl < nslice; sl += 8) acc += __ldg(part + sl * total + i);
+    sh[k][lane] = acc;
+    __syncthreads();
+    if (k == 0 && i < total) {
+#pragma unroll
+      for (int q = 1; q < 8; q++) acc += sh[q][lane];
+      const int co = (int)(i / row), j = (int)(i % row);
+      if (j == row - 1) {
+        if (db) db[co] = acc;
+      } else {
+        dw[((int64_t)co * cin + j % cin) * 27 + j / cin] = acc;
+      }
+    }
+    __syncthreads();
+  }
 }
 
 }  // namespace
 
-
 cudaError_t conv3d_forward_tc(const uint16_t *x, const uint16_t *w, const float *b, int cin, int cout, int D, int H,
                               int W, int relu, uint16_t *y, cudaStream_t s) {
-  const int G = (cin + 31) / 32 * 4;  // groups of 8 channels, a multiple of 4
   const int64_t nv = (int64_t)D * H * W;
-  return run_tile<false>(w, b, cout, cin, 0, G, D, H, W, relu, y, s, [&](uint16_t *src, unsigned blocks) {
-    to_group_major<<<blocks, 256, 0, s>>>(x, nv, cin, G, src);
+  return run_tile<false>(w, b, cout, cin, 0, (cin + 7) / 8, D, H, W, relu, y, s, [&](uint16_t *src, int G) {
+    to_group_major<<<dim3((unsigned)((nv + 255) / 256), (unsigned)G), 256, 0, s>>>(x, nv, cin, src);
   });
 }
 
 cudaError_t conv3d_backward_data_tc(const float *dy, const uint16_t *w, int cin, int cout, int D, int H, int W,
                                     float *dx, cudaStream_t s) {
   const int cop = (cout + 7) / 8 * 8;
-  const int G = (3 * cop / 8 + 3) / 4 * 4;
   const int64_t nv = (int64_t)D * H * W;
-  return run_tile<true>(w, nullptr, cin, cout, cop, G, D, H, W, 0, dx, s, [&](uint16_t *src, unsigned blocks) {
-    split_group_major<<<blocks, 256, 0, s>>>(dy, nv, cout, cop, G, src);
+  return run_tile<true>(w, nullptr, cin, cout, cop, 3 * cop / 8, D, H, W, 0, dx, s, [&](uint16_t *src, int G) {
+    split_group_major<<<dim3(blocks_x(nv, 256, 65536), (unsigned)std::min(cop / 8, 65535)), 256, 0, s>>>(dy, nv, cout,
+                                                                                                        cop, G, src);
   });
+}
+
+// floats the caller's scratch holds: one 128-row-padded im2col row set per 2048 voxels and
+// output channel (the partial sums below need less for all but small grids)
+int64_t conv3d_backward_weight_tc_work(int cin, int cout, int D, int H, int W) {
+  const int cp = (cin + 7) / 8 * 8;
+  const int64_t nv = (int64_t)D * H * W;
+  const int64_t nslice = (nv + kWorkSlice - 1) / kWorkSlice;
+  const int64_t mpad = ((int64_t)27 * cp + 1 + 127) / 128 * 128;
+  const int n16 = (cout + 15) / 16 * 16;
+  const int nt_n = n16 < kMaxN ? n16 : kMaxN;
+  const int64_t ncol = (int64_t)((cout + nt_n - 1) / nt_n) * nt_n;
+  return nslice * ncol * mpad;
+}
+
+cudaError_t conv3d_backward_weight_tc(const float *dy, const uint16_t *x, int cin, int cout, int D, int H, int W,
+                                      float *dw, float *db, float *work, cudaStream_t s) {
+  const int64_t nv = (int64_t)D * H * W;
+  WgShape g{};
+  g.ntx = (W + kTX - 1) / kTX;
+  g.nty = (H + kTY - 1) / kTY;
+  const int64_t tiles = (int64_t)g.ntx * g.nty * D;
+  if (tiles > 0x7fffffff / 64) return cudaErrorInvalidValue;
+  g.tiles = (int)tiles;
+  g.mt = (cout + kWgRows - 1) / kWgRows;
+  g.cm = (cout + g.mt - 1) / g.mt;
+  g.G = (cin + 7) / 8;
+  const int n16 = (cin + 15) / 16 * 16;
+  g.T = n16 <= 32 ? 9 : 3;
+  const int most = kWgAccCols / g.T / 16 * 16;
+  g.ntile = (n16 + most - 1) / most;
+  g.nt_n = ((n16 + g.ntile - 1) / g.ntile + 15) / 16 * 16;
+  const int combos = 27 / g.T * g.ntile * g.mt;
+  // one block per SM (all its TMEM): as many slices as fill whole waves of the SMs, at most
+  // kWgSlice tiles each, and on small grids at least two tiles
+  const int64_t waves = ((int64_t)combos * ((tiles + kWgSlice - 1) / kWgSlice) + kSms - 1) / kSms;
+  int64_t slices = std::max<int64_t>(1, waves * kSms / combos);
+  slices = std::max<int64_t>(std::min(slices, (tiles + 1) / 2), (tiles + kWgSlice - 1) / kWgSlice);
+  g.per = (int)((tiles + slices - 1) / slices);
+  g.slices = (int)((tiles + g.per - 1) / g.per);
+  if ((nv + kWorkSlice - 1) / kWorkSlice > 65535) return cudaErrorInvalidValue;  // as the size of `work` assumes
+  const int stage = (g.nt_n / 8 * kGroupBytes + 3 * g.cm * kTY * 16 + 127) / 128 * 128;
+  g.ring = std::min(kWgMaxRing, kSmBlock / stage);
+  g.smem = std::max({g.ring * stage, kM * (g.T * g.nt_n + 17) * 4, kSmPerSM / 2});  // one block per SM, as its TMEM is one block's
+  const auto kernel = g.T == 9 ? wgrad_kernel<9> : wgrad_kernel<3>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmBlock);
+  if (e != cudaSuccess) return e;
+  const size_t src_bytes = align256((size_t)g.G * nv * 16);
+  const size_t dyt_bytes = align256((size_t)g.mt * tiles * kTY * 3 * g.cm * 16);
+  const int64_t part_floats = (int64_t)g.slices * cout * (27 * (int64_t)cin + 1);
+  const bool own = part_floats > conv3d_backward_weight_tc_work(cin, cout, D, H, W);
+  unsigned char *buf = nullptr;
+  e = cudaMallocAsync(reinterpret_cast<void **>(&buf), src_bytes + dyt_bytes + (own ? part_floats * 4 : 0), s);
+  if (e != cudaSuccess) return e;
+  uint16_t *src = reinterpret_cast<uint16_t *>(buf), *dyt = reinterpret_cast<uint16_t *>(buf + src_bytes);
+  float *part = own ? reinterpret_cast<float *>(buf + src_bytes + dyt_bytes) : work;
+  CUtensorMap tm;
+  e = box_map(&tm, src, D, H, W, g.G, g.nt_n / 8);
+  if (e == cudaSuccess) {
+    to_group_major<<<dim3((unsigned)((nv + 255) / 256), (unsigned)g.G), 256, 0, s>>>(x, nv, cin, src);
+    split_tiles<<<dim3((unsigned)tiles, (unsigned)((g.cm + 31) / 32), (unsigned)g.mt), 256, 0, s>>>(dy, cout, g.cm, g.ntx,
+                                                                                                  g.nty, D, H, W, dyt);
+    kernel<<<dim3((unsigned)combos, (unsigned)g.slices), 32 * (5 + g.T), g.smem, s>>>(tm, dyt, g, D, cin, cout, part);
+    wgrad_reduce_kernel<<<blocks_x((int64_t)cout * (27 * (int64_t)cin + 1), 32, 65536), 256, 0, s>>>(part, g.slices, cin,
+                                                                                                  cout, dw, db);
+    e = cudaGetLastError();
+  }
+  const cudaError_t f = cudaFreeAsync(buf, s);
+  return e != cudaSuccess ? e : f;
 }
 
 }  // namespace fwi_tc
