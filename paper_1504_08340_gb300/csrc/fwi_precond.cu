@@ -90,66 +90,98 @@ struct Cells {
   }
 };
 
+// blockIdx.y walks the (channel, z) planes of the output and the threads its voxels (y, x) in
+// order, so an index costs one 32-bit division and consecutive threads write consecutive
+// voxels. Bound by HBM; one flat 64-bit index per value had taken three 64-bit divisions
+// (upsampling 56 channels to 65 x 129 x 129: 443 us, 75 us this way, 20 us of traffic).
+
+// f(c, z, y, x, i) for this thread's voxels of a [C][D][H][W] grid, i the voxel's offset in the plane
+template <class F>
+__device__ __forceinline__ void for_voxels(int C, int D, int H, int W, F f) {
+  const int64_t planes = (int64_t)C * D;
+  const int64_t n = (int64_t)H * W;
+  for (int64_t cz = blockIdx.y; cz < planes; cz += gridDim.y) {
+    const int c = (int)(cz / D), z = (int)(cz - (int64_t)c * D);
+    if (n <= 0x7fffffff) {
+#pragma unroll 4
+      for (unsigned i = blockIdx.x * kT + threadIdx.x; i < (unsigned)n; i += gridDim.x * kT) {
+        const unsigned y = i / (unsigned)W;
+        f(c, z, (int)y, (int)(i - y * W), (int64_t)i);
+      }
+    } else {
+      for (int64_t i = (int64_t)blockIdx.x * kT + threadIdx.x; i < n; i += (int64_t)gridDim.x * kT)
+        f(c, z, (int)(i / W), (int)(i % W), i);
+    }
+  }
+}
+
+// sum of the fine values of coarse cell (q0, q1, q2), r at its first voxel, in (z, y, x) order
+template <class T, class V>
+__device__ __forceinline__ float cell_sum(const T *__restrict__ r, const Cells &g, int q0, int q1, int q2, V value) {
+  const bool bz = 2 * q0 + 1 < g.D, by = 2 * q1 + 1 < g.H, bx = 2 * q2 + 1 < g.W;
+  const int64_t sz = (int64_t)g.H * g.W;
+  float s = 0.f;
+#pragma unroll
+  for (int a = 0; a < 2; a++)
+#pragma unroll
+    for (int b = 0; b < 2; b++)
+#pragma unroll
+      for (int e = 0; e < 2; e++)
+        if ((a == 0 || bz) && (b == 0 || by) && (e == 0 || bx)) s += value(r[a * sz + b * g.W + e]);
+  return s;
+}
+
 // y[c][q] = mean of x[c][p] over the fine voxels p of coarse cell q (FP32 sum, rounded to BF16)
 __global__ void __launch_bounds__(kT) pool2_fwd_kernel(const uint16_t *__restrict__ x, int C, Cells g,
                                                        uint16_t *__restrict__ y) {
-  const int64_t nc = (int64_t)g.Dc * g.Hc * g.Wc, n = nc * C;
-  for (int64_t i = (int64_t)blockIdx.x * kT + threadIdx.x; i < n; i += (int64_t)gridDim.x * kT) {
-    const int64_t c = i / nc, q = i % nc;
-    const int q2 = (int)(q % g.Wc), q1 = (int)((q / g.Wc) % g.Hc), q0 = (int)(q / ((int64_t)g.Wc * g.Hc));
-    const uint16_t *xc = x + c * (int64_t)g.D * g.H * g.W;
-    float s = 0.f;
-    for (int a = 0; a < 2; a++)
-      for (int b = 0; b < 2; b++)
-        for (int e = 0; e < 2; e++) {
-          const int z = 2 * q0 + a, yy = 2 * q1 + b, xx = 2 * q2 + e;
-          if (z < g.D && yy < g.H && xx < g.W) s += bf2f(xc[((int64_t)z * g.H + yy) * g.W + xx]);
-        }
-    y[i] = f2bf(s / (float)g.count(q0, q1, q2));
-  }
+  for_voxels(C, g.Dc, g.Hc, g.Wc, [&](int c, int q0, int q1, int q2, int64_t i) {
+    const float s = cell_sum(x + (((int64_t)c * g.D + 2 * q0) * g.H + 2 * q1) * g.W + 2 * q2, g, q0, q1, q2, bf2f);
+    y[((int64_t)c * g.Dc + q0) * g.Hc * g.Wc + i] = f2bf(s / (float)g.count(q0, q1, q2));
+  });
 }
 
 // dx[c][p] (+)= dy[c][cell(p)] / count(cell(p))
 __global__ void __launch_bounds__(kT) pool2_bwd_kernel(const float *__restrict__ dy, int C, Cells g, int acc,
                                                        float *__restrict__ dx) {
-  const int64_t nf = (int64_t)g.D * g.H * g.W, n = nf * C;
-  for (int64_t i = (int64_t)blockIdx.x * kT + threadIdx.x; i < n; i += (int64_t)gridDim.x * kT) {
-    const int64_t c = i / nf, p = i % nf;
-    const int x2 = (int)(p % g.W), x1 = (int)((p / g.W) % g.H), x0 = (int)(p / ((int64_t)g.W * g.H));
-    const int q0 = x0 >> 1, q1 = x1 >> 1, q2 = x2 >> 1;
-    const float v = dy[c * (int64_t)g.Dc * g.Hc * g.Wc + ((int64_t)q0 * g.Hc + q1) * g.Wc + q2] / (float)g.count(q0, q1, q2);
-    dx[i] = acc ? dx[i] + v : v;
-  }
+  for_voxels(C, g.D, g.H, g.W, [&](int c, int z, int y, int x, int64_t i) {
+    const int q0 = z >> 1, q1 = y >> 1, q2 = x >> 1;
+    const float v = dy[(((int64_t)c * g.Dc + q0) * g.Hc + q1) * g.Wc + q2] / (float)g.count(q0, q1, q2);
+    float *o = dx + ((int64_t)c * g.D + z) * g.H * g.W + i;
+    *o = acc ? *o + v : v;
+  });
 }
 
-// y[c][p] = x[c][cell(p)] (nearest neighbour)
+// y[c][p] = x[c][cell(p)] (nearest neighbour); a thread owns one x of a coarse row and writes
+// it to the up to four fine rows of that row's cells
 __global__ void __launch_bounds__(kT) up2_fwd_kernel(const uint16_t *__restrict__ x, int C, Cells g,
                                                      uint16_t *__restrict__ y) {
-  const int64_t nf = (int64_t)g.D * g.H * g.W, n = nf * C;
-  for (int64_t i = (int64_t)blockIdx.x * kT + threadIdx.x; i < n; i += (int64_t)gridDim.x * kT) {
-    const int64_t c = i / nf, p = i % nf;
-    const int x2 = (int)(p % g.W), x1 = (int)((p / g.W) % g.H), x0 = (int)(p / ((int64_t)g.W * g.H));
-    y[i] = x[c * (int64_t)g.Dc * g.Hc * g.Wc + ((int64_t)(x0 >> 1) * g.Hc + (x1 >> 1)) * g.Wc + (x2 >> 1)];
-  }
+  for_voxels(C, g.Dc, g.Hc, g.W, [&](int c, int q0, int q1, int xx, int64_t) {
+    const uint16_t v = __ldg(x + (((int64_t)c * g.Dc + q0) * g.Hc + q1) * g.Wc + (xx >> 1));
+    uint16_t *o = y + (((int64_t)c * g.D + 2 * q0) * g.H + 2 * q1) * g.W + xx;
+    const bool bz = 2 * q0 + 1 < g.D, by = 2 * q1 + 1 < g.H;
+    const int64_t sz = (int64_t)g.H * g.W;
+    o[0] = v;
+    if (by) o[g.W] = v;
+    if (bz) o[sz] = v;
+    if (by && bz) o[sz + g.W] = v;
+  });
 }
 
 // dx[c][q] (+)= sum of dy[c][p] over the fine voxels p of cell q, in a fixed order
 __global__ void __launch_bounds__(kT) up2_bwd_kernel(const float *__restrict__ dy, int C, Cells g, int acc,
                                                      float *__restrict__ dx) {
-  const int64_t nc = (int64_t)g.Dc * g.Hc * g.Wc, n = nc * C;
-  for (int64_t i = (int64_t)blockIdx.x * kT + threadIdx.x; i < n; i += (int64_t)gridDim.x * kT) {
-    const int64_t c = i / nc, q = i % nc;
-    const int q2 = (int)(q % g.Wc), q1 = (int)((q / g.Wc) % g.Hc), q0 = (int)(q / ((int64_t)g.Wc * g.Hc));
-    const float *dc = dy + c * (int64_t)g.D * g.H * g.W;
-    float s = 0.f;
-    for (int a = 0; a < 2; a++)
-      for (int b = 0; b < 2; b++)
-        for (int e = 0; e < 2; e++) {
-          const int z = 2 * q0 + a, yy = 2 * q1 + b, xx = 2 * q2 + e;
-          if (z < g.D && yy < g.H && xx < g.W) s += dc[((int64_t)z * g.H + yy) * g.W + xx];
-        }
-    dx[i] = acc ? dx[i] + s : s;
-  }
+  for_voxels(C, g.Dc, g.Hc, g.Wc, [&](int c, int q0, int q1, int q2, int64_t i) {
+    const float s = cell_sum(dy + (((int64_t)c * g.D + 2 * q0) * g.H + 2 * q1) * g.W + 2 * q2, g, q0, q1, q2,
+                             [](float v) { return v; });
+    float *o = dx + ((int64_t)c * g.Dc + q0) * g.Hc * g.Wc + i;
+    *o = acc ? *o + s : s;
+  });
+}
+
+// grid of for_voxels over C x D planes of H x W voxels: four voxels a thread
+dim3 plane_grid(int C, int D, int H, int W) {
+  const int64_t planes = (int64_t)C * D, b = ((int64_t)H * W + 4 * kT - 1) / (4 * kT);
+  return dim3((unsigned)(b < 65536 ? b : 65536), (unsigned)(planes < 65535 ? planes : 65535));
 }
 
 Cells cells(int D, int H, int W) { return Cells{D, H, W, (D + 1) / 2, (H + 1) / 2, (W + 1) / 2}; }
@@ -232,20 +264,19 @@ fwi_status fwi_nn_adam(float *master, uint16_t *w, const float *g, float *m, flo
 fwi_status fwi_nn_pool2_forward(const uint16_t *x, int C, int D, int H, int W, uint16_t *y, void *stream) {
   if (!x || !y || !sizes_ok(C, 1, D, H, W)) return FWI_E_INVAL;
   const Cells g = cells(D, H, W);
-  pool2_fwd_kernel<<<grid_for((int64_t)C * g.Dc * g.Hc * g.Wc), kT, 0, (cudaStream_t)stream>>>(x, C, g, y);
+  pool2_fwd_kernel<<<plane_grid(C, g.Dc, g.Hc, g.Wc), kT, 0, (cudaStream_t)stream>>>(x, C, g, y);
   return launched();
 }
 
 fwi_status fwi_nn_pool2_backward(const float *dy, int C, int D, int H, int W, int accumulate, float *dx, void *stream) {
   if (!dy || !dx || !sizes_ok(C, 1, D, H, W)) return FWI_E_INVAL;
-  pool2_bwd_kernel<<<grid_for((int64_t)C * D * H * W), kT, 0, (cudaStream_t)stream>>>(dy, C, cells(D, H, W),
-                                                                                      accumulate != 0, dx);
+  pool2_bwd_kernel<<<plane_grid(C, D, H, W), kT, 0, (cudaStream_t)stream>>>(dy, C, cells(D, H, W), accumulate != 0, dx);
   return launched();
 }
 
 fwi_status fwi_nn_upsample2_forward(const uint16_t *x, int C, int D, int H, int W, uint16_t *y, void *stream) {
   if (!x || !y || !sizes_ok(C, 1, D, H, W)) return FWI_E_INVAL;
-  up2_fwd_kernel<<<grid_for((int64_t)C * D * H * W), kT, 0, (cudaStream_t)stream>>>(x, C, cells(D, H, W), y);
+  up2_fwd_kernel<<<plane_grid(C, (D + 1) / 2, (H + 1) / 2, W), kT, 0, (cudaStream_t)stream>>>(x, C, cells(D, H, W), y);
   return launched();
 }
 
@@ -253,8 +284,7 @@ fwi_status fwi_nn_upsample2_backward(const float *dy, int C, int D, int H, int W
                                      void *stream) {
   if (!dy || !dx || !sizes_ok(C, 1, D, H, W)) return FWI_E_INVAL;
   const Cells g = cells(D, H, W);
-  up2_bwd_kernel<<<grid_for((int64_t)C * g.Dc * g.Hc * g.Wc), kT, 0, (cudaStream_t)stream>>>(dy, C, g,
-                                                                                             accumulate != 0, dx);
+  up2_bwd_kernel<<<plane_grid(C, g.Dc, g.Hc, g.Wc), kT, 0, (cudaStream_t)stream>>>(dy, C, g, accumulate != 0, dx);
   return launched();
 }
 
