@@ -270,8 +270,8 @@ fwi_status fwi_set_shot_batch(fwi_ctx *ctx, int batch);
 fwi_status fwi_tune_shot_batch(fwi_ctx *ctx, int shot0, int nshots, int max_batch, int steps, double mem_fraction,
                                int *chosen);
 
-/* Picks the launch shapes of the stage kernels by measurement: for each candidate (planes
- * per block of the interior kernel: 4, 8, 16, 32; node pairs per x segment of a PML warp
+/* Picks the launch shapes of the stage kernels by measurement: for each candidate (most
+ * planes per block of the interior kernel, fewer where that fills the GPU better: 4, 8, 16, 32; node pairs per x segment of a PML warp
  * task: 16, 32) it times `steps` forward RK4 steps (1 <= steps < nsteps) of the first
  * shot batch of shots [shot0, shot0 + nshots), keeps the fastest for later calls and
  * returns it in chosen[0] (planes) and chosen[1] (pairs). The shapes change no node's

@@ -20,13 +20,15 @@
 #include "../../include/fwi.h"
 #include "fwi_internal.h"
 
+constexpr int kSides = 3;  // side streams of a stage: interior, interface shell, outer-face nodes
+
 struct fwi_ctx {
   fwi_config cfg{};
   fwi::Geo geo{};
   cudaStream_t stream = nullptr;
-  cudaStream_t side[2] = {nullptr, nullptr};  // the stage's kernels fork onto these and join back
+  cudaStream_t side[kSides] = {};  // the stage's kernels fork onto these and join back
   cudaStream_t cap = nullptr;  // sweeps are recorded on this stream (the caller's may be the legacy one)
-  cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr};
+  cudaEvent_t ev_fork = nullptr, ev_join[kSides] = {};
   bool cuda_failed = false;
   std::string err;
   int64_t nelem = 0, npml_nodes = 0;
@@ -334,13 +336,14 @@ fwi_status check_status(fwi_ctx *c) {
 fwi_status stage(fwi_ctx *c, bool adj, const fwi::StageArgs &a) {
   cudaEvent_t e0;
   time_begin(c, &e0);
-  // fork: interior and interface/face kernels on the side streams, bulk PML here
+  // fork: interior, interface and outer-face kernels on the side streams, bulk PML here
   CUDA_TRY(c, cudaEventRecord(c->ev_fork, c->stream));
-  for (int i = 0; i < 2; i++) CUDA_TRY(c, cudaStreamWaitEvent(c->side[i], c->ev_fork, 0));
+  for (int i = 0; i < kSides; i++) CUDA_TRY(c, cudaStreamWaitEvent(c->side[i], c->ev_fork, 0));
   const int ni = fwi::launch_interior(c->geo, a, c->side[0]);
   if (ni < 0) return fail(c, FWI_E_CUDA, "no tensor map for the stage input (not 16-byte aligned, or no driver entry)");
-  const int nk = ni + fwi::launch_shell(c->geo, a, adj, c->side[1]) + fwi::launch_pml(c->geo, a, adj, c->stream);
-  for (int i = 0; i < 2; i++) {
+  const int nk = ni + fwi::launch_shell(c->geo, a, adj, c->side[1]) + fwi::launch_pml_face(c->geo, a, adj, c->side[2]) +
+                 fwi::launch_pml(c->geo, a, adj, c->stream);
+  for (int i = 0; i < kSides; i++) {
     CUDA_TRY(c, cudaEventRecord(c->ev_join[i], c->side[i]));
     CUDA_TRY(c, cudaStreamWaitEvent(c->stream, c->ev_join[i], 0));
   }
@@ -697,7 +700,7 @@ fwi_status fwi_create(const fwi_config *cfg, fwi_ctx **out) {
   g.stride = (px * nJ * nK + 63) / 64 * 64;
   g.inv_h = (float)(1.0 / cfg->h);
   g.rho = (float)cfg->rho;
-  g.int_kc = 8;
+  g.int_kc = 32;
   g.pml_seg = 32;
   g.inv_rho_h = (float)(1.0 / (cfg->rho * cfg->h));
   g.wdetj = (float)(0.125 * cfg->h * cfg->h * cfg->h);
@@ -738,7 +741,7 @@ fwi_status fwi_create(const fwi_config *cfg, fwi_ctx **out) {
     }
   }
   fwi_status st = FWI_OK;
-  for (int i = 0; i < 2 && st == FWI_OK; i++)
+  for (int i = 0; i < kSides && st == FWI_OK; i++)
     if (cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_join[i], cudaEventDisableTiming) != cudaSuccess)
       st = fail(c, FWI_E_CUDA, "stream setup failed");
@@ -887,7 +890,7 @@ void fwi_destroy(fwi_ctx *c) {
     dfree(*p);
   dfree(c->d_oflags);
   dfree(c->d_omax);
-  for (int i = 0; i < 2; i++) {
+  for (int i = 0; i < kSides; i++) {
     if (c->side[i]) {
       cudaStreamSynchronize(c->side[i]);
       cudaStreamDestroy(c->side[i]);

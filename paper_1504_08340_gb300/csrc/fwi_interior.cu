@@ -184,35 +184,46 @@ __device__ __forceinline__ void node_accel_dispatch(const Tile &t, int sy, int s
   }
 }
 
+// MODE 0: the rate (stage 0), 1: stage 1 (X is the stage input), 2: stages 2-3, 3: stage 4. A
+// template parameter, so that nothing between the loads of a node's own operands and their use
+// after the stencils waits for them.
+//
 // the node's own stage-update operands, loaded before the stencil work so that
 // their latency overlaps it
 struct Own {
   float yd[3];         // u rate of the stage input
-  float x1[3], x2[3];  // u and u rate at the step start
+  float x1[3], x2[3];  // u and u rate at the step start; stage 4: their -X + Y2 + 2 Y3
 };
 
+template <int MODE>
 __device__ __forceinline__ void load_own(const Geo &g, const StageArgs &a, int64_t node, Own &o) {
   const int64_t S = g.stride;
 #pragma unroll
   for (int c = 0; c < 3; c++) {
     const int64_t i1 = (int64_t)(9 + c) * S + node, i2 = (int64_t)(18 + c) * S + node;
     o.yd[c] = __ldg(a.Y + i2);
-    if (a.stage >= 2) {  // in stage 1 X is the stage input
+    if constexpr (MODE >= 2) {
       o.x1[c] = __ldcs(a.X + i1);
       o.x2[c] = __ldcs(a.X + i2);
+    }
+    if constexpr (MODE == 3) {
+      o.x1[c] = -o.x1[c] + __ldcs(a.Y2 + i1) + 2.f * __ldcs(a.Y3 + i1);
+      o.x2[c] = -o.x2[c] + __ldcs(a.Y2 + i2) + 2.f * __ldcs(a.Y3 + i2);
     }
   }
 }
 
-// RK4 stage update (see StageArgs); stage 4 reads Y2 and Y3 here
-__device__ __forceinline__ float stage_value(const StageArgs &a, int64_t idx, float x, float yv, float rate) {
-  if (a.stage == 0) return rate;
-  if (a.stage == 1) return yv + a.cdt * rate;
-  if (a.stage < 4) return x + a.cdt * rate;
-  return (-x + __ldcs(a.Y2 + idx) + 2.f * __ldcs(a.Y3 + idx) + yv) * (1.f / 3.f) + a.cdt * rate;
+// RK4 stage update (see StageArgs), x as load_own left it
+template <int MODE>
+__device__ __forceinline__ float stage_value(const StageArgs &a, float x, float yv, float rate) {
+  if constexpr (MODE == 0) return rate;
+  if constexpr (MODE == 1) return yv + a.cdt * rate;
+  if constexpr (MODE == 2) return x + a.cdt * rate;
+  return (x + yv) * (1.f / 3.f) + a.cdt * rate;
 }
 
 // write the stage outputs of one interior node
+template <int MODE>
 __device__ __forceinline__ void finish_node(const Geo &g, const StageArgs &a, int I, int J, int K, const Tile &t,
                                             const Own &o, const float acc[3]) {
   const int64_t S = g.stride;
@@ -223,12 +234,13 @@ __device__ __forceinline__ void finish_node(const Geo &g, const StageArgs &a, in
   for (int c = 0; c < 3; c++) {
     const int64_t i1 = (int64_t)(9 + c) * S + node, i2 = (int64_t)(18 + c) * S + node;
     const float u1 = t.v<0, 0, 0>(c);
-    const float v1 = stage_value(a, i1, o.x1[c], u1, o.yd[c]);
+    const float v1 = stage_value<MODE>(a, o.x1[c], u1, o.yd[c]);
     __stcs(a.out + (i1), v1);
-    __stcs(a.out + (i2), stage_value(a, i2, o.x2[c], o.yd[c], acc[c]));
-    if (a.hist) a.hist[(int64_t)c * g.nmat + mi] = v1;
+    __stcs(a.out + (i2), stage_value<MODE>(a, o.x2[c], o.yd[c], acc[c]));
+    if constexpr (MODE == 3)
+      if (a.hist) a.hist[(int64_t)c * g.nmat + mi] = v1;
   }
-  if (a.stage == 0) {  // history and stress do not exist on these nodes
+  if constexpr (MODE == 0) {  // history and stress do not exist on these nodes
     for (int f = 0; f < 27; f++)
       if (f % 9 >= 3 || f < 3) __stcs(a.out + ((int64_t)f * S + node), 0.f);
   }
@@ -275,6 +287,7 @@ __device__ __forceinline__ void copy_plane(float *dst, const CUtensorMap *tm, in
 // tm: the u fields of the stage input of the batch (see plane_map); the copies of a plane
 // are numbered from k0 - 2: copy q lands in ring slot q % kRing, and is that slot's
 // (q / kRing)-th phase
+template <int MODE>
 __global__ void __launch_bounds__(kTP *kTY, FWI_INT_MINB)
     interior_kernel(const __grid_constant__ CUtensorMap tm, Geo g, StageArgs a0) {
   float *smem = s_ring;
@@ -341,19 +354,19 @@ __global__ void __launch_bounds__(kTP *kTY, FWI_INT_MINB)
     const bool e_ok = got && even_ok && node_ok(g, kSiteInterior, rowbase + IE);
     const bool o_ok = got && odd_ok && node_ok(g, kSiteInterior, rowbase + IO);
     Own oe, oo;
-    if (e_ok) load_own(g, a, rowbase + IE, oe);
-    if (o_ok) load_own(g, a, rowbase + IO, oo);
+    if (e_ok) load_own<MODE>(g, a, rowbase + IE, oe);
+    if (o_ok) load_own<MODE>(g, a, rowbase + IO, oo);
     if (e_ok) {
       float acc[3];
       node_accel_dispatch<kEven>(t, sy, sz, sc, acc);
-      finish_node(g, a, IE, J, K, t, oe, acc);
+      finish_node<MODE>(g, a, IE, J, K, t, oe, acc);
     }
     t.o += 1;
     t.mi += 1;
     if (o_ok) {
       float acc[3];
       node_accel_dispatch<kOdd>(t, sy, sz, sc, acc);
-      finish_node(g, a, IO, J, K, t, oo, acc);
+      finish_node<MODE>(g, a, IO, J, K, t, oo, acc);
     }
     if (__syncthreads_or(!got)) {
       ok = false;
@@ -405,18 +418,30 @@ bool plane_map(const Geo &g, const StageArgs &a, CUtensorMap *tm) {
 }  // namespace
 
 cudaError_t prepare_interior() {
-  return cudaFuncSetAttribute(interior_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  for (auto kernel : {interior_kernel<0>, interior_kernel<1>, interior_kernel<2>, interior_kernel<3>}) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
-int launch_interior(const Geo &g, const StageArgs &a, cudaStream_t s) {
+int launch_interior(const Geo &g0, const StageArgs &a, cudaStream_t s) {
+  Geo g = g0;
   if (g.box_hi[0] < g.box_lo[0] || g.box_hi[1] < g.box_lo[1] || g.box_hi[2] < g.box_lo[2]) return 0;
   const int nx = g.box_hi[0] - (g.box_lo[0] - 1) + 1;
-  const dim3 grd((nx + 2 * kTP - 1) / (2 * kTP), (g.box_hi[1] - g.box_lo[1] + kTY) / kTY,
+  const int tx = (nx + 2 * kTP - 1) / (2 * kTP), ty = (g.box_hi[1] - g.box_lo[1] + kTY) / kTY;
+  // a ring fill costs about 1.5 planes: 5 planes of copies against 4.5 us per computed plane
+  g.int_kc = chunk_planes((int64_t)tx * ty * a.nshot, g.box_hi[2] - g.box_lo[2] + 1, FWI_INT_MINB * kSms, g0.int_kc, 1.5);
+  const dim3 grd(tx, ty,
                  (g.box_hi[2] - g.box_lo[2] + g.int_kc) / g.int_kc * a.nshot);
   CUtensorMap tm;
   std::memset(&tm, 0, sizeof(tm));
   if (!plane_map(g, a, &tm)) return -1;
-  interior_kernel<<<grd, dim3(kTP, kTY), kSmem, s>>>(tm, g, a);
+  const auto kernel = a.stage == 0   ? interior_kernel<0>
+                      : a.stage == 1 ? interior_kernel<1>
+                      : a.stage < 4  ? interior_kernel<2>
+                                     : interior_kernel<3>;
+  kernel<<<grd, dim3(kTP, kTY), kSmem, s>>>(tm, g, a);
   return 1;
 }
 

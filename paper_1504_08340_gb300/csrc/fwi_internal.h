@@ -63,7 +63,7 @@ struct Geo {
   long long wait_cycles;
   int copy_extra;
   // launch shapes (fwi_tune_tiles; they change no node's arithmetic)
-  int int_kc;             // planes per block of interior_kernel
+  int int_kc;             // most planes per block of interior_kernel (see chunk_planes)
   int pml_seg;            // node pairs per x segment of a pml_kernel warp task (<= 32)
 };
 
@@ -84,6 +84,27 @@ struct StageArgs {
   int nshot;
   int64_t sstride, hstride;
 };
+
+// Planes per block of a kernel whose blocks march along z: the power of two up to `most` that
+// takes the fewest plane steps, ceil(blocks / slots) (k + start), for `tiles` (x, y) tiles of
+// all shots, `planes` planes and `slots` blocks resident on the GPU; `start` is the cost of
+// filling a block's ring, in planes. Long chunks save ring fills on large grids; on small
+// ones they leave the SMs idle (16x16x8 elements: 8 blocks of 8 planes took 36 us where 64
+// blocks of one plane take 12 us).
+inline int chunk_planes(int64_t tiles, int planes, int slots, int most, double start) {
+  int best = 1;
+  double cost = -1.0;
+  for (int k = 1; k <= most; k *= 2) {
+    const int64_t blocks = tiles * ((planes + k - 1) / k);
+    const double c = (double)((blocks + slots - 1) / slots) * (k + start);
+    if (cost < 0.0 || c <= cost) {
+      cost = c;
+      best = k;
+    }
+  }
+  return best;
+}
+constexpr int kSms = 152;
 
 // the buffers of shot `shot` of the batch
 __host__ __device__ inline StageArgs shot_args(StageArgs a, int shot) {
@@ -109,8 +130,8 @@ __device__ __forceinline__ bool node_ok(const Geo &g, int site, long long node) 
 //                   the tensor map of the stage input could not be encoded (Y not
 //                   16-byte aligned, or the driver entry point missing);
 //  launch_pml:      nodes all of whose elements are PML, off the outer faces (fwi_pml.cu);
-//  launch_shell:    the interface shell (fwi_stage.cu) and the PML nodes on the
-//                   outer faces of the grid (launch_pml_face, fwi_pml.cu).
+//  launch_shell:    the interface shell (fwi_stage.cu);
+//  launch_pml_face: the PML nodes on the outer faces of the grid (fwi_pml.cu).
 int launch_interior(const Geo &g, const StageArgs &a, cudaStream_t s);
 int launch_pml(const Geo &g, const StageArgs &a, bool adjoint, cudaStream_t s);
 int launch_pml_face(const Geo &g, const StageArgs &a, bool adjoint, cudaStream_t s);

@@ -53,14 +53,15 @@ __global__ void sample_kernel(const float *buf, int64_t stride, int nrec, const 
 // (C.1f)/(C.1g) at one time level, in FP64: for every interior node, the sum over the
 // interior elements around it of W detJ times the products of the element-wise
 // gradients of w and u. A block owns a 32 x 8 tile of interior nodes in
-// (x, y) and marches up a chunk of kGKC levels in z. Plane k of the six fields (w and
+// (x, y) and marches up a chunk of kc levels in z. Plane k of the six fields (w and
 // u, three components each) is staged with its two-node x/y halo in a six-slot ring
 // by 4-byte cp.async; the copies of plane k + 3 are in flight while level k is
 // computed from planes k-2 .. k+2, so a level costs one barrier. Every derivative
 // candidate of an axis (C, or L and R) is formed from the five staged values and the
 // one the node's parity asks for is selected, so the x parity alternating across a
 // warp costs no divergence in the stencils.
-constexpr int kGX = 32, kGY = 8, kGKC = 16, kGH = 2;
+constexpr int kGX = 32, kGY = 8, kGKC = 16, kGH = 2;  // kGKC: most levels of a chunk
+constexpr int kGBlocks = 3;                           // blocks per SM
 constexpr int kGW = kGX + 2 * kGH, kGR = kGY + 2 * kGH, kGP = kGW * kGR;  // staged positions per plane
 constexpr int kGSlots = 6, kGFields = 6;
 constexpr size_t kGSmem = sizeof(float) * kGSlots * kGFields * kGP;
@@ -98,14 +99,14 @@ __device__ __forceinline__ void grad_axis(float a, float b, float c, float d, fl
   s1 = (-3.f * c + 4.f * d - e) * inv_h;
 }
 
-__global__ void __launch_bounds__(kGX *kGY, 3) gradient_kernel(Geo g, const float *__restrict__ ws0,
+__global__ void __launch_bounds__(kGX *kGY, kGBlocks) gradient_kernel(Geo g, const float *__restrict__ ws0,
                                                                      const float *__restrict__ uh0, double wdt,
                                                                      double *gl, double *gm, int nshot,
-                                                                     int64_t sstride, int64_t hstride) {
+                                                                     int64_t sstride, int64_t hstride, int kc) {
   extern __shared__ float ring[];
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kGX + tx;
-  const int x0 = blockIdx.x * kGX, y0 = blockIdx.y * kGY, k0 = blockIdx.z * kGKC;
-  const int m2 = g.m[2], k1 = min(k0 + kGKC, m2);
+  const int x0 = blockIdx.x * kGX, y0 = blockIdx.y * kGY, k0 = blockIdx.z * kc;
+  const int m2 = g.m[2], k1 = min(k0 + kc, m2);
   const int i = x0 + tx, j = y0 + ty;
   const bool own = i < g.m[0] && j < g.m[1];
   // element sides present along each axis: odd coordinate -> the one element it is
@@ -248,9 +249,10 @@ void launch_gradient(const Geo &g, const float *w_state, const float *u_hist, do
     cudaFuncSetAttribute(gradient_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGSmem);
     attr = true;
   }
-  const dim3 grid((g.m[0] + kGX - 1) / kGX, (g.m[1] + kGY - 1) / kGY, (g.m[2] + kGKC - 1) / kGKC);
-  gradient_kernel<<<grid, dim3(kGX, kGY), kGSmem, s>>>(g, w_state, u_hist, wdt, gl, gm, nshot, sstride,
-                                                             hstride);
+  const int tx = (g.m[0] + kGX - 1) / kGX, ty = (g.m[1] + kGY - 1) / kGY;
+  const int kc = chunk_planes((int64_t)tx * ty, g.m[2], kGBlocks * kSms, kGKC, 2.5);
+  gradient_kernel<<<dim3(tx, ty, (g.m[2] + kc - 1) / kc), dim3(kGX, kGY), kGSmem, s>>>(g, w_state, u_hist, wdt, gl, gm,
+                                                                                     nshot, sstride, hstride, kc);
 
 }
 

@@ -315,37 +315,66 @@ __device__ __forceinline__ NodeCtx node_ctx(const Geo &g, int I, int J, int K) {
 // interior and PML elements (and, without a PML, the fixed outer faces). Their
 // node numbers come from a list built once per context (g.shell, g.nshell).
 //
-// A block owns 32 list nodes and has three warps. In the first phase warp j forms
-// the axis-j terms of every sum at its nodes (the element line quadratures along j
-// of the u rows, column j of H of the S rows) and leaves them in shared memory; in
-// the second phase warp w writes displacement component w and stress components
-// w and w + 3 of the same nodes.
+// A block owns 32 list nodes and has three or six warps. In the first phase warp j (and 3 + j)
+// forms the axis-j terms of every sum at its nodes and leaves them in shared memory: the
+// interior elements' line quadratures of the u rows, the PML elements', and column j of H of
+// the S rows. In the second phase warp w writes displacement component w and stress components
+// w and w + 3 of the same nodes. With six warps the interior and the PML elements' terms are
+// two warps' work: each warp's sums are a chain of dependent load rounds, and on a mesh whose
+// blocks do not fill the SMs that chain is the kernel's time (8x8x4 elements, 78 blocks: 26
+// against 20 us). Where they do, three warps are the faster form, since each warp computes its
+// nodes' coefficients anew (64x64x32: 59 against 67 us).
 constexpr int kShellNodes = 32;
 
 struct ShellShared {
-  float f[3][3][kShellNodes];  // [axis][component][node]: u-row terms s_rd fr + s_pml fp of one axis
+  float fr[3][3][kShellNodes], fp[3][3][kShellNodes];  // [axis][component][node]: u-row terms of one axis
   float H[3][3][kShellNodes];  // [i][j][node]
 };
 
+// axis-J terms of the node: of the interior elements (rd) and of the PML elements (pm)
 template <bool ADJ, int J>
-__device__ __forceinline__ void shell_axis(const Geo &g, const StageArgs &a, const NodeCtx &n, ShellShared &sh,
-                                           int lane) {
+__device__ __forceinline__ void shell_axis(const Geo &g, const StageArgs &a, const NodeCtx &n, ShellShared &sh, int lane,
+                                           bool rd, bool pm) {
   const float *__restrict__ Y = a.Y;
   const int64_t S = g.stride;
-  if (!n.dir) {
-    float fr[3] = {0.f, 0.f, 0.f}, fp[3] = {0.f, 0.f, 0.f};
+  if (rd && !n.dir) {
+    float fr[3] = {0.f, 0.f, 0.f};
     interior_force_axis<J>(g, Y + 9 * S, n.node, n.c3, n.st, n.ax, false, fr);
-    if (n.pml) pml_force_axis<ADJ, J>(g, Y, n.node, n.c3, n.st, n.ax, n.Le, n.Lp, n.Lw, fp);
-    const float s_rd = g.inv_h * g.inv_h * (1.f / 3.f), s_pml = g.inv_h * (1.f / 3.f);
 #pragma unroll
-    for (int c = 0; c < 3; c++) sh.f[J][c][lane] = s_rd * fr[c] + s_pml * fp[c];
+    for (int c = 0; c < 3; c++) sh.fr[J][c][lane] = fr[c];
   }
-  if (n.pml) {
+  if (pm && !n.dir) {
+    float fp[3] = {0.f, 0.f, 0.f};
+    if (n.pml) pml_force_axis<ADJ, J>(g, Y, n.node, n.c3, n.st, n.ax, n.Le, n.Lp, n.Lw, fp);
+#pragma unroll
+    for (int c = 0; c < 3; c++) sh.fp[J][c][lane] = fp[c];
+  }
+  if (pm && n.pml) {
     float H[3][3];
     pml_strain_axis<J>(g, Y, n.node, n.st, n.ax, n.Le, n.Lp, n.Lw, H);
 #pragma unroll
     for (int i = 0; i < 3; i++) sh.H[i][J][lane] = H[i][J];
   }
+}
+
+// first phase of warp w of W
+template <bool ADJ, int W>
+__device__ __forceinline__ void shell_terms(const Geo &g, const StageArgs &a, const NodeCtx &n, ShellShared &sh, int lane,
+                                            int w) {
+  const int j = w % 3;
+  const bool rd = W == 3 || w < 3, pm = W == 3 || w >= 3;
+  if (j == 0) shell_axis<ADJ, 0>(g, a, n, sh, lane, rd, pm);
+  else if (j == 1) shell_axis<ADJ, 1>(g, a, n, sh, lane, rd, pm);
+  else shell_axis<ADJ, 2>(g, a, n, sh, lane, rd, pm);
+}
+
+// u-row force of component c
+__device__ __forceinline__ float shell_force(const Geo &g, const ShellShared &sh, int c, int lane) {
+  const float s_rd = g.inv_h * g.inv_h * (1.f / 3.f), s_pml = g.inv_h * (1.f / 3.f);
+  float f[3];
+#pragma unroll
+  for (int j = 0; j < 3; j++) f[j] = s_rd * sh.fr[j][c][lane] + s_pml * sh.fp[j][c][lane];
+  return f[0] + f[1] + f[2];
 }
 
 // stress component c (order xx yy zz yz xz xy) of the node: its three levels
@@ -396,7 +425,7 @@ __device__ __forceinline__ void shell_disp(const Geo &g, const StageArgs &a, con
     }
     return;
   }
-  const float fsum = sh.f[0][c][lane] + sh.f[1][c][lane] + sh.f[2][c][lane];
+  const float fsum = shell_force(g, sh, c, lane);
   const float inv_m = n.inv_a / (g.rho * (float)n.nel);
   const float u0 = __ldg(Y + i0), u1 = __ldg(Y + i1), u2 = __ldg(Y + i2);
   const float acc = -fsum * inv_m - (n.cb * u2 + n.cc * u1 + n.cd * u0) * n.inv_a;
@@ -407,11 +436,8 @@ __device__ __forceinline__ void shell_disp(const Geo &g, const StageArgs &a, con
   if (a.hist) write_hist(g, a, n.c3[0], n.c3[1], n.c3[2], c, v1);
 }
 
-#ifndef FWI_SHELL_MINB
-#define FWI_SHELL_MINB 8
-#endif
-template <bool ADJ>
-__global__ void __launch_bounds__(3 * kShellNodes, FWI_SHELL_MINB) shell_kernel(Geo g, StageArgs a0) {
+template <bool ADJ, int W>
+__global__ void __launch_bounds__(W *kShellNodes, 24 / W) shell_kernel(Geo g, StageArgs a0) {
   __shared__ ShellShared sh;
   const int nbs = (g.nshell + kShellNodes - 1) / kShellNodes;  // blocks per shot
   const StageArgs a = shot_args(a0, blockIdx.x / nbs);
@@ -423,15 +449,12 @@ __global__ void __launch_bounds__(3 * kShellNodes, FWI_SHELL_MINB) shell_kernel(
     const int node = g.shell[i];
     const int I = node % g.px, r = node / g.px;
     n = node_ctx(g, I, r % g.n[1], r / g.n[1]);
-    if (w == 0) shell_axis<ADJ, 0>(g, a, n, sh, lane);
-    else if (w == 1) shell_axis<ADJ, 1>(g, a, n, sh, lane);
-    else shell_axis<ADJ, 2>(g, a, n, sh, lane);
+    shell_terms<ADJ, W>(g, a, n, sh, lane, w);
   }
   __syncthreads();
   if (live) {
-    shell_disp(g, a, n, sh, lane, w);
-    shell_stress<ADJ>(g, a, n, sh, lane, w);
-    shell_stress<ADJ>(g, a, n, sh, lane, w + 3);
+    if (w < 3) shell_disp(g, a, n, sh, lane, w);
+    for (int c = w; c < 6; c += W) shell_stress<ADJ>(g, a, n, sh, lane, c);
   }
 }
 
@@ -480,7 +503,7 @@ __device__ __forceinline__ void persist_disp(const Geo &g, const StageArgs &a, c
   const float *__restrict__ Y = a.Y;
   const int64_t i0 = (int64_t)c * S + n.node, i1 = (int64_t)(9 + c) * S + n.node, i2 = (int64_t)(18 + c) * S + n.node;
   if (n.dir) return;
-  const float fsum = sh.f[0][c][lane] + sh.f[1][c][lane] + sh.f[2][c][lane];
+  const float fsum = shell_force(g, sh, c, lane);
   const float inv_m = n.inv_a / (g.rho * (float)n.nel);
   const float u0 = __ldg(Y + i0), u1 = __ldg(Y + i1), u2 = __ldg(Y + i2);
   const float acc = -fsum * inv_m - (n.cb * u2 + n.cc * u1 + n.cd * u0) * n.inv_a;
@@ -501,7 +524,11 @@ __device__ __forceinline__ void persist_disp(const Geo &g, const StageArgs &a, c
   }
 }
 
-__global__ void __launch_bounds__(3 * kShellNodes) persistent_forward_kernel(Geo g, PersistArgs p) {
+// six warps a block: the sweep is meant for meshes of about one wave of blocks, where a stage
+// takes one node chunk's chain of loads (8x8x4 elements, a 100-step sweep: 7.07 ms; with three
+// warps and 4 blocks an SM 8.09 ms, with six warps and 2 blocks 8.71 ms)
+constexpr int kPersistWarps = 6;
+__global__ void __launch_bounds__(kPersistWarps *kShellNodes, 3) persistent_forward_kernel(Geo g, PersistArgs p) {
   __shared__ ShellShared sh;
   const int lane = threadIdx.x, w = threadIdx.y;
   const int nch = (p.nall + kShellNodes - 1) / kShellNodes;  // node chunks per shot
@@ -531,15 +558,12 @@ __global__ void __launch_bounds__(3 * kShellNodes) persistent_forward_kernel(Geo
           const int node = p.nodes[i];
           const int I = node % g.px, r = node / g.px;
           n = node_ctx(g, I, r % g.n[1], r / g.n[1]);
-          if (w == 0) shell_axis<false, 0>(g, a, n, sh, lane);
-          else if (w == 1) shell_axis<false, 1>(g, a, n, sh, lane);
-          else shell_axis<false, 2>(g, a, n, sh, lane);
+          shell_terms<false, kPersistWarps>(g, a, n, sh, lane, w);
         }
         __syncthreads();
         if (live) {
-          persist_disp(g, a, n, sh, lane, w, p, b, step, s);
-          shell_stress<false>(g, a, n, sh, lane, w);
-          shell_stress<false>(g, a, n, sh, lane, w + 3);
+          if (w < 3) persist_disp(g, a, n, sh, lane, w, p, b, step, s);
+          for (int c = w; c < 6; c += kPersistWarps) shell_stress<false>(g, a, n, sh, lane, c);
         }
         __syncthreads();
       }
@@ -555,14 +579,14 @@ cudaError_t launch_persistent_forward(const Geo &g, const PersistArgs &p, cudaSt
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_forward_kernel, 3 * kShellNodes, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_forward_kernel, kPersistWarps * kShellNodes, 0);
   if (e != cudaSuccess) return e;
   const int chunks = (p.nall + kShellNodes - 1) / kShellNodes * p.nshot;
   const int grid = std::max(1, std::min(per_sm * nsm, chunks));
   Geo gg = g;
   PersistArgs pp = p;
   void *args[2] = {&gg, &pp};
-  return cudaLaunchCooperativeKernel((const void *)persistent_forward_kernel, dim3(grid), dim3(kShellNodes, 3), args,
+  return cudaLaunchCooperativeKernel((const void *)persistent_forward_kernel, dim3(grid), dim3(kShellNodes, kPersistWarps), args,
                                      0, s);
 }
 
@@ -571,13 +595,12 @@ int launch_shell(const Geo &g, const StageArgs &a, bool adjoint, cudaStream_t s)
   if (g.nshell > 0) {
     n = 1;
     const int nb = (g.nshell + kShellNodes - 1) / kShellNodes * a.nshot;
-    const dim3 blk(kShellNodes, 3);
-    if (adjoint)
-      shell_kernel<true><<<nb, blk, 0, s>>>(g, a);
-    else
-      shell_kernel<false><<<nb, blk, 0, s>>>(g, a);
+    const bool six = nb <= 2 * kSms;
+    const auto kernel = adjoint ? (six ? shell_kernel<true, 6> : shell_kernel<true, 3>)
+                                : (six ? shell_kernel<false, 6> : shell_kernel<false, 3>);
+    kernel<<<nb, dim3(kShellNodes, six ? 6 : 3), 0, s>>>(g, a);
   }
-  return n + launch_pml_face(g, a, adjoint, s);
+  return n;
 }
 
 }  // namespace fwi
