@@ -46,6 +46,8 @@ struct fwi_ctx {
 
   int nshots = 0;
   std::vector<int64_t> src_node;
+  int src_k[2] = {1, 0}, rec_k[2] = {1, 0};  // planes (first, last) that hold sources, receivers
+  bool src_pml = false, rec_pml = false;     // some of them on a node of pml_kernel
   std::vector<double> src_dir;
   int wavelet = 0;
   double wparams[3] = {0, 0, 0};
@@ -102,7 +104,7 @@ struct fwi_ctx {
   bool persistent = false;
   double wait_ms = 1000.0;
   int bar_extra = 0;
-  int *d_all = nullptr, *d_rec_of = nullptr;  // every node; node -> receiver index
+  int *d_all = nullptr, *d_rec_of = nullptr;  // every node; node -> receiver index (or -1)
   unsigned *d_bar = nullptr;
   int *d_status = nullptr;                    // FWI_E_TIMEOUT when a bounded device wait gave up
 
@@ -181,6 +183,14 @@ size_t snap_floats(const fwi_ctx *c) { return (size_t)6 * c->geo.stride + (size_
 bool is_dirichlet(const fwi_ctx *c, int i, int j, int k) {
   const int *n = c->geo.n;
   return i == 0 || i == n[0] - 1 || j == 0 || j == n[1] - 1 || k == n[2] - 1 || (c->geo.top_dir && k == 0);
+}
+
+// a node of pml_kernel: off the grid's faces and outside the closed interior box
+bool is_deep_pml(const fwi_ctx *c, int i, int j, int k) {
+  const fwi::Geo &g = c->geo;
+  if (i == 0 || i == g.n[0] - 1 || j == 0 || j == g.n[1] - 1 || k == 0 || k == g.n[2] - 1) return false;
+  return !(i >= 2 * g.lo[0] && i <= 2 * g.hi[0] && j >= 2 * g.lo[1] && j <= 2 * g.hi[1] && k >= 2 * g.lo[2] &&
+           k <= 2 * g.hi[2]);
 }
 
 // number of elements containing node coordinate cc along axis ax
@@ -333,20 +343,21 @@ fwi_status check_status(fwi_ctx *c) {
   return FWI_OK;
 }
 
-fwi_status stage(fwi_ctx *c, bool adj, const fwi::StageArgs &a) {
+fwi_status stage(fwi_ctx *c, bool adj, const fwi::StageArgs &a, const fwi::Points &q, bool pml_points) {
   cudaEvent_t e0;
   time_begin(c, &e0);
   // fork: interior, interface and outer-face kernels on the side streams, bulk PML here
   CUDA_TRY(c, cudaEventRecord(c->ev_fork, c->stream));
   for (int i = 0; i < kSides; i++) CUDA_TRY(c, cudaStreamWaitEvent(c->side[i], c->ev_fork, 0));
-  const int ni = fwi::launch_interior(c->geo, a, c->side[0]);
+  const int ni = fwi::launch_interior(c->geo, a, q, c->side[0]);
   if (ni < 0) return fail(c, FWI_E_CUDA, "no tensor map for the stage input (not 16-byte aligned, or no driver entry)");
-  const int nk = ni + fwi::launch_shell(c->geo, a, adj, c->side[1]) + fwi::launch_pml_face(c->geo, a, adj, c->side[2]) +
-                 fwi::launch_pml(c->geo, a, adj, c->stream);
+  int nk = ni + fwi::launch_shell(c->geo, a, q, adj, c->side[1]) +
+           fwi::launch_pml_face(c->geo, a, q, adj, c->side[2]) + fwi::launch_pml(c->geo, a, adj, c->stream);
   for (int i = 0; i < kSides; i++) {
     CUDA_TRY(c, cudaEventRecord(c->ev_join[i], c->side[i]));
     CUDA_TRY(c, cudaStreamWaitEvent(c->stream, c->ev_join[i], 0));
   }
+  if (q.k0 <= q.k1 && (!q.fused || pml_points)) nk += fwi::launch_points(c->geo, a, q, c->d_rec_node, c->stream);
   time_end(c, e0, 0);
   c->t_launch[3] += nk - 1;  // time_end counted the stage once; count its kernels
   CUDA_TRY(c, cudaGetLastError());
@@ -354,12 +365,19 @@ fwi_status stage(fwi_ctx *c, bool adj, const fwi::StageArgs &a) {
   return FWI_OK;
 }
 
-fwi_status point(fwi_ctx *c, const fwi::PointArgs &p) {
-  fwi::launch_point(p, c->stream);
-  c->t_launch[2]++;
-  c->t_launch[3]++;
-  CUDA_TRY(c, cudaGetLastError());
-  return FWI_OK;
+// nodes of all shots of a launch up to which the stage kernels apply the points (see Points;
+// at 2.4 M nodes, 64x64x32, fused 75.0 against 75.8 ms, at 25 M, four shots of 96x96x48, 277.1
+// against 274.9 ms)
+constexpr int64_t kFusedNodes = 8000000;
+
+// the sources of the shots from shot0 on as load 1
+void source_points(const fwi_ctx *c, int shot0, fwi::Points *q) {
+  q->load = 1;
+  q->src_node = c->d_src_node + shot0;
+  q->src_vec = c->d_src_vec + 3 * shot0;
+  q->table = c->d_wave;
+  q->k0 = c->src_k[0];
+  q->k1 = c->src_k[1];
 }
 
 fwi_status zero_state(fwi_ctx *c) {
@@ -373,8 +391,11 @@ fwi_status zero_state(fwi_ctx *c) {
 // samples, or receiver residuals). Both run the forward stage kernels (see below); the
 // transposed kernels serve fwi_rhs's adjoint rate.
 // nb shots (shot0 .. shot0 + nb - 1 for the sources) advance together; shot b's history
-// level goes to hist_slot + b * hstride
-fwi_status rk4_step(fwi_ctx *c, bool adj, int n, int shot0, int nb, float *hist_slot, int64_t hstride) {
+// level goes to hist_slot + b * hstride; sample: a forward step's receiver samples go to
+// d_traces. Point loads and samples are done by the stage kernels' threads that own the
+// nodes (a kernel of their own after each stage had cost about 4 us, five times a step)
+fwi_status rk4_step(fwi_ctx *c, bool adj, int n, int shot0, int nb, float *hist_slot, int64_t hstride,
+                    bool sample = false) {
   const float dt = (float)c->cfg.dt;
   float *X = c->state[0], *Y2 = c->state[1], *Y3 = c->state[2], *Y4 = c->state[3];
   const float *ins[4] = {X, Y2, Y3, Y4};
@@ -394,41 +415,42 @@ fwi_status rk4_step(fwi_ctx *c, bool adj, int n, int shot0, int nb, float *hist_
     a.nshot = nb;
     a.sstride = (int64_t)set_floats(c);
     a.hstride = hstride;
+    fwi::Points q{};
+    q.nrec = c->nrec;
+    q.rec_of = c->d_rec_of;
+    q.tstride = (int64_t)trace_floats(c);
+    q.i1 = -1;
+    q.fused = (int64_t)nb * c->geo.nnode <= kFusedNodes;
+    bool pml_points = false;
+    if (!adj) {
+      // stage times t_n, t_n + dt/2, t_n + dt/2, t_n + dt; wavelet sampled every dt/2. The
+      // last stage's output is the state at t_{n+1}, sampled at the receivers
+      source_points(c, shot0, &q);
+      q.i0 = (s == 0) ? 2 * n : (s == 3 ? 2 * n + 2 : 2 * n + 1);
+      pml_points = c->src_pml;
+      if (s == 3 && sample) {
+        q.traces = c->d_traces + (int64_t)(n + 1) * c->nrec * 3;
+        q.k0 = std::min(q.k0, c->rec_k[0]);
+        q.k1 = std::max(q.k1, c->rec_k[1]);
+        pml_points = pml_points || c->rec_pml;
+      }
+    } else {
+      // reversed time: s_m <-> t_{N-m}; half steps use the mean of the two samples
+      q.load = 2;
+      q.rec_vec = c->d_rec_vec;
+      q.table = c->d_resid;
+      q.i0 = (s == 3) ? N - n - 1 : N - n;
+      q.i1 = (s == 1 || s == 2) ? N - n - 1 : -1;
+      q.k0 = c->rec_k[0];
+      q.k1 = c->rec_k[1];
+      pml_points = c->rec_pml;
+    }
     // The adjoint sweep advances (w, W = tau(T)) rather than (w, T): tau is linear,
     // node-local and constant in time, so applied to the transposed system's stress rows it
     // gives exactly the forward system's form (tau on P(H) in the S rows, the plain stress
     // columns in the u rows), and the forward stage kernels advance it. The displacement w,
     // all the gradient reads, is the same; the stress slots hold tau(T).
-    TRY(stage(c, false, a));
-    fwi::PointArgs p{};
-    p.nnode_pad = (int64_t)c->geo.px * c->geo.n[1] * c->geo.n[2];
-    p.oob = c->geo.oob;
-    p.buf = outs[s];
-    p.stride = c->geo.stride;
-    p.cdt = cdt[s];
-    p.nshot = nb;
-    p.sstride = (int64_t)set_floats(c);
-    p.tstride = (int64_t)trace_floats(c);
-    if (!adj) {
-      // stage times t_n, t_n + dt/2, t_n + dt/2, t_n + dt; wavelet sampled every dt/2
-      p.mode = 0;
-      p.npts = 1;
-      p.node = c->d_src_node + shot0;
-      p.vec = c->d_src_vec + 3 * shot0;
-      p.table = c->d_wave;
-      p.i0 = (s == 0) ? 2 * n : (s == 3 ? 2 * n + 2 : 2 * n + 1);
-      p.i1 = -1;
-    } else {
-      // reversed time: s_m <-> t_{N-m}; half steps use the mean of the two samples
-      p.mode = 1;
-      p.npts = c->nrec;
-      p.node = c->d_rec_node;
-      p.vec = c->d_rec_vec;
-      p.table = c->d_resid;
-      p.i0 = (s == 3) ? N - n - 1 : N - n;
-      p.i1 = (s == 1 || s == 2) ? N - n - 1 : -1;
-    }
-    TRY(point(c, p));
+    TRY(stage(c, false, a, q, pml_points));
   }
   return FWI_OK;
 }
@@ -511,17 +533,9 @@ fwi_status forward_sweep_body(fwi_ctx *c, int shot0, int nb, float *hist, int64_
   if (hist)
     for (int b = 0; b < nb; b++)
       CUDA_TRY(c, cudaMemsetAsync(hist + b * hstride, 0, sizeof(float) * hstep, c->stream));
-  fwi::launch_sample(c->state[0], c->geo.stride, c->nrec, c->d_rec_node, c->d_traces, c->stream, nb,
-                     (int64_t)sfloats, tf, c->geo.oob);
+  // the samples at t_0: the state is zero
+  CUDA_TRY(c, cudaMemset2DAsync(c->d_traces, sizeof(float) * tf, 0, sizeof(float) * per_step, nb, c->stream));
   if (c->persistent) {
-    if (!c->d_rec_of) {
-      std::vector<int> rec_of((size_t)c->geo.stride, -1);
-      for (int r = 0; r < c->nrec; r++) rec_of[(size_t)c->rec_node[r]] = r;
-      TRY(dalloc(c, &c->d_rec_of, rec_of.size()));
-      CUDA_TRY(c, cudaMemcpyAsync(c->d_rec_of, rec_of.data(), sizeof(int) * rec_of.size(), cudaMemcpyHostToDevice,
-                                  c->stream));
-      CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    }
     // one cooperative launch per checkpoint segment (the whole sweep without snapshots)
     fwi::PersistArgs p{};
     for (int b = 0; b < 4; b++) p.st[b] = c->state[b];
@@ -530,13 +544,15 @@ fwi_status forward_sweep_body(fwi_ctx *c, int shot0, int nb, float *hist, int64_
     p.dt = (float)c->cfg.dt;
     p.nodes = c->d_all;
     p.nall = (int)c->geo.nnode;
-    p.src_node = c->d_src_node + shot0;
-    p.src_vec = c->d_src_vec + 3 * shot0;
-    p.wave = c->d_wave;
-    p.rec_of = c->d_rec_of;
-    p.traces = c->d_traces;
-    p.tstride = tf;
-    p.nrec = c->nrec;
+    source_points(c, shot0, &p.pts);
+    p.pts.fused = true;  // every node set
+    p.pts.i1 = -1;
+    p.pts.nrec = c->nrec;
+    p.pts.rec_of = c->d_rec_of;
+    p.pts.tstride = tf;
+    p.pts.traces = c->d_traces;
+    p.pts.k0 = std::min(p.pts.k0, c->rec_k[0]);
+    p.pts.k1 = std::max(p.pts.k1, c->rec_k[1]);
     p.hist = hist;
     p.hstep = (int64_t)hstep;
     p.hstride = hstride;
@@ -558,11 +574,7 @@ fwi_status forward_sweep_body(fwi_ctx *c, int shot0, int nb, float *hist, int64_
   }
   for (int n = 0; n < c->cfg.nsteps; n++) {
     if (snap && n % every == 0) TRY(take_snapshot(c, snap, n / every, nseg, nb));
-    TRY(rk4_step(c, false, n, shot0, nb, hist ? hist + (size_t)(n + 1) * hstep : nullptr, hstride));
-    fwi::launch_sample(c->state[0], c->geo.stride, c->nrec, c->d_rec_node, c->d_traces + (n + 1) * per_step,
-                       c->stream, nb, (int64_t)sfloats, tf, c->geo.oob);
-    c->t_launch[2]++;
-    c->t_launch[3]++;
+    TRY(rk4_step(c, false, n, shot0, nb, hist ? hist + (size_t)(n + 1) * hstep : nullptr, hstride, true));
   }
   CUDA_TRY(c, cudaGetLastError());
   return FWI_OK;
@@ -965,12 +977,17 @@ fwi_status fwi_set_sources(fwi_ctx *c, int nshots, const int *node_ijk, const do
   if (wavelet == FWI_WAVELET_GAUSS && !(wparams[1] > 0)) return fail(c, FWI_E_INVAL, "gauss sigma must be > 0");
   std::vector<int64_t> nodes(nshots);
   std::vector<float> vec(3 * (size_t)nshots);
+  int k0 = c->geo.n[2], k1 = -1;
+  bool pml = false;
   for (int s = 0; s < nshots; s++) {
     const int i = node_ijk[3 * s], j = node_ijk[3 * s + 1], k = node_ijk[3 * s + 2];
     if (i < 0 || j < 0 || k < 0 || i >= c->geo.n[0] || j >= c->geo.n[1] || k >= c->geo.n[2])
       return fail(c, FWI_E_INVAL, "source %d node (%d,%d,%d) outside the mesh", s, i, j, k);
     if (is_dirichlet(c, i, j, k)) return fail(c, FWI_E_INVAL, "source %d on a fixed (Dirichlet) face", s);
     nodes[s] = ((int64_t)k * c->geo.n[1] + j) * c->geo.px + i;
+    k0 = std::min(k0, k);
+    k1 = std::max(k1, k);
+    pml = pml || is_deep_pml(c, i, j, k);
     const double minv = 1.0 / mass_u(c, i, j, k);
     for (int d = 0; d < 3; d++) {
       if (!std::isfinite(dir[3 * s + d])) return fail(c, FWI_E_NONFINITE, "non-finite source direction");
@@ -1003,6 +1020,9 @@ fwi_status fwi_set_sources(fwi_ctx *c, int nshots, const int *node_ijk, const do
   CUDA_TRY(c, cudaMemcpy(c->d_wave, wave.data(), sizeof(float) * nw, cudaMemcpyHostToDevice));
   c->nshots = nshots;
   c->src_node = nodes;
+  c->src_k[0] = k0;
+  c->src_k[1] = k1;
+  c->src_pml = pml;
   c->src_dir.assign(dir, dir + 3 * (size_t)nshots);
   c->wavelet = wavelet;
   std::memcpy(c->wparams, wparams, sizeof c->wparams);
@@ -1015,12 +1035,17 @@ fwi_status fwi_set_receivers(fwi_ctx *c, int nrec, const int *node_ijk) {
   if (nrec < 1 || !node_ijk) return fail(c, FWI_E_INVAL, "bad receiver arguments");
   std::vector<int64_t> nodes(nrec);
   std::vector<float> vec(3 * (size_t)nrec);
+  int k0 = c->geo.n[2], k1 = -1;
+  bool pml = false;
   for (int r = 0; r < nrec; r++) {
     const int i = node_ijk[3 * r], j = node_ijk[3 * r + 1], k = node_ijk[3 * r + 2];
     if (i < 0 || j < 0 || k < 0 || i >= c->geo.n[0] || j >= c->geo.n[1] || k >= c->geo.n[2])
       return fail(c, FWI_E_INVAL, "receiver %d node (%d,%d,%d) outside the mesh", r, i, j, k);
     if (is_dirichlet(c, i, j, k)) return fail(c, FWI_E_INVAL, "receiver %d on a fixed (Dirichlet) face", r);
     nodes[r] = ((int64_t)k * c->geo.n[1] + j) * c->geo.px + i;
+    k0 = std::min(k0, k);
+    k1 = std::max(k1, k);
+    pml = pml || is_deep_pml(c, i, j, k);
     const float minv = (float)(1.0 / mass_u(c, i, j, k));
     vec[3 * r] = vec[3 * r + 1] = vec[3 * r + 2] = minv;
   }
@@ -1039,9 +1064,15 @@ fwi_status fwi_set_receivers(fwi_ctx *c, int nrec, const int *node_ijk) {
   TRY(dalloc(c, &c->d_rec_vec, 3 * (size_t)nrec));
   CUDA_TRY(c, cudaMemcpy(c->d_rec_node, nodes.data(), sizeof(int64_t) * nrec, cudaMemcpyHostToDevice));
   CUDA_TRY(c, cudaMemcpy(c->d_rec_vec, vec.data(), sizeof(float) * 3 * nrec, cudaMemcpyHostToDevice));
+  TRY(dalloc(c, &c->d_rec_of, (size_t)c->geo.stride));
+  fwi::launch_rec_map(c->d_rec_node, nrec, c->d_rec_of, c->geo.stride, c->stream);
+  CUDA_TRY(c, cudaGetLastError());
+  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   c->nrec = nrec;
   c->rec_node = nodes;
-  dfree(c->d_rec_of);  // rebuilt by the next persistent sweep
+  c->rec_k[0] = k0;
+  c->rec_k[1] = k1;
+  c->rec_pml = pml;
   return FWI_OK;
 }
 
@@ -1527,7 +1558,9 @@ fwi_status fwi_rhs(fwi_ctx *c, int adjoint, const float *state, float *rate, int
   a.out = out;
   a.stage = 0;
   a.nshot = 1;
-  TRY(stage(c, adjoint != 0, a));
+  fwi::Points none{};
+  none.k0 = 1;  // no plane has points
+  TRY(stage(c, adjoint != 0, a, none, false));
   if (!on_device)
     CUDA_TRY(c, cudaMemcpyAsync(rate, c->state[2], n * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));

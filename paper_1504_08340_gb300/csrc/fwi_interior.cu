@@ -287,9 +287,10 @@ __device__ __forceinline__ void copy_plane(float *dst, const CUtensorMap *tm, in
 // tm: the u fields of the stage input of the batch (see plane_map); the copies of a plane
 // are numbered from k0 - 2: copy q lands in ring slot q % kRing, and is that slot's
 // (q / kRing)-th phase
-template <int MODE>
+// PTS: this launch applies the points on its nodes
+template <int MODE, bool PTS>
 __global__ void __launch_bounds__(kTP *kTY, FWI_INT_MINB)
-    interior_kernel(const __grid_constant__ CUtensorMap tm, Geo g, StageArgs a0) {
+    interior_kernel(const __grid_constant__ CUtensorMap tm, Geo g, StageArgs a0, Points pts) {
   float *smem = s_ring;
   uint64_t *bar = reinterpret_cast<uint64_t *>(s_ring + kRing * kPS);
   const int kc = g.int_kc;                                   // planes per block
@@ -368,6 +369,12 @@ __global__ void __launch_bounds__(kTP *kTY, FWI_INT_MINB)
       node_accel_dispatch<kOdd>(t, sy, sz, sc, acc);
       finish_node<MODE>(g, a, IO, J, K, t, oo, acc);
     }
+    if constexpr (PTS)
+      if (has_points(pts, K)) {
+#pragma unroll 1
+        for (int h = 0; h < 2; h++)
+          if (h ? o_ok : e_ok) node_points(pts, a, shot, g.stride, rowbase + IE + h, 0, 3, g.oob);
+      }
     if (__syncthreads_or(!got)) {
       ok = false;
       break;
@@ -418,14 +425,15 @@ bool plane_map(const Geo &g, const StageArgs &a, CUtensorMap *tm) {
 }  // namespace
 
 cudaError_t prepare_interior() {
-  for (auto kernel : {interior_kernel<0>, interior_kernel<1>, interior_kernel<2>, interior_kernel<3>}) {
+  for (auto kernel : {interior_kernel<0, false>, interior_kernel<1, false>, interior_kernel<2, false>,
+                      interior_kernel<3, false>, interior_kernel<1, true>, interior_kernel<2, true>, interior_kernel<3, true>}) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
-int launch_interior(const Geo &g0, const StageArgs &a, cudaStream_t s) {
+int launch_interior(const Geo &g0, const StageArgs &a, const Points &q, cudaStream_t s) {
   Geo g = g0;
   if (g.box_hi[0] < g.box_lo[0] || g.box_hi[1] < g.box_lo[1] || g.box_hi[2] < g.box_lo[2]) return 0;
   const int nx = g.box_hi[0] - (g.box_lo[0] - 1) + 1;
@@ -437,11 +445,12 @@ int launch_interior(const Geo &g0, const StageArgs &a, cudaStream_t s) {
   CUtensorMap tm;
   std::memset(&tm, 0, sizeof(tm));
   if (!plane_map(g, a, &tm)) return -1;
-  const auto kernel = a.stage == 0   ? interior_kernel<0>
-                      : a.stage == 1 ? interior_kernel<1>
-                      : a.stage < 4  ? interior_kernel<2>
-                                     : interior_kernel<3>;
-  kernel<<<grd, dim3(kTP, kTY), kSmem, s>>>(tm, g, a);
+  const bool pts = q.fused && q.k0 <= g.box_hi[2];
+  const auto kernel = a.stage == 0   ? interior_kernel<0, false>
+                      : a.stage == 1 ? (pts ? interior_kernel<1, true> : interior_kernel<1, false>)
+                      : a.stage < 4  ? (pts ? interior_kernel<2, true> : interior_kernel<2, false>)
+                                     : (pts ? interior_kernel<3, true> : interior_kernel<3, false>);
+  kernel<<<grd, dim3(kTP, kTY), kSmem, s>>>(tm, g, a, q);
   return 1;
 }
 

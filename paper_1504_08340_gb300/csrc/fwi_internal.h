@@ -85,6 +85,28 @@ struct StageArgs {
   int64_t sstride, hstride;
 };
 
+// Point loads on the rate-level displacement of a stage's output and receiver samples of its
+// value level. fused: the thread that writes a node applies them (kernels of few blocks, where
+// a launch of their own would be a good part of the stage: 16x16x8, 4 % of a gradient; only
+// planes k0 .. k1 have any, none when k1 < k0, so the other planes pay one comparison), except
+// on launch_pml's nodes, where a point is rare and the check would cost registers. Else, and
+// there, points_kernel does, after the stage's kernels (in the kernels of a 96x96x48 mesh the
+// check's code and registers cost 3 % of the interior and 2 % of the shell kernel).
+//  load 1 (sources): + cdt table[i0] src_vec[3 b + c] at src_node[b] of shot b;
+//  load 2 (receiver residuals): + cdt e rec_vec[3 r + c] at receiver r, e = table[i0][r][c], or
+//    the mean with table[i1] when i1 >= 0 (shot b's table at + b tstride);
+//  traces: [nrec][3] of shot b at + b tstride, or null.
+struct Points {
+  bool fused;
+  int load, i0, i1, nrec;
+  int k0, k1;
+  const int64_t *src_node;
+  const float *src_vec, *rec_vec, *table;
+  const int *rec_of;  // node -> receiver, or -1
+  float *traces;
+  int64_t tstride;
+};
+
 // Planes per block of a kernel whose blocks march along z: the power of two up to `most` that
 // takes the fewest plane steps, ceil(blocks / slots) (k + start), for `tiles` (x, y) tiles of
 // all shots, `planes` planes and `slots` blocks resident on the GPU; `start` is the cost of
@@ -118,6 +140,30 @@ __host__ __device__ inline StageArgs shot_args(StageArgs a, int shot) {
   return a;
 }
 
+__device__ __forceinline__ bool has_points(const Points &q, int K) { return K >= q.k0 && K <= q.k1; }
+
+// a node of a plane with points, after this thread wrote its components c0 .. c1 - 1: adds the
+// point load and takes the sample. It reads the values back (by the thread that wrote them), so
+// that the rest of a kernel holds nothing for it.
+__device__ __forceinline__ void node_points(const Points &q, const StageArgs &a, int64_t b, int64_t S, int64_t node, int c0,
+                                            int c1, unsigned long long *oob) {
+  const int r = q.load == 2 || q.traces ? __ldg(q.rec_of + node) : -1;
+  const bool rec = r >= 0 && guard(oob, kSitePoint, r, q.nrec), src = q.load == 1 && node == __ldg(q.src_node + b);
+  if (!rec && !src) return;
+#pragma unroll 1
+  for (int c = c0; c < c1; c++) {
+    if (src) {
+      a.out[(18 + c) * S + node] += a.cdt * __ldg(q.table + q.i0) * __ldg(q.src_vec + 3 * b + c);
+    } else if (q.load == 2) {
+      const float *t = q.table + b * q.tstride + 3 * (int64_t)r + c;
+      float e = __ldg(t + (int64_t)q.i0 * q.nrec * 3);
+      if (q.i1 >= 0) e = 0.5f * (e + __ldg(t + (int64_t)q.i1 * q.nrec * 3));
+      a.out[(18 + c) * S + node] += a.cdt * e * __ldg(q.rec_vec + 3 * (int64_t)r + c);
+    }
+    if (q.traces && rec) q.traces[b * q.tstride + (int64_t)r * 3 + c] = a.out[(9 + c) * S + node];
+  }
+}
+
 // a node number of the state layout: inside the grid and not in a row's padding
 __device__ __forceinline__ bool node_ok(const Geo &g, int site, long long node) {
   return guard(g.oob, site, node, (long long)g.px * g.n[1] * g.n[2]) && guard(g.oob, site, node % g.px, g.n[0]);
@@ -132,10 +178,13 @@ __device__ __forceinline__ bool node_ok(const Geo &g, int site, long long node) 
 //  launch_pml:      nodes all of whose elements are PML, off the outer faces (fwi_pml.cu);
 //  launch_shell:    the interface shell (fwi_stage.cu);
 //  launch_pml_face: the PML nodes on the outer faces of the grid (fwi_pml.cu).
-int launch_interior(const Geo &g, const StageArgs &a, cudaStream_t s);
+// launch_points: points_kernel over the sources and receivers (only those on launch_pml's
+// nodes when q.fused), after the stage's kernels.
+int launch_interior(const Geo &g, const StageArgs &a, const Points &q, cudaStream_t s);
 int launch_pml(const Geo &g, const StageArgs &a, bool adjoint, cudaStream_t s);
-int launch_pml_face(const Geo &g, const StageArgs &a, bool adjoint, cudaStream_t s);
-int launch_shell(const Geo &g, const StageArgs &a, bool adjoint, cudaStream_t s);
+int launch_points(const Geo &g, const StageArgs &a, const Points &q, const int64_t *rec_node, cudaStream_t s);
+int launch_pml_face(const Geo &g, const StageArgs &a, const Points &q, bool adjoint, cudaStream_t s);
+int launch_shell(const Geo &g, const StageArgs &a, const Points &q, bool adjoint, cudaStream_t s);
 // raises the interior kernel's shared-memory limit on the current device
 cudaError_t prepare_interior();
 
@@ -154,13 +203,7 @@ struct PersistArgs {
   float dt;
   const int *nodes;           // every node of the grid, (k, j, i) order
   int nall;
-  const int64_t *src_node;    // shot b's source node and load vector (dir / M) at src_node[b], src_vec[3 b]
-  const float *src_vec;
-  const float *wave;          // wavelet samples every dt / 2
-  const int *rec_of;          // node -> receiver index, or -1
-  float *traces;              // shot b's traces at traces + b tstride, [n][nrec][3]
-  int64_t tstride;
-  int nrec;
+  Points pts;                 // the sources, and the receivers' samples of level 0 (load 1)
   float *hist;                // displacement history, level n at hist + n hstep (shot b at + b hstride), or null
   int64_t hstep, hstride;
   unsigned *bar;              // [2]: arrival count and generation, zero before the launch
@@ -170,34 +213,8 @@ struct PersistArgs {
 };
 cudaError_t launch_persistent_forward(const Geo &g, const PersistArgs &p, cudaStream_t s);
 
-// Point loads on level-2 displacement rows of buffer `buf`:
-// buf[9*2 + c][node[p]] += cdt * amp_p * vec[p][c], where
-//   mode 0 (sources): amp_p = wave[widx0] (or 0.5*(wave[widx0]+wave[widx1]))
-//   mode 1 (receiver residuals): amp_p = 1 and vec = minv * (resid[t0][p] (+ resid[t1][p])/2)
-struct PointArgs {
-  float *buf;
-  int64_t stride;
-  int npts;
-  const int64_t *node;
-  const float *vec;      // [npts][3]: dir * Minv (sources) or Minv replicated (receivers)
-  const float *table;    // sources: wavelet samples at t = j dt/2; receivers: residual [nt][npts][3]
-  int i0, i1;            // sample indices (i1 < 0: single sample)
-  float cdt;
-  int mode;
-  // batch: shot b adds into buf + b * sstride; sources: its point is node[b], vec[b];
-  // receivers: its residuals start at table + b * tstride
-  int nshot;
-  int64_t sstride, tstride;
-  int64_t nnode_pad;          // valid node numbers: [0, nnode_pad) (bounds-checked build)
-  unsigned long long *oob;    // error word of the bounds-checked build (else null)
-};
-void launch_point(const PointArgs &p, cudaStream_t s);
-
-// traces[b][r][c] = buf[b * sstride + (9 + c) * stride + node[r]] for the nshot shots of a
-// batch (trace of shot b at traces + b * tstride)
-void launch_sample(const float *buf, int64_t stride, int nrec, const int64_t *node, float *traces,
-                   cudaStream_t s, int nshot = 1, int64_t sstride = 0, int64_t tstride = 0,
-                   unsigned long long *oob = nullptr);
+// rec_of[node[r]] = r for the nrec receivers, -1 at the other `stride` entries
+void launch_rec_map(const int64_t *node, int nrec, int *rec_of, int64_t stride, cudaStream_t s);
 
 // Gradient integrand of (C.1f)/(C.1g) at one time level, accumulated in FP64:
 // gl[i] -= wdt * sum_e W detJ (div w)(div u), gm[i] -= wdt * sum_e W detJ 2 eps(w):eps(u),

@@ -1,6 +1,6 @@
 // fwi_kernels.cu -- CUDA kernels of the gradient path other than the RK4 stage
-// (sm_103a): point loads, receiver sampling, the FP64 gradient integrals
-// (C.1f)/(C.1g) of arXiv:1504.08340 and the FP64 misfit reduction.
+// (sm_103a): the FP64 gradient integrals (C.1f)/(C.1g) of arXiv:1504.08340 and the
+// FP64 misfit reduction.
 //
 // Element-wise derivatives at a node use the one-sided / centred 3-point stencils
 // of the 27-node LGL element along each axis:
@@ -17,37 +17,29 @@ namespace {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-__global__ void point_kernel(PointArgs p) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= p.npts * p.nshot) return;
-  const int b = t / p.npts, i = t - b * p.npts;  // shot of the batch, point
-  const int k = p.mode == 0 ? b : i;             // sources: one point per shot
-  const int64_t n = p.node[k];
-  if (!guard(p.oob, kSitePoint, n, p.nnode_pad)) return;
-  float *buf = p.buf + (int64_t)b * p.sstride;
-  const float *table = p.mode == 0 ? p.table : p.table + (int64_t)b * p.tstride;
-  for (int c = 0; c < 3; c++) {
-    float amp;
-    if (p.mode == 0) {
-      amp = table[p.i0];
-      if (p.i1 >= 0) amp = 0.5f * (amp + table[p.i1]);
-    } else {
-      amp = table[((int64_t)p.i0 * p.npts + i) * 3 + c];
-      if (p.i1 >= 0) amp = 0.5f * (amp + table[((int64_t)p.i1 * p.npts + i) * 3 + c]);
-    }
-    buf[(int64_t)(18 + c) * p.stride + n] += p.cdt * amp * p.vec[k * 3 + c];
-  }
+__global__ void rec_map_kernel(const int64_t *node, int nrec, int *rec_of) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r < nrec) rec_of[node[r]] = r;
 }
 
-__global__ void sample_kernel(const float *buf, int64_t stride, int nrec, const int64_t *node, float *tr,
-                              int nshot, int64_t sstride, int64_t tstride, unsigned long long *oob) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nrec * 3 * nshot) return;
-  const int b = t / (nrec * 3), i = t - b * nrec * 3;
-  const int r = i / 3, c = i % 3;
-  const int64_t n = node[r];
-  if (!guard(oob, kSiteSample, n, stride)) return;
-  tr[(int64_t)b * tstride + i] = buf[(int64_t)b * sstride + (int64_t)(9 + c) * stride + n];
+// the sources (load 1, one per shot) and receivers of a stage (see Points): thread per shot and
+// receiver (thread nrec of a shot: its source)
+__global__ void points_kernel(Geo g, StageArgs a0, Points q, const int64_t *__restrict__ rec_node) {
+  const int per = q.nrec + 1;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, b = t / per, i = t - b * per;
+  if (b >= a0.nshot || (i == q.nrec && q.load != 1) || (i < q.nrec && q.load == 1 && !q.traces)) return;
+  const int64_t node = i < q.nrec ? rec_node[i] : q.src_node[b];
+  if (!guard(g.oob, kSitePoint, node, g.stride)) return;
+  // a source that is sampled too is the receiver's thread's
+  if (i == q.nrec && q.traces && q.rec_of[node] >= 0) return;
+  if (q.fused) {
+    const int I = (int)(node % g.px), r = (int)(node / g.px), J = r % g.n[1], K = r / g.n[1];
+    const bool face = I == 0 || I == g.n[0] - 1 || J == 0 || J == g.n[1] - 1 || K == 0 || K == g.n[2] - 1;
+    const bool box = I >= 2 * g.lo[0] && I <= 2 * g.hi[0] && J >= 2 * g.lo[1] && J <= 2 * g.hi[1] && K >= 2 * g.lo[2] &&
+                     K <= 2 * g.hi[2];
+    if (face || box) return;  // its stage kernel applied it
+  }
+  node_points(q, shot_args(a0, b), b, g.stride, node, 0, 3, g.oob);
 }
 
 // (C.1f)/(C.1g) at one time level, in FP64: for every interior node, the sum over the
@@ -230,16 +222,14 @@ inline unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + thre
 
 }  // namespace
 
-void launch_point(const PointArgs &p, cudaStream_t s) {
-  if (p.npts <= 0 || p.nshot <= 0) return;
-  point_kernel<<<blocks_for((int64_t)p.npts * p.nshot, 128), 128, 0, s>>>(p);
+int launch_points(const Geo &g, const StageArgs &a, const Points &q, const int64_t *rec_node, cudaStream_t s) {
+  points_kernel<<<blocks_for((int64_t)a.nshot * (q.nrec + 1), 128), 128, 0, s>>>(g, a, q, rec_node);
+  return 1;
 }
 
-void launch_sample(const float *buf, int64_t stride, int nrec, const int64_t *node, float *traces,
-                   cudaStream_t s, int nshot, int64_t sstride, int64_t tstride, unsigned long long *oob) {
-  if (nrec <= 0 || nshot <= 0) return;
-  sample_kernel<<<blocks_for((int64_t)nrec * 3 * nshot, 256), 256, 0, s>>>(buf, stride, nrec, node, traces, nshot,
-                                                                           sstride, tstride, oob);
+void launch_rec_map(const int64_t *node, int nrec, int *rec_of, int64_t stride, cudaStream_t s) {
+  cudaMemsetAsync(rec_of, 0xff, sizeof(int) * (size_t)stride, s);
+  rec_map_kernel<<<blocks_for(nrec, 256), 256, 0, s>>>(node, nrec, rec_of);
 }
 
 void launch_gradient(const Geo &g, const float *w_state, const float *u_hist, double wdt, double *gl,

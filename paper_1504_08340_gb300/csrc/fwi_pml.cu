@@ -452,7 +452,7 @@ __device__ __forceinline__ void face_axis(const Geo &g, const StageArgs &a, cons
 
 template <bool ADJ>
 __device__ __forceinline__ void face_write(const Geo &g, const StageArgs &a, const FaceCtx &n, int I, int J, int K,
-                                           const FaceShared &sh, int lane, int w) {
+                                           const FaceShared &sh, int lane, int w, const Points &q, int shot) {
   const int S = (int)g.stride;
   const float *__restrict__ Y = a.Y;
   // ---- displacement component w
@@ -466,6 +466,7 @@ __device__ __forceinline__ void face_write(const Geo &g, const StageArgs &a, con
       __stcs(a.out + i0, stage_value(a, i0, u0, u1));
       __stcs(a.out + i1, stage_value(a, i1, u1, u2));
       __stcs(a.out + i2, stage_value(a, i2, u2, acc));
+      if (q.fused && has_points(q, K)) node_points(q, a, shot, S, n.node, c, c + 1, g.oob);
     } else if (a.stage == 0) {
       __stcs(a.out + i0, 0.f);
       __stcs(a.out + i1, 0.f);
@@ -580,7 +581,7 @@ __global__ void __launch_bounds__(kBX *kBY, MODE == 3 ? FWI_PML_STAGE4_MINB : (P
 }
 
 template <bool ADJ>
-__global__ void __launch_bounds__(3 * kFaceNodes, FWI_FACE_MINB) pml_face_kernel(Geo g, StageArgs a0) {
+__global__ void __launch_bounds__(3 * kFaceNodes, FWI_FACE_MINB) pml_face_kernel(Geo g, StageArgs a0, Points q) {
   __shared__ FaceShared sh;
   const int nbs = (g.nface + kFaceNodes - 1) / kFaceNodes;  // blocks per shot
   const StageArgs a = shot_args(a0, blockIdx.x / nbs);
@@ -601,7 +602,7 @@ __global__ void __launch_bounds__(3 * kFaceNodes, FWI_FACE_MINB) pml_face_kernel
     else face_axis<ADJ, 2>(g, a, n, I, J, K, sh, lane);
   }
   __syncthreads();
-  if (live) face_write<ADJ>(g, a, n, I, J, K, sh, lane, w);
+  if (live) face_write<ADJ>(g, a, n, I, J, K, sh, lane, w, q, blockIdx.x / nbs);
 }
 
 }  // namespace
@@ -653,34 +654,30 @@ int launch_pml(const Geo &g, const StageArgs &a, bool adjoint, cudaStream_t s) {
   if (tasks == 0) return 0;
   const dim3 grd((tasks + kBY - 1) / kBY * a.nshot), blk(kBX, kBY);
   const int mode = a.stage == 0 ? 0 : (a.stage == 1 ? 1 : (a.stage < 4 ? 2 : 3));
-  auto go = [&](auto part, cudaStream_t st) {
-    constexpr int P = decltype(part)::value;
-    if (adjoint) {
-      if (mode == 0) pml_kernel<true, 0, P><<<grd, blk, 0, st>>>(g, a, r);
-      else if (mode == 1) pml_kernel<true, 1, P><<<grd, blk, 0, st>>>(g, a, r);
-      else if (mode == 2) pml_kernel<true, 2, P><<<grd, blk, 0, st>>>(g, a, r);
-      else pml_kernel<true, 3, P><<<grd, blk, 0, st>>>(g, a, r);
-    } else {
-      if (mode == 0) pml_kernel<false, 0, P><<<grd, blk, 0, st>>>(g, a, r);
-      else if (mode == 1) pml_kernel<false, 1, P><<<grd, blk, 0, st>>>(g, a, r);
-      else if (mode == 2) pml_kernel<false, 2, P><<<grd, blk, 0, st>>>(g, a, r);
-      else pml_kernel<false, 3, P><<<grd, blk, 0, st>>>(g, a, r);
-    }
-  };
-  // one launch: per pair the stress rows, then the displacement rows (disjoint outputs, the
+  // PART 3: one launch, per pair the stress rows, then the displacement rows (disjoint outputs, the
   // same inputs), each part with the registers of its own update
-  go(std::integral_constant<int, 3>{}, s);
+  if (adjoint) {
+    if (mode == 0) pml_kernel<true, 0, 3><<<grd, blk, 0, s>>>(g, a, r);
+    else if (mode == 1) pml_kernel<true, 1, 3><<<grd, blk, 0, s>>>(g, a, r);
+    else if (mode == 2) pml_kernel<true, 2, 3><<<grd, blk, 0, s>>>(g, a, r);
+    else pml_kernel<true, 3, 3><<<grd, blk, 0, s>>>(g, a, r);
+  } else {
+    if (mode == 0) pml_kernel<false, 0, 3><<<grd, blk, 0, s>>>(g, a, r);
+    else if (mode == 1) pml_kernel<false, 1, 3><<<grd, blk, 0, s>>>(g, a, r);
+    else if (mode == 2) pml_kernel<false, 2, 3><<<grd, blk, 0, s>>>(g, a, r);
+    else pml_kernel<false, 3, 3><<<grd, blk, 0, s>>>(g, a, r);
+  }
   return 1;
 }
 
-int launch_pml_face(const Geo &g, const StageArgs &a, bool adjoint, cudaStream_t s) {
+int launch_pml_face(const Geo &g, const StageArgs &a, const Points &q, bool adjoint, cudaStream_t s) {
   if (g.nface <= 0) return 0;
   const int nb = (g.nface + kFaceNodes - 1) / kFaceNodes * a.nshot;
   const dim3 blk(kFaceNodes, 3);
   if (adjoint)
-    pml_face_kernel<true><<<nb, blk, 0, s>>>(g, a);
+    pml_face_kernel<true><<<nb, blk, 0, s>>>(g, a, q);
   else
-    pml_face_kernel<false><<<nb, blk, 0, s>>>(g, a);
+    pml_face_kernel<false><<<nb, blk, 0, s>>>(g, a, q);
   return 1;
 }
 

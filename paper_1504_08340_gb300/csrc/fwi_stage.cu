@@ -412,8 +412,9 @@ __device__ __forceinline__ void shell_stress(const Geo &g, const StageArgs &a, c
 }
 
 // displacement component c of the node: its three levels
-__device__ __forceinline__ void shell_disp(const Geo &g, const StageArgs &a, const NodeCtx &n, const ShellShared &sh,
-                                           int lane, int c) {
+template <bool PTS>
+__device__ __forceinline__ void shell_disp(const Geo &g, const StageArgs &a, const Points &q, int shot, const NodeCtx &n,
+                                           const ShellShared &sh, int lane, int c) {
   const int64_t S = g.stride;
   const float *__restrict__ Y = a.Y;
   const int64_t i0 = (int64_t)c * S + n.node, i1 = (int64_t)(9 + c) * S + n.node, i2 = (int64_t)(18 + c) * S + n.node;
@@ -433,14 +434,17 @@ __device__ __forceinline__ void shell_disp(const Geo &g, const StageArgs &a, con
   const float v1 = stage_value(a, i1, u1, u2);
   __stcs(a.out + i1, v1);
   __stcs(a.out + i2, stage_value(a, i2, u2, acc));
+  if constexpr (PTS)
+    if (has_points(q, n.c3[2])) node_points(q, a, shot, S, n.node, c, c + 1, g.oob);
   if (a.hist) write_hist(g, a, n.c3[0], n.c3[1], n.c3[2], c, v1);
 }
 
-template <bool ADJ, int W>
-__global__ void __launch_bounds__(W *kShellNodes, 24 / W) shell_kernel(Geo g, StageArgs a0) {
+template <bool ADJ, int W, bool PTS>
+__global__ void __launch_bounds__(W *kShellNodes, 24 / W) shell_kernel(Geo g, StageArgs a0, Points q) {
   __shared__ ShellShared sh;
   const int nbs = (g.nshell + kShellNodes - 1) / kShellNodes;  // blocks per shot
-  const StageArgs a = shot_args(a0, blockIdx.x / nbs);
+  const int shot = blockIdx.x / nbs;
+  const StageArgs a = shot_args(a0, shot);
   const int lane = threadIdx.x, w = threadIdx.y;
   const int i = (blockIdx.x % nbs) * kShellNodes + lane;
   const bool live = i < g.nshell && node_ok(g, kSiteShell, g.shell[i]);
@@ -453,7 +457,7 @@ __global__ void __launch_bounds__(W *kShellNodes, 24 / W) shell_kernel(Geo g, St
   }
   __syncthreads();
   if (live) {
-    if (w < 3) shell_disp(g, a, n, sh, lane, w);
+    if (w < 3) shell_disp<PTS>(g, a, q, shot, n, sh, lane, w);
     for (int c = w; c < 6; c += W) shell_stress<ADJ>(g, a, n, sh, lane, c);
   }
 }
@@ -493,37 +497,6 @@ __device__ bool grid_barrier(const PersistArgs &p, unsigned expected) {
   return ok_s != 0;
 }
 
-// displacement component c of a node for the persistent sweep: shell_disp, plus the
-// source load of the shot (forward point load, as point_kernel adds it) and the receiver
-// sample after the last stage
-__device__ __forceinline__ void persist_disp(const Geo &g, const StageArgs &a, const NodeCtx &n,
-                                             const ShellShared &sh, int lane, int c, const PersistArgs &p, int b,
-                                             int step, int stage) {
-  const int64_t S = g.stride;
-  const float *__restrict__ Y = a.Y;
-  const int64_t i0 = (int64_t)c * S + n.node, i1 = (int64_t)(9 + c) * S + n.node, i2 = (int64_t)(18 + c) * S + n.node;
-  if (n.dir) return;
-  const float fsum = shell_force(g, sh, c, lane);
-  const float inv_m = n.inv_a / (g.rho * (float)n.nel);
-  const float u0 = __ldg(Y + i0), u1 = __ldg(Y + i1), u2 = __ldg(Y + i2);
-  const float acc = -fsum * inv_m - (n.cb * u2 + n.cc * u1 + n.cd * u0) * n.inv_a;
-  if (n.pml) __stcs(a.out + i0, stage_value(a, i0, u0, u1));
-  const float v1 = stage_value(a, i1, u1, u2);
-  __stcs(a.out + i1, v1);
-  float v2 = stage_value(a, i2, u2, acc);
-  if (n.node == p.src_node[b]) {
-    // stage times t_n, t_n + dt/2, t_n + dt/2, t_n + dt: samples 2n, 2n+1, 2n+1, 2n+2
-    const float amp = p.wave[stage == 0 ? 2 * step : (stage == 3 ? 2 * step + 2 : 2 * step + 1)];
-    v2 += a.cdt * amp * p.src_vec[3 * b + c];
-  }
-  __stcs(a.out + i2, v2);
-  if (a.hist) write_hist(g, a, n.c3[0], n.c3[1], n.c3[2], c, v1);
-  if (stage == 3) {
-    const int r = p.rec_of[n.node];
-    if (r >= 0 && guard(g.oob, kSitePersist, r, p.nrec)) p.traces[(int64_t)b * p.tstride + ((int64_t)(step + 1) * p.nrec + r) * 3 + c] = v1;
-  }
-}
-
 // six warps a block: the sweep is meant for meshes of about one wave of blocks, where a stage
 // takes one node chunk's chain of loads (8x8x4 elements, a 100-step sweep: 7.07 ms; with three
 // warps and 4 blocks an SM 8.09 ms, with six warps and 2 blocks 8.71 ms)
@@ -548,6 +521,10 @@ __global__ void __launch_bounds__(kPersistWarps *kShellNodes, 3) persistent_forw
       a0.nshot = p.nshot;
       a0.sstride = p.sstride;
       a0.hstride = p.hstride;
+      // stage times t_n, t_n + dt/2, t_n + dt/2, t_n + dt: wavelet samples 2n, 2n+1, 2n+1, 2n+2
+      Points q = p.pts;
+      q.i0 = s == 0 ? 2 * step : (s == 3 ? 2 * step + 2 : 2 * step + 1);
+      q.traces = s == 3 ? p.pts.traces + (int64_t)(step + 1) * q.nrec * 3 : nullptr;
       for (int ch = blockIdx.x; ch < nch * p.nshot; ch += gridDim.x) {
         const int b = ch / nch;
         const StageArgs a = shot_args(a0, b);
@@ -562,7 +539,7 @@ __global__ void __launch_bounds__(kPersistWarps *kShellNodes, 3) persistent_forw
         }
         __syncthreads();
         if (live) {
-          if (w < 3) persist_disp(g, a, n, sh, lane, w, p, b, step, s);
+          if (w < 3) shell_disp<true>(g, a, q, b, n, sh, lane, w);
           for (int c = w; c < 6; c += kPersistWarps) shell_stress<false>(g, a, n, sh, lane, c);
         }
         __syncthreads();
@@ -590,15 +567,16 @@ cudaError_t launch_persistent_forward(const Geo &g, const PersistArgs &p, cudaSt
                                      0, s);
 }
 
-int launch_shell(const Geo &g, const StageArgs &a, bool adjoint, cudaStream_t s) {
+int launch_shell(const Geo &g, const StageArgs &a, const Points &q, bool adjoint, cudaStream_t s) {
   int n = 0;
   if (g.nshell > 0) {
     n = 1;
     const int nb = (g.nshell + kShellNodes - 1) / kShellNodes * a.nshot;
     const bool six = nb <= 2 * kSms;
-    const auto kernel = adjoint ? (six ? shell_kernel<true, 6> : shell_kernel<true, 3>)
-                                : (six ? shell_kernel<false, 6> : shell_kernel<false, 3>);
-    kernel<<<nb, dim3(kShellNodes, six ? 6 : 3), 0, s>>>(g, a);
+    const auto kernel = adjoint   ? (six ? shell_kernel<true, 6, false> : shell_kernel<true, 3, false>)
+                        : q.fused ? (six ? shell_kernel<false, 6, true> : shell_kernel<false, 3, true>)
+                                  : (six ? shell_kernel<false, 6, false> : shell_kernel<false, 3, false>);
+    kernel<<<nb, dim3(kShellNodes, six ? 6 : 3), 0, s>>>(g, a, q);
   }
   return n;
 }
