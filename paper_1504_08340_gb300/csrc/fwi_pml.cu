@@ -57,18 +57,20 @@ __device__ __forceinline__ float ddiv(float g_m2, float g_m1, float g0, float g_
 __host__ __device__ constexpr int sym(int i, int j) { return i == j ? i : (i + j == 1 ? 5 : (i + j == 2 ? 4 : 3)); }
 
 // PML boxes and their warp tasks. The node pairs of a box row are cut into nseg
-// x segments of at most `per` <= 32 pairs. A warp task is one segment of R rows of
-// one plane with equal y parity (J0, J0 + 2, ..., J0 + 2(R-1)): R = 32 / per for
-// narrow boxes, else 1. The side kinds along y and z are then uniform across the
-// warp. Tasks run segment by segment, so the warps resident at one time cover one
-// x segment of many rows and planes, and the rows that their y and z stencils
-// share stay in L2.
+// x segments of at most `per` <= 32 pairs. The rows of one plane with equal y parity
+// (J0, J0 + 2, ...) form a class; a warp task takes 32 consecutive places of the class's
+// (row, pair) list of one segment, a row holding `slot` places: the segment's pairs when
+// rows are packed (a task may then end in the middle of a row), or 32 when they are not.
+// The side kinds along y and z are uniform across the warp either way. Tasks run segment
+// by segment, so the warps resident at one time cover one x segment of many rows and
+// planes, and the rows that their y and z stencils share stay in L2.
 struct Region {
   int nbox;
   int lo[6][3], hi[6][3];  // inclusive node boxes
-  int P[6], R[6];          // node pairs per row, rows per warp task
+  int P[6];                // node pairs per row
   int nseg[6], per[6];     // x segments per row, pairs per segment (the last may have fewer)
-  int jfirst[6][2], nj[6][2], groups[6][2];  // per y-parity class: first J, row count, warp groups per plane
+  bool packed[6];
+  int jfirst[6][2], nj[6][2], groups[6][2];  // per y-parity class: first J, row count, warp tasks per plane and segment
   int tasks_before[7];     // prefix sums of warp tasks per box
 };
 
@@ -515,6 +517,7 @@ __device__ __forceinline__ void face_write(const Geo &g, const StageArgs &a, con
 #define FWI_FACE_MINB 10
 #endif
 constexpr int kBX = 32, kBY = FWI_PML_BY;
+constexpr int kPackBelow = 28;  // pairs of an x segment below which its rows are packed (see Region)
 
 // grid.x: blocks of kBY warp tasks (see Region); tasks of a box run plane by plane.
 // The boxes exclude the outer faces of the grid, so every node takes the bulk path.
@@ -546,17 +549,16 @@ __global__ void __launch_bounds__(kBX *kBY, MODE == 3 ? FWI_PML_STAGE4_MINB : (P
   const int pb = (task - r.tasks_before[b]) / per_seg * r.per[b];  // first pair of the segment
   const int K = r.lo[b][2] + t / G;
   const int qa = t % G;
-  const int P = min(r.per[b], r.P[b] - pb), R = r.R[b];  // pairs of this segment
+  const int P = min(r.per[b], r.P[b] - pb);  // pairs of this segment
   const int x0 = r.lo[b][0] & ~1;  // pairs start at even x
   const int kz = side_kind(K, g.n[2]);
   const int cls = qa < r.groups[b][0] ? 0 : 1;
   const int q = cls ? qa - r.groups[b][0] : qa;
-  const int rr = R > 1 ? threadIdx.x / P : 0;  // row of the group handled by this lane
-  const int jrow = q * R + rr;
-  if (rr >= R || jrow >= r.nj[b][cls]) return;
+  const int slot = r.packed[b] ? P : 32, place = q * 32 + threadIdx.x;
+  const int jrow = place / slot, p = place - jrow * slot;  // row of the class, pair of the segment
+  if (jrow >= r.nj[b][cls]) return;
   const int J = r.jfirst[b][cls] + 2 * jrow;
   const int ky = side_kind(r.jfirst[b][cls], g.n[1]);
-  const int p = R > 1 ? threadIdx.x % P : threadIdx.x;  // pair of the segment (P <= 32)
   if (p < P) {
     const int I0 = x0 + 2 * (pb + p);
     // reach of the pair's stencils: the x window I0-2 .. I0+3 of its row, +-1 (odd) or
@@ -633,13 +635,16 @@ static Region pml_region(const Geo &g) {
     r.P[b] = (r.hi[b][0] - (r.lo[b][0] & ~1)) / 2 + 1;
     r.nseg[b] = (r.P[b] + g.pml_seg - 1) / g.pml_seg;
     r.per[b] = (r.P[b] + r.nseg[b] - 1) / r.nseg[b];
-    r.R[b] = r.per[b] > 16 ? 1 : 32 / r.per[b];  // rows per warp task: fill the 32 lanes
+    // packed rows keep every lane busy, but a warp's row loads then break at row ends: worth it
+    // below kPackBelow of 32 lanes (18 of 32 lanes, 16x16x8 elements: a gradient in 36.7 ms
+    // unpacked, 30.6 ms packed; 29 of 32, 96x96x48, four shots: 276.0 against 279.5 ms)
+    r.packed[b] = r.per[b] < kPackBelow;
     int per_plane = 0;
     for (int c = 0; c < 2; c++) {
       const int jf = r.lo[b][1] + ((r.lo[b][1] & 1) != c ? 1 : 0);  // first J of parity c
       r.jfirst[b][c] = jf;
       r.nj[b][c] = jf > r.hi[b][1] ? 0 : (r.hi[b][1] - jf) / 2 + 1;
-      r.groups[b][c] = (r.nj[b][c] + r.R[b] - 1) / r.R[b];
+      r.groups[b][c] = (r.nj[b][c] * (r.packed[b] ? r.per[b] : 32) + 31) / 32;
       per_plane += r.groups[b][c];
     }
     r.tasks_before[b + 1] = r.tasks_before[b] + r.nseg[b] * per_plane * (r.hi[b][2] - r.lo[b][2] + 1);
