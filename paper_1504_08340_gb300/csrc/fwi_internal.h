@@ -64,7 +64,7 @@ struct Geo {
   int copy_extra;
   // launch shapes (fwi_tune_tiles; they change no node's arithmetic)
   int int_kc;             // most planes per block of interior_kernel (see chunk_planes)
-  int pml_seg;            // node pairs per x segment of a pml_kernel warp task (<= 32)
+  int pml_seg;            // an x segment of pml_kernel is up to 4 pml_seg node pairs wide (see Region there)
 };
 
 // One RK4 stage over every node (see fwi_kernels.cu).

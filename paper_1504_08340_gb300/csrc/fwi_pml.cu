@@ -57,13 +57,17 @@ __device__ __forceinline__ float ddiv(float g_m2, float g_m1, float g0, float g_
 __host__ __device__ constexpr int sym(int i, int j) { return i == j ? i : (i + j == 1 ? 5 : (i + j == 2 ? 4 : 3)); }
 
 // PML boxes and their warp tasks. The node pairs of a box row are cut into nseg
-// x segments of at most `per` <= 32 pairs. The rows of one plane with equal y parity
+// x segments of at most `per` <= kSegWarps pml_seg pairs. The rows of one plane with equal y parity
 // (J0, J0 + 2, ...) form a class; a warp task takes 32 consecutive places of the class's
 // (row, pair) list of one segment, a row holding `slot` places: the segment's pairs when
 // rows are packed (a task may then end in the middle of a row), or 32 when they are not.
 // The side kinds along y and z are uniform across the warp either way. Tasks run segment
 // by segment, so the warps resident at one time cover one x segment of many rows and
-// planes, and the rows that their y and z stencils share stay in L2.
+// planes, and the rows that their y and z stencils share stay in L2. A segment's ends cost
+// each of its rows partial sectors in every field, read and written again by the next
+// segment's tasks much later, so a segment is as wide as four warps: 96x96x48 elements, four
+// shots, a gradient in 275.9 ms with segments of 29 pairs (one warp), 271.3 with 58, 265.1 with
+// 116 (whole rows).
 struct Region {
   int nbox;
   int lo[6][3], hi[6][3];  // inclusive node boxes
@@ -90,7 +94,9 @@ __device__ __forceinline__ float stage_value(const StageArgs &a, int idx, float 
 // node, .y: the odd node). x-window of a field: values at I0-2 .. I0+3; the even
 // node's x kind is LR, the odd node's C.
 __device__ __forceinline__ float2 ld2(const float *p) { return __ldg(reinterpret_cast<const float2 *>(p)); }
-__device__ __forceinline__ float2 ldcs2(const float *p) { return __ldcs(reinterpret_cast<const float2 *>(p)); }
+// step-start values, read once: L2 only, normal eviction (a warp's first and last sectors are its
+// neighbours' too, and an evict-first read let them go: 96x96x48, four shots: 264.7 against 263.5 ms a gradient)
+__device__ __forceinline__ float2 ldcg2(const float *p) { return __ldcg(reinterpret_cast<const float2 *>(p)); }
 __device__ __forceinline__ void st2(float *p, float2 v, bool even_ok) {
   if (even_ok)
     __stcs(reinterpret_cast<float2 *>(p), v);
@@ -180,9 +186,9 @@ template <int MODE>
 __device__ __forceinline__ float2 stage2(const StageArgs &a, int idx, float2 y, float2 r) {
   if constexpr (MODE == 0) return r;
   if constexpr (MODE == 1) return pfma(bc(a.cdt), r, y);
-  const float2 x = ldcs2(a.X + idx);
+  const float2 x = ldcg2(a.X + idx);
   if constexpr (MODE == 2) return pfma(bc(a.cdt), r, x);
-  const float2 b = ldcs2(a.Y2 + idx), c = ldcs2(a.Y3 + idx);
+  const float2 b = ldcg2(a.Y2 + idx), c = ldcg2(a.Y3 + idx);
   return pfma(bc(1.f / 3.f), padd(pfma(bc(2.f), c, psub(b, x)), y), pmul(bc(a.cdt), r));
 }
 
@@ -505,7 +511,7 @@ __device__ __forceinline__ void face_write(const Geo &g, const StageArgs &a, con
 #define FWI_PML_STAGE4_MINB 7  // stage 4 reads three more step-start rows: 72 registers, no spills
 #endif
 #ifndef FWI_PML_SPLIT_MINB
-#define FWI_PML_SPLIT_MINB 8
+#define FWI_PML_SPLIT_MINB 9  // 56 registers, 40 bytes of spills: 64x64x32 gradient 71.1 ms, at 8 blocks 73.8, at 10 76.4
 #endif
 #ifndef FWI_PML_BY
 #define FWI_PML_BY 4
@@ -517,6 +523,7 @@ __device__ __forceinline__ void face_write(const Geo &g, const StageArgs &a, con
 #define FWI_FACE_MINB 10
 #endif
 constexpr int kBX = 32, kBY = FWI_PML_BY;
+constexpr int kSegWarps = 4;    // warps whose pairs an x segment is wide
 constexpr int kPackBelow = 28;  // pairs of an x segment below which its rows are packed (see Region)
 
 // grid.x: blocks of kBY warp tasks (see Region); tasks of a box run plane by plane.
@@ -633,12 +640,12 @@ static Region pml_region(const Geo &g) {
   r.tasks_before[0] = 0;
   for (int b = 0; b < r.nbox; b++) {
     r.P[b] = (r.hi[b][0] - (r.lo[b][0] & ~1)) / 2 + 1;
-    r.nseg[b] = (r.P[b] + g.pml_seg - 1) / g.pml_seg;
+    r.nseg[b] = (r.P[b] + kSegWarps * g.pml_seg - 1) / (kSegWarps * g.pml_seg);
     r.per[b] = (r.P[b] + r.nseg[b] - 1) / r.nseg[b];
     // packed rows keep every lane busy, but a warp's row loads then break at row ends: worth it
     // below kPackBelow of 32 lanes (18 of 32 lanes, 16x16x8 elements: a gradient in 36.7 ms
     // unpacked, 30.6 ms packed; 29 of 32, 96x96x48, four shots: 276.0 against 279.5 ms)
-    r.packed[b] = r.per[b] < kPackBelow;
+    r.packed[b] = r.per[b] < kPackBelow || r.per[b] > 32;
     int per_plane = 0;
     for (int c = 0; c < 2; c++) {
       const int jf = r.lo[b][1] + ((r.lo[b][1] & 1) != c ? 1 : 0);  // first J of parity c
