@@ -48,6 +48,7 @@ struct fwi_ctx {
   std::vector<int64_t> src_node;
   int src_k[2] = {1, 0}, rec_k[2] = {1, 0};  // planes (first, last) that hold sources, receivers
   bool src_pml = false, rec_pml = false;     // some of them on a node of pml_kernel
+  int64_t rec0 = 0, rec_n = 0;               // nodes d_rec_of covers
   std::vector<double> src_dir;
   int wavelet = 0;
   double wparams[3] = {0, 0, 0};
@@ -104,7 +105,7 @@ struct fwi_ctx {
   bool persistent = false;
   double wait_ms = 1000.0;
   int bar_extra = 0;
-  int *d_all = nullptr, *d_rec_of = nullptr;  // every node; node -> receiver index (or -1)
+  int *d_all = nullptr, *d_rec_of = nullptr;  // every node; node -> receiver index, or -1 (see Points)
   unsigned *d_bar = nullptr;
   int *d_status = nullptr;                    // FWI_E_TIMEOUT when a bounded device wait gave up
 
@@ -418,6 +419,8 @@ fwi_status rk4_step(fwi_ctx *c, bool adj, int n, int shot0, int nb, float *hist_
     fwi::Points q{};
     q.nrec = c->nrec;
     q.rec_of = c->d_rec_of;
+    q.rec0 = c->rec0;
+    q.rec_n = c->rec_n;
     q.tstride = (int64_t)trace_floats(c);
     q.i1 = -1;
     q.fused = (int64_t)nb * c->geo.nnode <= kFusedNodes;
@@ -549,6 +552,8 @@ fwi_status forward_sweep_body(fwi_ctx *c, int shot0, int nb, float *hist, int64_
     p.pts.i1 = -1;
     p.pts.nrec = c->nrec;
     p.pts.rec_of = c->d_rec_of;
+    p.pts.rec0 = c->rec0;
+    p.pts.rec_n = c->rec_n;
     p.pts.tstride = tf;
     p.pts.traces = c->d_traces;
     p.pts.k0 = std::min(p.pts.k0, c->rec_k[0]);
@@ -1055,19 +1060,23 @@ fwi_status fwi_set_receivers(fwi_ctx *c, int nrec, const int *node_ijk) {
     for (int r = 1; r < nrec; r++)
       if (sorted[r] == sorted[r - 1]) return fail(c, FWI_E_INVAL, "receivers must be distinct nodes");
   }
+  c->nrec = 0;  // until the new ones are in place
   dfree(c->d_rec_node);
   dfree(c->d_rec_vec);
+  dfree(c->d_rec_of);
   dfree(c->d_traces);
   dfree(c->d_obs);
   dfree(c->d_resid);
   TRY(dalloc(c, &c->d_rec_node, (size_t)nrec));
   TRY(dalloc(c, &c->d_rec_vec, 3 * (size_t)nrec));
-  CUDA_TRY(c, cudaMemcpy(c->d_rec_node, nodes.data(), sizeof(int64_t) * nrec, cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpyAsync(c->d_rec_node, nodes.data(), sizeof(int64_t) * nrec, cudaMemcpyHostToDevice, c->stream));
   CUDA_TRY(c, cudaMemcpy(c->d_rec_vec, vec.data(), sizeof(float) * 3 * nrec, cudaMemcpyHostToDevice));
-  TRY(dalloc(c, &c->d_rec_of, (size_t)c->geo.stride));
-  fwi::launch_rec_map(c->d_rec_node, nrec, c->d_rec_of, c->geo.stride, c->stream);
+  const int64_t plane = (int64_t)c->geo.px * c->geo.n[1];
+  c->rec0 = k0 * plane;
+  c->rec_n = (k1 - k0 + 1) * plane;
+  TRY(dalloc(c, &c->d_rec_of, (size_t)c->rec_n));
+  fwi::launch_rec_map(c->d_rec_node, nrec, c->d_rec_of, c->rec0, c->rec_n, c->stream);
   CUDA_TRY(c, cudaGetLastError());
-  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   c->nrec = nrec;
   c->rec_node = nodes;
   c->rec_k[0] = k0;

@@ -102,7 +102,8 @@ struct Points {
   int k0, k1;
   const int64_t *src_node;
   const float *src_vec, *rec_vec, *table;
-  const int *rec_of;  // node -> receiver, or -1
+  const int *rec_of;  // of the nodes rec0 .. rec0 + rec_n - 1 (the receivers' planes): receiver, or -1
+  int64_t rec0, rec_n;
   float *traces;
   int64_t tstride;
 };
@@ -142,12 +143,18 @@ __host__ __device__ inline StageArgs shot_args(StageArgs a, int shot) {
 
 __device__ __forceinline__ bool has_points(const Points &q, int K) { return K >= q.k0 && K <= q.k1; }
 
+// receiver at a node, or -1
+__device__ __forceinline__ int rec_at(const Points &q, int64_t node) {
+  const int64_t m = node - q.rec0;
+  return m >= 0 && m < q.rec_n ? __ldg(q.rec_of + m) : -1;
+}
+
 // a node of a plane with points, after this thread wrote its components c0 .. c1 - 1: adds the
 // point load and takes the sample. It reads the values back (by the thread that wrote them), so
 // that the rest of a kernel holds nothing for it.
 __device__ __forceinline__ void node_points(const Points &q, const StageArgs &a, int64_t b, int64_t S, int64_t node, int c0,
                                             int c1, unsigned long long *oob) {
-  const int r = q.load == 2 || q.traces ? __ldg(q.rec_of + node) : -1;
+  const int r = q.load == 2 || q.traces ? rec_at(q, node) : -1;
   const bool rec = r >= 0 && guard(oob, kSitePoint, r, q.nrec), src = q.load == 1 && node == __ldg(q.src_node + b);
   if (!rec && !src) return;
 #pragma unroll 1
@@ -213,8 +220,8 @@ struct PersistArgs {
 };
 cudaError_t launch_persistent_forward(const Geo &g, const PersistArgs &p, cudaStream_t s);
 
-// rec_of[node[r]] = r for the nrec receivers, -1 at the other `stride` entries
-void launch_rec_map(const int64_t *node, int nrec, int *rec_of, int64_t stride, cudaStream_t s);
+// rec_of[node[r] - rec0] = r for the nrec receivers, -1 at the other of its rec_n entries
+void launch_rec_map(const int64_t *node, int nrec, int *rec_of, int64_t rec0, int64_t rec_n, cudaStream_t s);
 
 // Gradient integrand of (C.1f)/(C.1g) at one time level, accumulated in FP64:
 // gl[i] -= wdt * sum_e W detJ (div w)(div u), gm[i] -= wdt * sum_e W detJ 2 eps(w):eps(u),

@@ -17,9 +17,9 @@ namespace {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-__global__ void rec_map_kernel(const int64_t *node, int nrec, int *rec_of) {
+__global__ void rec_map_kernel(const int64_t *node, int nrec, int *rec_of, int64_t rec0) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < nrec) rec_of[node[r]] = r;
+  if (r < nrec) rec_of[node[r] - rec0] = r;
 }
 
 // the sources (load 1, one per shot) and receivers of a stage (see Points): thread per shot and
@@ -31,7 +31,7 @@ __global__ void points_kernel(Geo g, StageArgs a0, Points q, const int64_t *__re
   const int64_t node = i < q.nrec ? rec_node[i] : q.src_node[b];
   if (!guard(g.oob, kSitePoint, node, g.stride)) return;
   // a source that is sampled too is the receiver's thread's
-  if (i == q.nrec && q.traces && q.rec_of[node] >= 0) return;
+  if (i == q.nrec && q.traces && rec_at(q, node) >= 0) return;
   if (q.fused) {
     const int I = (int)(node % g.px), r = (int)(node / g.px), J = r % g.n[1], K = r / g.n[1];
     const bool face = I == 0 || I == g.n[0] - 1 || J == 0 || J == g.n[1] - 1 || K == 0 || K == g.n[2] - 1;
@@ -227,9 +227,9 @@ int launch_points(const Geo &g, const StageArgs &a, const Points &q, const int64
   return 1;
 }
 
-void launch_rec_map(const int64_t *node, int nrec, int *rec_of, int64_t stride, cudaStream_t s) {
-  cudaMemsetAsync(rec_of, 0xff, sizeof(int) * (size_t)stride, s);
-  rec_map_kernel<<<blocks_for(nrec, 256), 256, 0, s>>>(node, nrec, rec_of);
+void launch_rec_map(const int64_t *node, int nrec, int *rec_of, int64_t rec0, int64_t rec_n, cudaStream_t s) {
+  cudaMemsetAsync(rec_of, 0xff, sizeof(int) * (size_t)rec_n, s);
+  rec_map_kernel<<<blocks_for(nrec, 256), 256, 0, s>>>(node, nrec, rec_of, rec0);
 }
 
 void launch_gradient(const Geo &g, const float *w_state, const float *u_hist, double wdt, double *gl,
