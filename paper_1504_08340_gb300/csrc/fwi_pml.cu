@@ -180,16 +180,35 @@ __device__ __forceinline__ Coef2 coef_pair(const Geo &g, int I0, int J, int K) {
   return c;
 }
 
-// stage output of a node pair from its own input value y and rate r; MODE 0: the
-// rate, 1: stage 1 (X is the stage input, so x = y), 2: stages 2-3, 3: stage 4
+// Stage output of a node pair from its own input value y, rate r and the step-start value x that
+// step_start loaded; MODE 0: the rate, 1: stage 1 (X is the stage input, so x = y), 2: stages
+// 2-3, 3: stage 4 (x: -X + Y2 + 2 Y3)
 template <int MODE>
-__device__ __forceinline__ float2 stage2(const StageArgs &a, int idx, float2 y, float2 r) {
+__device__ __forceinline__ float2 step_start(const StageArgs &a, int idx) {
+  if constexpr (MODE <= 1) return bc(0.f);
+  const float2 x = ldcg2(a.X + idx);
+  if constexpr (MODE == 2) return x;
+  const float2 b = ldcg2(a.Y2 + idx), c = ldcg2(a.Y3 + idx);
+  return pfma(bc(2.f), c, psub(b, x));
+}
+template <int MODE>
+__device__ __forceinline__ float2 stage2(const StageArgs &a, float2 x, float2 y, float2 r) {
   if constexpr (MODE == 0) return r;
   if constexpr (MODE == 1) return pfma(bc(a.cdt), r, y);
-  const float2 x = ldcg2(a.X + idx);
   if constexpr (MODE == 2) return pfma(bc(a.cdt), r, x);
-  const float2 b = ldcg2(a.Y2 + idx), c = ldcg2(a.Y3 + idx);
-  return pfma(bc(1.f / 3.f), padd(pfma(bc(2.f), c, psub(b, x)), y), pmul(bc(a.cdt), r));
+  return pfma(bc(1.f / 3.f), padd(x, y), pmul(bc(a.cdt), r));
+}
+// the step-start values of three variables from field f on, loaded together: a.out may be a.X, so
+// the compiler keeps these loads behind the stores of the variables before, and each group waits
+// once for its own. One variable at a time, the nine waits in a row made the kernel's end a chain
+// (64x64x32 gradient 71.0 ms, two at a time 69.9, three 68.2, all six of the stresses 72.6).
+constexpr int kXG = 3;
+template <int MODE>
+__device__ __forceinline__ void step_starts(const StageArgs &a, int f, int S, int node, float2 x[kXG][3]) {
+#pragma unroll
+  for (int k = 0; k < kXG; k++)
+#pragma unroll
+    for (int lv = 0; lv < 3; lv++) x[k][lv] = step_start<MODE>(a, (9 * lv + f + k) * S + node);
 }
 
 // adjoint: column j of sum_lv Lambda^lv_jj tau(T^lv) at the nodes (I0, J, K) and
@@ -235,8 +254,8 @@ __device__ __forceinline__ void adj_yz(const Geo &g, const float *__restrict__ Y
   }
 }
 
-// PART 0: the whole pair update; 1: the stress rows only; 2: the displacement rows only
-template <bool ADJ, int MODE, int KY, int KZ, int PART = 0>
+// PART 1: the stress rows; 2: the displacement rows
+template <bool ADJ, int MODE, int KY, int KZ, int PART>
 __device__ void pml_pair(const Geo &g, const StageArgs &a, int I0, int J, int K, bool even_ok) {
   constexpr bool DO_S = PART != 2, DO_U = PART != 1;
   const int S = (int)g.stride;
@@ -301,9 +320,12 @@ __device__ void pml_pair(const Geo &g, const StageArgs &a, int I0, int J, int K,
   const float2 ih = bc(g.inv_h);
   // S components in the order xx yy zz yz xz xy; for each: (c, j) pairs it feeds
   constexpr bool PHASE_B = DO_S || !ADJ;  // the adjoint u rows need nothing from this loop
+  float2 xs[kXG][3];
 #pragma unroll
   for (int comp = 0; comp < (PHASE_B ? 6 : 0); comp++) {
     float2 sv[3];  // own values per level
+    if constexpr (DO_S)
+      if (comp % kXG == 0) step_starts<MODE>(a, 3 + comp, S, node, xs);
 #pragma unroll
     for (int lv = 0; lv < 3; lv++) {
       const float *p = Yn + (9 * lv + 3 + comp) * S;
@@ -333,22 +355,26 @@ __device__ void pml_pair(const Geo &g, const StageArgs &a, int I0, int J, int K,
     // stress update of this component: S'' = (src - b S' - c S - d Sbar) / a
     const int i0 = (3 + comp) * S + node, i1 = (12 + comp) * S + node, i2 = (21 + comp) * S + node;
     const float2 acc = pmul(pfma(cf.nb, sv[2], pfma(cf.nc, sv[1], pfma(cf.nd, sv[0], pmul(s[comp], ih)))), cf.ia);
-    st2(a.out + i0, stage2<MODE>(a, i0, sv[0], sv[1]), even_ok);
-    st2(a.out + i1, stage2<MODE>(a, i1, sv[1], sv[2]), even_ok);
-    st2(a.out + i2, stage2<MODE>(a, i2, sv[2], acc), even_ok);
+    const float2 *x = xs[comp % kXG];
+    st2(a.out + i0, stage2<MODE>(a, x[0], sv[0], sv[1]), even_ok);
+    st2(a.out + i1, stage2<MODE>(a, x[1], sv[1], sv[2]), even_ok);
+    st2(a.out + i2, stage2<MODE>(a, x[2], sv[2], acc), even_ok);
   }
   // ---- displacement update: u'' = (f / h) / (rho a) - (b u' + c u + d ubar) / a
   // (own u values read again here rather than held since the S rows)
   if constexpr (!DO_U) return;
   const float2 irh = bc(g.inv_rho_h);
+  float2 xu[kXG][3];
+  step_starts<MODE>(a, 0, S, node, xu);
 #pragma unroll
   for (int c = 0; c < 3; c++) {
     const int i0 = c * S + node, i1 = (9 + c) * S + node, i2 = (18 + c) * S + node;
     const float2 u0 = ld2(Yn + c * S), u1 = ld2(Yn + (9 + c) * S), u2 = ld2(Yn + (18 + c) * S);
     const float2 acc = pmul(pfma(cf.nb, u2, pfma(cf.nc, u1, pfma(cf.nd, u0, pmul(irh, f[c])))), cf.ia);
-    st2(a.out + i0, stage2<MODE>(a, i0, u0, u1), even_ok);
-    st2(a.out + i1, stage2<MODE>(a, i1, u1, u2), even_ok);
-    st2(a.out + i2, stage2<MODE>(a, i2, u2, acc), even_ok);
+    const float2 *x = xu[c];
+    st2(a.out + i0, stage2<MODE>(a, x[0], u0, u1), even_ok);
+    st2(a.out + i1, stage2<MODE>(a, x[1], u1, u2), even_ok);
+    st2(a.out + i2, stage2<MODE>(a, x[2], u2, acc), even_ok);
   }
 }
 
@@ -508,16 +534,13 @@ __device__ __forceinline__ void face_write(const Geo &g, const StageArgs &a, con
 }
 
 #ifndef FWI_PML_STAGE4_MINB
-#define FWI_PML_STAGE4_MINB 7  // stage 4 reads three more step-start rows: 72 registers, no spills
-#endif
-#ifndef FWI_PML_SPLIT_MINB
-#define FWI_PML_SPLIT_MINB 9  // 56 registers, 40 bytes of spills: 64x64x32 gradient 71.1 ms, at 8 blocks 73.8, at 10 76.4
-#endif
-#ifndef FWI_PML_BY
-#define FWI_PML_BY 4
+#define FWI_PML_STAGE4_MINB 6  // stage 4 reads three step-start rows: 80 registers
 #endif
 #ifndef FWI_PML_MINB
 #define FWI_PML_MINB 7
+#endif
+#ifndef FWI_PML_BY
+#define FWI_PML_BY 4
 #endif
 #ifndef FWI_FACE_MINB
 #define FWI_FACE_MINB 10
@@ -528,21 +551,17 @@ constexpr int kPackBelow = 28;  // pairs of an x segment below which its rows ar
 
 // grid.x: blocks of kBY warp tasks (see Region); tasks of a box run plane by plane.
 // The boxes exclude the outer faces of the grid, so every node takes the bulk path.
-// PART 3 runs the stress-row update and then the displacement-row update of the same
-// pair in the same thread: each part keeps its own register footprint, and the second
-// part's loads (the rows the first part just read) hit in L1/L2 instead of DRAM.
-template <bool ADJ, int MODE, int KY, int KZ, int PART>
+// A task runs the stress-row update and then the displacement-row update of the same pair in
+// the same thread: each part keeps its own register footprint, and the second part's loads
+// (the rows the first part just read) hit in L1/L2 instead of DRAM.
+template <bool ADJ, int MODE, int KY, int KZ>
 __device__ __forceinline__ void pml_task(const Geo &g, const StageArgs &a, int I0, int J, int K, bool even_ok) {
-  if constexpr (PART == 3) {
-    pml_pair<ADJ, MODE, KY, KZ, 1>(g, a, I0, J, K, even_ok);
-    pml_pair<ADJ, MODE, KY, KZ, 2>(g, a, I0, J, K, even_ok);
-  } else {
-    pml_pair<ADJ, MODE, KY, KZ, PART>(g, a, I0, J, K, even_ok);
-  }
+  pml_pair<ADJ, MODE, KY, KZ, 1>(g, a, I0, J, K, even_ok);
+  pml_pair<ADJ, MODE, KY, KZ, 2>(g, a, I0, J, K, even_ok);
 }
 
-template <bool ADJ, int MODE, int PART>
-__global__ void __launch_bounds__(kBX *kBY, MODE == 3 ? FWI_PML_STAGE4_MINB : (PART == 0 ? FWI_PML_MINB : FWI_PML_SPLIT_MINB))
+template <bool ADJ, int MODE>
+__global__ void __launch_bounds__(kBX *kBY, MODE == 3 ? FWI_PML_STAGE4_MINB : FWI_PML_MINB)
     pml_kernel(Geo g, StageArgs a0, Region r) {
   const int nbs = (r.tasks_before[r.nbox] + kBY - 1) / kBY;  // blocks per shot
   const StageArgs a = shot_args(a0, blockIdx.x / nbs);
@@ -580,11 +599,11 @@ __global__ void __launch_bounds__(kBX *kBY, MODE == 3 ? FWI_PML_STAGE4_MINB : (P
     // the even node of a box's first pair may not be (its results are dropped)
     const bool even_ok = I0 >= r.lo[b][0];
     if (ky == kSC) {
-      if (kz == kSC) pml_task<ADJ, MODE, kSC, kSC, PART>(g, a, I0, J, K, even_ok);
-      else pml_task<ADJ, MODE, kSC, kSLR, PART>(g, a, I0, J, K, even_ok);
+      if (kz == kSC) pml_task<ADJ, MODE, kSC, kSC>(g, a, I0, J, K, even_ok);
+      else pml_task<ADJ, MODE, kSC, kSLR>(g, a, I0, J, K, even_ok);
     } else {
-      if (kz == kSC) pml_task<ADJ, MODE, kSLR, kSC, PART>(g, a, I0, J, K, even_ok);
-      else pml_task<ADJ, MODE, kSLR, kSLR, PART>(g, a, I0, J, K, even_ok);
+      if (kz == kSC) pml_task<ADJ, MODE, kSLR, kSC>(g, a, I0, J, K, even_ok);
+      else pml_task<ADJ, MODE, kSLR, kSLR>(g, a, I0, J, K, even_ok);
     }
   }
 }
@@ -666,19 +685,15 @@ int launch_pml(const Geo &g, const StageArgs &a, bool adjoint, cudaStream_t s) {
   if (tasks == 0) return 0;
   const dim3 grd((tasks + kBY - 1) / kBY * a.nshot), blk(kBX, kBY);
   const int mode = a.stage == 0 ? 0 : (a.stage == 1 ? 1 : (a.stage < 4 ? 2 : 3));
-  // PART 3: one launch, per pair the stress rows, then the displacement rows (disjoint outputs, the
-  // same inputs), each part with the registers of its own update
-  if (adjoint) {
-    if (mode == 0) pml_kernel<true, 0, 3><<<grd, blk, 0, s>>>(g, a, r);
-    else if (mode == 1) pml_kernel<true, 1, 3><<<grd, blk, 0, s>>>(g, a, r);
-    else if (mode == 2) pml_kernel<true, 2, 3><<<grd, blk, 0, s>>>(g, a, r);
-    else pml_kernel<true, 3, 3><<<grd, blk, 0, s>>>(g, a, r);
-  } else {
-    if (mode == 0) pml_kernel<false, 0, 3><<<grd, blk, 0, s>>>(g, a, r);
-    else if (mode == 1) pml_kernel<false, 1, 3><<<grd, blk, 0, s>>>(g, a, r);
-    else if (mode == 2) pml_kernel<false, 2, 3><<<grd, blk, 0, s>>>(g, a, r);
-    else pml_kernel<false, 3, 3><<<grd, blk, 0, s>>>(g, a, r);
-  }
+  const auto kernel = adjoint ? (mode == 0   ? pml_kernel<true, 0>
+                                 : mode == 1 ? pml_kernel<true, 1>
+                                 : mode == 2 ? pml_kernel<true, 2>
+                                             : pml_kernel<true, 3>)
+                              : (mode == 0   ? pml_kernel<false, 0>
+                                 : mode == 1 ? pml_kernel<false, 1>
+                                 : mode == 2 ? pml_kernel<false, 2>
+                                             : pml_kernel<false, 3>);
+  kernel<<<grd, blk, 0, s>>>(g, a, r);
   return 1;
 }
 
