@@ -207,8 +207,8 @@ __device__ __forceinline__ void load_own(const Geo &g, const StageArgs &a, int64
       o.x2[c] = __ldcs(a.X + i2);
     }
     if constexpr (MODE == 3) {
-      o.x1[c] = -o.x1[c] + __ldcs(a.Y2 + i1) + 2.f * __ldcs(a.Y3 + i1);
-      o.x2[c] = -o.x2[c] + __ldcs(a.Y2 + i2) + 2.f * __ldcs(a.Y3 + i2);
+      o.x1[c] = __fmaf_rn(2.f, __ldcs(a.Y3 + i1), __ldcs(a.Y2 + i1) - o.x1[c]);
+      o.x2[c] = __fmaf_rn(2.f, __ldcs(a.Y3 + i2), __ldcs(a.Y2 + i2) - o.x2[c]);
     }
   }
 }
@@ -217,9 +217,9 @@ __device__ __forceinline__ void load_own(const Geo &g, const StageArgs &a, int64
 template <int MODE>
 __device__ __forceinline__ float stage_value(const StageArgs &a, float x, float yv, float rate) {
   if constexpr (MODE == 0) return rate;
-  if constexpr (MODE == 1) return yv + a.cdt * rate;
-  if constexpr (MODE == 2) return x + a.cdt * rate;
-  return (x + yv) * (1.f / 3.f) + a.cdt * rate;
+  if constexpr (MODE == 1) return __fmaf_rn(a.cdt, rate, yv);
+  if constexpr (MODE == 2) return __fmaf_rn(a.cdt, rate, x);
+  return __fmaf_rn(1.f / 3.f, x + yv, __fmul_rn(a.cdt, rate));
 }
 
 // write the stage outputs of one interior node

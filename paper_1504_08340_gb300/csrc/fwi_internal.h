@@ -143,6 +143,35 @@ __host__ __device__ inline StageArgs shot_args(StageArgs a, int shot) {
 
 __device__ __forceinline__ bool has_points(const Points &q, int K) { return K >= q.k0 && K <= q.k1; }
 
+// RK4 stage update of one variable's three levels at a node, for the list kernels: the step-start
+// values are loaded together and before any of the node's stores (a.out may be a.X, so a load
+// after a store waits its own latency: nine in a row for a node's three variables made up much of
+// those kernels' time). The levels of variable f are the fields f, 9 + f, 18 + f. The fused
+// multiply-adds are written out: a node's value must not depend on which variant of a kernel
+// (warps per block, points) a launch's size picks, and the compiler contracts a sum of two
+// products either way.
+struct StepStart {
+  float v[3];
+};
+__device__ __forceinline__ StepStart load_start(const StageArgs &a, int64_t i0, int64_t nine) {
+  StepStart x{{0.f, 0.f, 0.f}};
+  if (a.stage >= 2) {  // in stage 1 X is the stage input
+#pragma unroll
+    for (int l = 0; l < 3; l++) x.v[l] = __ldcs(a.X + i0 + l * nine);
+  }
+  if (a.stage == 4) {
+#pragma unroll
+    for (int l = 0; l < 3; l++) x.v[l] = __fmaf_rn(2.f, __ldcs(a.Y3 + i0 + l * nine), __ldcs(a.Y2 + i0 + l * nine) - x.v[l]);
+  }
+  return x;
+}
+__device__ __forceinline__ float stage_value(const StageArgs &a, float x, float yv, float rate) {
+  if (a.stage == 0) return rate;
+  if (a.stage == 1) return __fmaf_rn(a.cdt, rate, yv);
+  if (a.stage < 4) return __fmaf_rn(a.cdt, rate, x);
+  return __fmaf_rn(1.f / 3.f, x + yv, __fmul_rn(a.cdt, rate));
+}
+
 // receiver at a node, or -1
 __device__ __forceinline__ int rec_at(const Points &q, int64_t node) {
   const int64_t m = node - q.rec0;

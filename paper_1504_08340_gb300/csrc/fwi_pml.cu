@@ -78,14 +78,6 @@ struct Region {
   int tasks_before[7];     // prefix sums of warp tasks per box
 };
 
-__device__ __forceinline__ float stage_value(const StageArgs &a, int idx, float yv, float rate) {
-  if (a.stage == 0) return rate;
-  if (a.stage == 1) return yv + a.cdt * rate;  // X is the stage input
-  if (a.stage < 4) return __ldcs(a.X + idx) + a.cdt * rate;
-  return (-__ldcs(a.X + idx) + __ldcs(a.Y2 + idx) + 2.f * __ldcs(a.Y3 + idx) + yv) * (1.f / 3.f) + a.cdt * rate;
-}
-
-
 // ---------------------------------------------------------------------------
 // Vectorised pair path: a thread owns the nodes (I0, I0 + 1), I0 even, of a bulk
 // row. Rows are padded to a multiple of 4 nodes, so every (I0, I0 + 1) pair is
@@ -489,17 +481,22 @@ __device__ __forceinline__ void face_write(const Geo &g, const StageArgs &a, con
                                            const FaceShared &sh, int lane, int w, const Points &q, int shot) {
   const int S = (int)g.stride;
   const float *__restrict__ Y = a.Y;
+  const int f[3] = {w, 3 + w, 6 + w};  // displacement component w, stress components w and w + 3
+  StepStart x[3];
+  if (!n.dir) x[0] = load_start(a, f[0] * S + n.node, 9 * S);
+#pragma unroll
+  for (int h = 1; h < 3; h++) x[h] = load_start(a, f[h] * S + n.node, 9 * S);
   // ---- displacement component w
   {
     const int c = w;
     const int i0 = c * S + n.node, i1 = (9 + c) * S + n.node, i2 = (18 + c) * S + n.node;
     if (!n.dir) {
-      const float f = sh.f[0][c][lane] + sh.f[1][c][lane] + sh.f[2][c][lane];
+      const float fc = sh.f[0][c][lane] + sh.f[1][c][lane] + sh.f[2][c][lane];
       const float u0 = __ldg(Y + i0), u1 = __ldg(Y + i1), u2 = __ldg(Y + i2);
-      const float acc = (g.inv_rho_h * f - (n.cb * u2 + n.cc * u1 + n.cd * u0)) * n.inv_a;
-      __stcs(a.out + i0, stage_value(a, i0, u0, u1));
-      __stcs(a.out + i1, stage_value(a, i1, u1, u2));
-      __stcs(a.out + i2, stage_value(a, i2, u2, acc));
+      const float acc = (g.inv_rho_h * fc - (n.cb * u2 + n.cc * u1 + n.cd * u0)) * n.inv_a;
+      __stcs(a.out + i0, stage_value(a, x[0].v[0], u0, u1));
+      __stcs(a.out + i1, stage_value(a, x[0].v[1], u1, u2));
+      __stcs(a.out + i2, stage_value(a, x[0].v[2], u2, acc));
       if (q.fused && has_points(q, K)) node_points(q, a, shot, S, n.node, c, c + 1, g.oob);
     } else if (a.stage == 0) {
       __stcs(a.out + i0, 0.f);
@@ -527,9 +524,10 @@ __device__ __forceinline__ void face_write(const Geo &g, const StageArgs &a, con
     }
     const int i0 = (3 + c) * S + n.node, i1 = (12 + c) * S + n.node, i2 = (21 + c) * S + n.node;
     const float s0 = __ldg(Y + i0), s1 = __ldg(Y + i1), s2 = __ldg(Y + i2);
-    __stcs(a.out + i0, stage_value(a, i0, s0, s1));
-    __stcs(a.out + i1, stage_value(a, i1, s1, s2));
-    __stcs(a.out + i2, stage_value(a, i2, s2, (g.inv_h * src - n.cb * s2 - n.cc * s1 - n.cd * s0) * n.inv_a));
+    const StepStart &xs = x[1 + h];
+    __stcs(a.out + i0, stage_value(a, xs.v[0], s0, s1));
+    __stcs(a.out + i1, stage_value(a, xs.v[1], s1, s2));
+    __stcs(a.out + i2, stage_value(a, xs.v[2], s2, (g.inv_h * src - n.cb * s2 - n.cc * s1 - n.cd * s0) * n.inv_a));
   }
 }
 

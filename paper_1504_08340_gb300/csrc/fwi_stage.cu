@@ -106,15 +106,6 @@ __device__ __forceinline__ int point_type(int p) { return p == 0 ? kR : (p == 1 
 __host__ __device__ constexpr int sym(int i, int j) { return i == j ? i : (i + j == 1 ? 5 : (i + j == 2 ? 4 : 3)); }
 
 
-// RK4 stage update of one field value with stage-input value yv (see StageArgs;
-// in stage 1 X is the stage input)
-__device__ __forceinline__ float stage_value(const StageArgs &a, int64_t idx, float yv, float rate) {
-  if (a.stage == 0) return rate;
-  if (a.stage == 1) return yv + a.cdt * rate;
-  if (a.stage < 4) return __ldcs(a.X + idx) + a.cdt * rate;
-  return (-__ldcs(a.X + idx) + __ldcs(a.Y2 + idx) + 2.f * __ldcs(a.Y3 + idx) + yv) * (1.f / 3.f) + a.cdt * rate;
-}
-
 __device__ __forceinline__ void write_hist(const Geo &g, const StageArgs &a, int I, int J, int K, int c, float v) {
   const int i = I - 2 * g.lo[0], j = J - 2 * g.lo[1], k = K - 2 * g.lo[2];
   if (i >= 0 && i < g.m[0] && j >= 0 && j < g.m[1] && k >= 0 && k < g.m[2])
@@ -373,14 +364,14 @@ __device__ __forceinline__ float shell_force(const Geo &g, const ShellShared &sh
   const float s_rd = g.inv_h * g.inv_h * (1.f / 3.f), s_pml = g.inv_h * (1.f / 3.f);
   float f[3];
 #pragma unroll
-  for (int j = 0; j < 3; j++) f[j] = s_rd * sh.fr[j][c][lane] + s_pml * sh.fp[j][c][lane];
+  for (int j = 0; j < 3; j++) f[j] = __fmaf_rn(s_rd, sh.fr[j][c][lane], __fmul_rn(s_pml, sh.fp[j][c][lane]));
   return f[0] + f[1] + f[2];
 }
 
 // stress component c (order xx yy zz yz xz xy) of the node: its three levels
 template <bool ADJ>
 __device__ __forceinline__ void shell_stress(const Geo &g, const StageArgs &a, const NodeCtx &n,
-                                             const ShellShared &sh, int lane, int c) {
+                                             const ShellShared &sh, int lane, int c, const StepStart &x) {
   const int64_t S = g.stride;
   const float *__restrict__ Y = a.Y;
   const int64_t i0 = (int64_t)(3 + c) * S + n.node, i1 = (int64_t)(12 + c) * S + n.node,
@@ -396,25 +387,25 @@ __device__ __forceinline__ void shell_stress(const Geo &g, const StageArgs &a, c
   const float sc = g.inv_h / (float)n.npml;
   // P(H): diagonal H_ii, off-diagonal H_ij + H_ji
   auto P = [&](int k) {
-    if (k < 3) return sc * sh.H[k][k][lane];
+    if (k < 3) return __fmul_rn(sc, sh.H[k][k][lane]);
     const int i = k == 5 ? 0 : (k == 4 ? 0 : 1), j = k == 5 ? 1 : 2;  // xy, xz, yz
-    return sc * (sh.H[i][j][lane] + sh.H[j][i][lane]);
+    return __fmul_rn(sc, sh.H[i][j][lane] + sh.H[j][i][lane]);
   };
   float src = P(c);
   if (!ADJ) {  // tau(P(H)) = mu (P + diag P) + lambda tr(P) I
     const float lam = __ldg(g.lam_n + n.node), mu = __ldg(g.mu_n + n.node);
-    src = c < 3 ? 2.f * mu * src + lam * (P(0) + P(1) + P(2)) : mu * src;
+    src = c < 3 ? __fmaf_rn(lam, P(0) + P(1) + P(2), __fmul_rn(2.f * mu, src)) : __fmul_rn(mu, src);
   }
   const float s0 = __ldg(Y + i0), s1 = __ldg(Y + i1), s2 = __ldg(Y + i2);
-  __stcs(a.out + i0, stage_value(a, i0, s0, s1));
-  __stcs(a.out + i1, stage_value(a, i1, s1, s2));
-  __stcs(a.out + i2, stage_value(a, i2, s2, (src - n.cb * s2 - n.cc * s1 - n.cd * s0) * n.inv_a));
+  __stcs(a.out + i0, stage_value(a, x.v[0], s0, s1));
+  __stcs(a.out + i1, stage_value(a, x.v[1], s1, s2));
+  __stcs(a.out + i2, stage_value(a, x.v[2], s2, __fmul_rn(__fmaf_rn(-n.cd, s0, __fmaf_rn(-n.cc, s1, __fmaf_rn(-n.cb, s2, src))), n.inv_a)));
 }
 
 // displacement component c of the node: its three levels
 template <bool PTS>
 __device__ __forceinline__ void shell_disp(const Geo &g, const StageArgs &a, const Points &q, int shot, const NodeCtx &n,
-                                           const ShellShared &sh, int lane, int c) {
+                                           const ShellShared &sh, int lane, int c, const StepStart &x) {
   const int64_t S = g.stride;
   const float *__restrict__ Y = a.Y;
   const int64_t i0 = (int64_t)c * S + n.node, i1 = (int64_t)(9 + c) * S + n.node, i2 = (int64_t)(18 + c) * S + n.node;
@@ -429,14 +420,31 @@ __device__ __forceinline__ void shell_disp(const Geo &g, const StageArgs &a, con
   const float fsum = shell_force(g, sh, c, lane);
   const float inv_m = n.inv_a / (g.rho * (float)n.nel);
   const float u0 = __ldg(Y + i0), u1 = __ldg(Y + i1), u2 = __ldg(Y + i2);
-  const float acc = -fsum * inv_m - (n.cb * u2 + n.cc * u1 + n.cd * u0) * n.inv_a;
-  if (n.pml || a.stage == 0) __stcs(a.out + i0, stage_value(a, i0, u0, n.pml ? u1 : 0.f));
-  const float v1 = stage_value(a, i1, u1, u2);
+  const float decay = __fmaf_rn(n.cd, u0, __fmaf_rn(n.cc, u1, __fmul_rn(n.cb, u2)));
+  const float acc = -__fmaf_rn(decay, n.inv_a, __fmul_rn(fsum, inv_m));
+  if (n.pml || a.stage == 0) __stcs(a.out + i0, stage_value(a, x.v[0], u0, n.pml ? u1 : 0.f));
+  const float v1 = stage_value(a, x.v[1], u1, u2);
   __stcs(a.out + i1, v1);
-  __stcs(a.out + i2, stage_value(a, i2, u2, acc));
+  __stcs(a.out + i2, stage_value(a, x.v[2], u2, acc));
   if constexpr (PTS)
     if (has_points(q, n.c3[2])) node_points(q, a, shot, S, n.node, c, c + 1, g.oob);
   if (a.hist) write_hist(g, a, n.c3[0], n.c3[1], n.c3[2], c, v1);
+}
+
+// second phase of warp w of W: displacement component w (w < 3), stress components w, w + W, ...
+template <bool ADJ, int W, bool PTS>
+__device__ __forceinline__ void shell_write(const Geo &g, const StageArgs &a, const Points &q, int shot, const NodeCtx &n,
+                                            const ShellShared &sh, int lane, int w) {
+  constexpr int NS = 6 / W;
+  const int64_t S = g.stride;
+  StepStart xu{}, xs[NS];
+  if (w < 3 && !n.dir) xu = load_start(a, w * S + n.node, 9 * S);
+#pragma unroll
+  for (int h = 0; h < NS; h++)
+    if (n.pml) xs[h] = load_start(a, (3 + w + h * W) * S + n.node, 9 * S);
+  if (w < 3) shell_disp<PTS>(g, a, q, shot, n, sh, lane, w, xu);
+#pragma unroll
+  for (int h = 0; h < NS; h++) shell_stress<ADJ>(g, a, n, sh, lane, w + h * W, xs[h]);
 }
 
 template <bool ADJ, int W, bool PTS>
@@ -456,10 +464,7 @@ __global__ void __launch_bounds__(W *kShellNodes, 24 / W) shell_kernel(Geo g, St
     shell_terms<ADJ, W>(g, a, n, sh, lane, w);
   }
   __syncthreads();
-  if (live) {
-    if (w < 3) shell_disp<PTS>(g, a, q, shot, n, sh, lane, w);
-    for (int c = w; c < 6; c += W) shell_stress<ADJ>(g, a, n, sh, lane, c);
-  }
+  if (live) shell_write<ADJ, W, PTS>(g, a, q, shot, n, sh, lane, w);
 }
 
 // ---- persistent forward sweep (see PersistArgs)
@@ -538,10 +543,7 @@ __global__ void __launch_bounds__(kPersistWarps *kShellNodes, 3) persistent_forw
           shell_terms<false, kPersistWarps>(g, a, n, sh, lane, w);
         }
         __syncthreads();
-        if (live) {
-          if (w < 3) shell_disp<true>(g, a, q, b, n, sh, lane, w);
-          for (int c = w; c < 6; c += kPersistWarps) shell_stress<false>(g, a, n, sh, lane, c);
-        }
+        if (live) shell_write<false, kPersistWarps, true>(g, a, q, b, n, sh, lane, w);
         __syncthreads();
       }
       if (!grid_barrier(p, expected)) return;
