@@ -255,7 +255,7 @@ cudaError_t box_map(CUtensorMap *tm, uint16_t *src, int D, int H, int W, int G, 
 //
 // Issuing an MMA costs its thread 50 to 150 clocks of descriptor arithmetic and moves to
 // uniform registers (measured), more than an MMA of N = 32 runs (40 clocks): so warp p issues
-// the MMAs of plane p, and the four chains keep the tensor pipe fed. Warp 4 copies.
+// the MMAs of plane p, and the four chains keep the tensor pipe fed. Warp 4 copies, warps 5 to 8 write the results.
 //
 // Bound: in the MMA phase the operands' shared-memory reads (M = 128, K = 16: 4 KB of A for
 // any N); the epilogue's stores (8 voxels of a row per channel) overlap it only across the
@@ -263,7 +263,7 @@ cudaError_t box_map(CUtensorMap *tm, uint16_t *src, int D, int H, int W, int G, 
 // one plane a block, 28 -> 28 channels moved 90 KB through L2 per 128 voxels, 27 KB now.
 // Measured at 65 x 129 x 129 voxels: forward 28 -> 28 226 -> 142 us, backward data 28 -> 84
 // 1359 -> 546 us (one thread issuing for one plane a block before).
-constexpr int kTileThreads = 160;
+constexpr int kTileThreads = 288;
 constexpr int kRingB = 4;      // most weight copies in flight
 constexpr int kMaxPlanes = 4;  // output planes of a block
 constexpr int kMaxBox = 2;     // box buffers (passes in flight)
@@ -273,7 +273,10 @@ struct TileShape {
   int gp, npass, G;  // groups per pass, passes, groups of the source (even)
   int planes, nbox;  // output planes per block, box buffers
   int taps, ring;    // taps per weight copy (1, 3 or 9), weight buffers
+  int nacc;          // accumulator sets (2: a tile's epilogue runs beside the next tile's MMAs)
   int cols, smem;    // TMEM columns, dynamic shared memory
+  int64_t tiles;     // (x, y) tiles x plane chunks x N tiles
+  int grid;          // blocks
 };
 
 // weight chunks: for N tile nt, pass ps, tap t: nt_n x (gp x 8) K-major, core (kg, ng) at
@@ -305,43 +308,50 @@ __global__ void tile_pack_kernel(const uint16_t *__restrict__ w, int n_rows, int
 }
 
 template <bool BWD>
-__global__ void __launch_bounds__(kTileThreads)
+__global__ void __launch_bounds__(kTileThreads, 2)
     tile_conv_kernel(const __grid_constant__ CUtensorMap tm, const uint16_t *__restrict__ wpack,
                      const float *__restrict__ bias, int n_out, TileShape ts, int D, int H, int W, int relu,
                      void *__restrict__ yout) {
   extern __shared__ __align__(1024) unsigned char sm[];
-  __shared__ uint64_t loaded[kRingB], done[kRingB], box_full[kMaxBox][kMaxPlanes + 2], box_free[kMaxBox], fin;
+  __shared__ uint64_t loaded[kRingB], done[kRingB], box_full[kMaxBox][kMaxPlanes + 2], box_free[kMaxBox], acc_full[2],
+      acc_free[2], fin;
   __shared__ unsigned tslot;
-  __shared__ int okslot;
   __shared__ float sbias[kMaxN];
-  const int nt_n = ts.nt_n, gp = ts.gp, P = ts.planes, nbox = ts.nbox, npass = ts.npass;
+  const int nt_n = ts.nt_n, gp = ts.gp, P = ts.planes, nbox = ts.nbox, npass = ts.npass, nacc = ts.nacc;
   const int plane_bytes = kGroupBytes * gp, box_bytes = plane_bytes * (P + 2);
   const int t_bytes = nt_n * gp * 16;  // one tap's weights
   const int taps = ts.taps, ring = ts.ring, b_bytes = t_bytes * taps;
   unsigned char *sb = sm + nbox * box_bytes;
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-  const int ntx = (W + kTX - 1) / kTX;
-  const int x0 = (blockIdx.x % ntx) * kTX, y0 = (blockIdx.x / ntx) * kTY, z0 = blockIdx.y * P;
-  const int np = min(P, D - z0);  // planes of this block inside the grid
-  const int nt = blockIdx.z;
+  const int ntx = (W + kTX - 1) / kTX, txy = ntx * ((H + kTY - 1) / kTY), nz = (D + P - 1) / P;
   const unsigned lbo_b = (unsigned)(nt_n / 8) * 128u;
   const int per = 27 / taps, nch = npass * per;  // weight copies per pass, in all
+  // tile t of the grid: N tile, plane chunk, (x, y) tile
+  struct Tile {
+    int nt, z0, np, x0, y0;
+  };
+  auto tile_at = [&](int64_t t) {
+    const int xy = (int)(t % txy), zc = (int)(t / txy % nz);
+    return Tile{(int)(t / txy / nz), zc * P, min(P, D - zc * P), (xy % ntx) * kTX, (xy / ntx) * kTY};
+  };
 
   if (tid == 0) {
     for (int i = 0; i < kRingB; i++) {
       bar_init(&loaded[i]);
-      bar_init(&done[i], np);
+      bar_init(&done[i], P);
     }
     for (int b = 0; b < nbox; b++) {
       for (int i = 0; i < P + 2; i++) bar_init(&box_full[b][i]);
-      bar_init(&box_free[b], np);
+      bar_init(&box_free[b], P);
     }
-    bar_init(&fin, np);
-    okslot = 1;
+    for (int i = 0; i < 2; i++) {
+      bar_init(&acc_full[i], P);
+      bar_init(&acc_free[i], 4);
+    }
+    bar_init(&fin, P);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  for (int i = tid; i < nt_n; i += kTileThreads) sbias[i] = bias && nt * nt_n + i < n_out ? __ldg(bias + nt * nt_n + i) : 0.f;
   if (warp == 0) tmem_alloc(&tslot, ts.cols);
   fence_before();
   __syncthreads();
@@ -349,135 +359,169 @@ __global__ void __launch_bounds__(kTileThreads)
   const unsigned tmem = tslot;
 
   const bool one = elect_one();
-  if (warp == 4 && one) {  // copies: the planes' boxes pass by pass, the weight chunks in order
-    const uint16_t *wt = wpack + (int64_t)nt * nch * (b_bytes / 2);
-    auto issue_box = [&](int ps) {
-      const int b = ps % nbox;
-      for (int k = 0; k < np + 2; k++) {
-        const int i = BWD ? np + 1 - k : k;  // in the order the taps need them
-        bar_expect(&box_full[b][i], plane_bytes);
-        tma_box(sm + b * box_bytes + i * plane_bytes, &tm, x0, y0, z0 - 1 + i, ps * gp, &box_full[b][i]);
-      }
-    };
+  if (warp == 4 && one) {  // copies: the planes' boxes pass by pass, the weight copies in order
     bool ok = true;
-    int boxes = 0, c = 0;
-    for (; boxes < nbox && boxes < npass; boxes++) issue_box(boxes);
-    for (; c < nch && ok; c++) {
-      if (c % per == 0 && c > 0 && boxes < npass && boxes < c / per + nbox) {
-        // the buffer of pass boxes - nbox is free once that pass's MMAs have run
-        ok = bar_wait(&box_free[boxes % nbox], ((boxes / nbox) - 1) & 1);
+    int it = 0, boxes = 0;  // tiles done, boxes issued (all passes of all tiles in order)
+    int64_t bt = blockIdx.x;  // tile and pass of the next box
+    int bp = 0;
+    auto issue_box = [&]() {
+      const Tile t = tile_at(bt);
+      const int b = boxes % nbox;
+      if (boxes >= nbox && !bar_wait(&box_free[b], ((boxes / nbox) - 1) & 1)) return false;
+      // planes past the grid read zero, and count towards the barriers of every box
+      for (int k = 0; k < P + 2; k++) {
+        const int i = BWD ? P + 1 - k : k;  // in the order the taps need them
+        bar_expect(&box_full[b][i], plane_bytes);
+        tma_box(sm + b * box_bytes + i * plane_bytes, &tm, t.x0, t.y0, t.z0 - 1 + i, bp * gp, &box_full[b][i]);
+      }
+      boxes++;
+      if (++bp == npass) {
+        bp = 0;
+        bt += gridDim.x;
+      }
+      return true;
+    };
+    int s = 0, c = 0;
+    unsigned turn = 1;  // a ring buffer's first use does not wait
+    for (int64_t t = blockIdx.x; t < ts.tiles && ok; t += gridDim.x, it++) {
+      const uint16_t *wt = wpack + (int64_t)tile_at(t).nt * nch * (b_bytes / 2);
+      for (int q = 0; q < nch && ok; q++, c++) {
+        if (q % per == 0)
+          while (ok && bt < ts.tiles && boxes < it * npass + q / per + nbox) ok = issue_box();
+        ok = ok && (c < ring || bar_wait(&done[s], turn));
         if (!ok) break;
-        issue_box(boxes++);
+        bar_expect(&loaded[s], b_bytes);
+        bulk_copy(sb + s * b_bytes, wt + (int64_t)q * (b_bytes / 2), b_bytes, &loaded[s]);
+        if (++s == ring) {
+          s = 0;
+          turn ^= 1u;
+        }
       }
-      const int s = c % ring;
-      if (c >= ring && !bar_wait(&done[s], ((c / ring) - 1) & 1)) {
-        ok = false;
-        break;
-      }
-      bar_expect(&loaded[s], b_bytes);
-      bulk_copy(sb + s * b_bytes, wt + (int64_t)c * (b_bytes / 2), b_bytes, &loaded[s]);
     }
     // every copy lands before the shared memory is released
-    for (int q = max(0, c - ring); q < c; q++) ok = bar_wait(&loaded[q % ring], (q / ring) & 1) && ok;
+    for (int q = max(0, c - ring); q < c; q++) bar_wait(&loaded[q % ring], (q / ring) & 1);
     for (int q = max(0, boxes - nbox); q < boxes; q++)
-      for (int i = 0; i < np + 2; i++) ok = bar_wait(&box_full[q % nbox][i], (q / nbox) & 1) && ok;
-    if (!ok) atomicExch(&okslot, 0);
-  } else if (warp < np && one) {  // MMAs of plane `warp`
+      for (int i = 0; i < P + 2; i++) bar_wait(&box_full[q % nbox][i], (q / nbox) & 1);
+  } else if (warp < P && one) {  // MMAs of plane `warp`
     const uint32_t idesc = instr_desc(nt_n);
-    const unsigned d = tmem + (unsigned)(warp * nt_n);
     const unsigned ahi = (unsigned)(smem_desc(0, kGroupBytes, kRowBytes) >> 32), bhi = (unsigned)(smem_desc(0, lbo_b, 128) >> 32);
     const unsigned blo = (unsigned)smem_desc(su32(sb), lbo_b, 128), bj = (2 * lbo_b) >> 4;
     bool ok = true;
-    int s = 0, tc = 0;
-    unsigned turn = 0, acc = 0;  // ring buffer and its phase; 0 for the accumulator's first MMA
-    for (int ps = 0; ps < npass && ok; ps++) {
-      const int b = ps % nbox;
-      const unsigned ph = (ps / nbox) & 1;
-      const unsigned box = (unsigned)smem_desc(su32(sm + b * box_bytes + warp * plane_bytes), kGroupBytes, kRowBytes);
-      // the taps of the pass with JN group pairs
-      auto run = [&](auto pairs) {
-        constexpr int JN = decltype(pairs)::value;
-        for (int r = 0; r < 9; r++) {  // (kz, ky): three taps
-          // the tap's shift, mirrored in the backward pass
-          const int sz = BWD ? 2 - r / 3 : r / 3, sy = BWD ? 2 - r % 3 : r % 3;
-          if (r % 3 == 0) ok = bar_wait(&box_full[b][warp + sz], ph);
-          const unsigned al = box + (((unsigned)sz * plane_bytes + (unsigned)sy * kRowBytes) >> 4);
+    int s = 0, tc = 0, it = 0, box_n = 0;
+    unsigned turn = 0;  // phase of the ring buffer
+    for (int64_t t = blockIdx.x; t < ts.tiles && ok; t += gridDim.x, it++) {
+      const bool live = warp < tile_at(t).np;  // a plane past the grid keeps the barriers only
+      const int as = it % nacc;
+      if (it >= nacc) ok = bar_wait(&acc_free[as], ((it / nacc) - 1) & 1);
+      fence_after();
+      const unsigned d = tmem + (unsigned)((as * P + warp) * nt_n);
+      unsigned acc = 0;  // 0 for the accumulator's first MMA
+      for (int ps = 0; ps < npass && ok; ps++, box_n++) {
+        const int b = box_n % nbox;
+        const unsigned ph = (box_n / nbox) & 1;
+        const unsigned box = (unsigned)smem_desc(su32(sm + b * box_bytes + warp * plane_bytes), kGroupBytes, kRowBytes);
+        // the taps of the pass with JN group pairs
+        auto run = [&](auto pairs) {
+          constexpr int JN = decltype(pairs)::value;
+          for (int r = 0; r < 9; r++) {  // (kz, ky): three taps
+            // the tap's shift, mirrored in the backward pass
+            const int sz = BWD ? 2 - r / 3 : r / 3, sy = BWD ? 2 - r % 3 : r % 3;
+            if (r % 3 == 0) ok = bar_wait(&box_full[b][warp + sz], ph);
+            const unsigned al = box + (((unsigned)sz * plane_bytes + (unsigned)sy * kRowBytes) >> 4);
 #pragma unroll
-          for (int kx = 0; kx < 3; kx++) {
-            if (tc == 0) ok = ok && bar_wait(&loaded[s], turn);
-            if (!ok) return;
-            fence_after();
-            const unsigned bl = blo + ((unsigned)(s * b_bytes + tc * t_bytes) >> 4);
+            for (int kx = 0; kx < 3; kx++) {
+              if (tc == 0) ok = ok && bar_wait(&loaded[s], turn);
+              if (!ok) return;
+              fence_after();
+              const unsigned bl = blo + ((unsigned)(s * b_bytes + tc * t_bytes) >> 4);
+              if (live) {
 #pragma unroll
-            for (int j = 0; j < JN; j++) {
-              mma_ss(d, al + (BWD ? 2 - kx : kx) + j * ((2 * kGroupBytes) >> 4), ahi, bl + j * bj, bhi, idesc, acc);
-              acc = 1u;
-            }
-            if (++tc == taps) {
-              mma_commit(&done[s]);
-              tc = 0;
-              if (++s == ring) {
-                s = 0;
-                turn ^= 1u;
+                for (int j = 0; j < JN; j++) {
+                  mma_ss(d, al + (BWD ? 2 - kx : kx) + j * ((2 * kGroupBytes) >> 4), ahi, bl + j * bj, bhi, idesc, acc);
+                  acc = 1u;
+                }
+              }
+              if (++tc == taps) {
+                mma_commit(&done[s]);
+                tc = 0;
+                if (++s == ring) {
+                  s = 0;
+                  turn ^= 1u;
+                }
               }
             }
           }
+          mma_commit(&box_free[b]);
+        };
+        switch (min(gp, ts.G - ps * gp) / 2) {
+          case 1: run(std::integral_constant<int, 1>{}); break;
+          case 2: run(std::integral_constant<int, 2>{}); break;
+          case 3: run(std::integral_constant<int, 3>{}); break;
+          case 4: run(std::integral_constant<int, 4>{}); break;
+          case 5: run(std::integral_constant<int, 5>{}); break;
+          default: run(std::integral_constant<int, 6>{});
         }
-        mma_commit(&box_free[b]);
-      };
-      switch (min(gp, ts.G - ps * gp) / 2) {
-        case 1: run(std::integral_constant<int, 1>{}); break;
-        case 2: run(std::integral_constant<int, 2>{}); break;
-        case 3: run(std::integral_constant<int, 3>{}); break;
-        case 4: run(std::integral_constant<int, 4>{}); break;
-        case 5: run(std::integral_constant<int, 5>{}); break;
-        default: run(std::integral_constant<int, 6>{});
       }
+      if (ok) mma_commit(&acc_full[as]);
     }
     mma_commit(&fin);
-    if (!bar_wait(&fin, 0)) ok = false;
-    if (!ok) atomicExch(&okslot, 0);
-  }
-  __syncthreads();
-  const bool ok = *(volatile int *)&okslot != 0;
-  fence_after();
-  // epilogue: warp q reads TMEM lanes 32 q .. 32 q + 31 (tile rows 4 q .. 4 q + 3)
-  const int m = warp * 32 + lane;
-  const int ox = x0 + (m & 7), oy = y0 + (m >> 3);
-  const bool in = ox < W && oy < H;
-  const int64_t nv = (int64_t)D * H * W;
-  using Out = typename std::conditional<BWD, float, uint16_t>::type;
-  if (warp < 4)
-    for (int p = 0; p < np; p++) {
-      Out *o = static_cast<Out *>(yout) + (int64_t)nt * nt_n * nv + ((int64_t)(z0 + p) * H + oy) * W + ox;
-      for (int c0 = 0; c0 < nt_n; c0 += 16) {
-        uint32_t r[16];
-        tmem_ld16(r, tmem + ((unsigned)(warp * 32) << 16) + (unsigned)(p * nt_n + c0));
-        const int nc = min(16, n_out - nt * nt_n - c0);
-        Out v[16];
-#pragma unroll
-        for (int j = 0; j < 16; j++) {
-          if constexpr (BWD) {
-            v[j] = ok ? __uint_as_float(r[j]) : __uint_as_float(0x7FC00000u);
-          } else {
-            float f = __uint_as_float(r[j]) + sbias[c0 + j];
-            if (relu) f = fmaxf(f, 0.f);
-            v[j] = ok ? __bfloat16_as_ushort(__float2bfloat16_rn(f)) : (uint16_t)0x7FC0;
-          }
-        }
-        if (in) {
-          if (nc == 16) {
-#pragma unroll
-            for (int j = 0; j < 16; j++) o[j * nv] = v[j];
-          } else {
-#pragma unroll
-            for (int j = 0; j < 16; j++)
-              if (j < nc) o[j * nv] = v[j];
-          }
-        }
-        o += 16 * nv;
+    bar_wait(&fin, 0);
+  } else if (warp > 4) {  // results: warp q reads TMEM lanes 32 q .. 32 q + 31 (tile rows 4 q .. 4 q + 3)
+    const int quad = warp & 3, m = quad * 32 + lane;
+    const int64_t nv = (int64_t)D * H * W;
+    using Out = typename std::conditional<BWD, float, uint16_t>::type;
+    bool ok = true;
+    int it = 0, bias_nt = -1;
+    for (int64_t t = blockIdx.x; t < ts.tiles; t += gridDim.x, it++) {
+      const Tile tl = tile_at(t);
+      const int as = it % nacc;
+      if (tl.nt != bias_nt) {
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        for (int i = tid - 160; i < nt_n; i += 128)
+          sbias[i] = bias && tl.nt * nt_n + i < n_out ? __ldg(bias + tl.nt * nt_n + i) : 0.f;
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        bias_nt = tl.nt;
       }
+      // once a wait gave up, this and the block's later tiles get NaN
+      ok = ok && __all_sync(0xffffffffu, bar_wait(&acc_full[as], (it / nacc) & 1));
+      fence_after();
+      const int ox = tl.x0 + (m & 7), oy = tl.y0 + (m >> 3);
+      const bool in = ox < W && oy < H;
+      for (int p = 0; p < tl.np; p++) {
+        Out *o = static_cast<Out *>(yout) + (int64_t)tl.nt * nt_n * nv + ((int64_t)(tl.z0 + p) * H + oy) * W + ox;
+        for (int c0 = 0; c0 < nt_n; c0 += 16) {
+          uint32_t r[16];
+          tmem_ld16(r, tmem + ((unsigned)(quad * 32) << 16) + (unsigned)((as * P + p) * nt_n + c0));
+          const int nc = min(16, n_out - tl.nt * nt_n - c0);
+          Out v[16];
+#pragma unroll
+          for (int j = 0; j < 16; j++) {
+            if constexpr (BWD) {
+              v[j] = ok ? __uint_as_float(r[j]) : __uint_as_float(0x7FC00000u);
+            } else {
+              float f = __uint_as_float(r[j]) + sbias[c0 + j];
+              if (relu) f = fmaxf(f, 0.f);
+              v[j] = ok ? __bfloat16_as_ushort(__float2bfloat16_rn(f)) : (uint16_t)0x7FC0;
+            }
+          }
+          if (in) {
+            if (nc == 16) {
+#pragma unroll
+              for (int j = 0; j < 16; j++) o[j * nv] = v[j];
+            } else {
+#pragma unroll
+              for (int j = 0; j < 16; j++)
+                if (j < nc) o[j * nv] = v[j];
+            }
+          }
+          o += 16 * nv;
+        }
+      }
+      fence_before();
+      __syncwarp();
+      if (lane == 0) bar_arrive(&acc_free[as]);
     }
+  }
   fence_before();
   __syncthreads();
   if (warp == 0) tmem_free(tmem, ts.cols);
@@ -511,45 +555,54 @@ bool tile_shape(int n_rows, int groups, int64_t tiles_xy, int D, TileShape *out)
   const int npass = ts.npass = (ts.G + gp - 1) / gp;
   double best = 0;
   for (int planes : {4, 2, 1})
-    for (int nbox = 1; nbox <= (npass > 1 ? kMaxBox : 1); nbox++)
-      for (int taps : {9, 3, 1})
-        for (int ring = 2; ring <= kRingB; ring++) {
-          if (planes * ts.nt_n > kTmemCols) continue;
-          const int cols = pow2_cols(planes * ts.nt_n);
-          const int box = kGroupBytes * gp * (planes + 2), copy = taps * ts.nt_n * gp * 16;
-          int smem = nbox * box + ring * copy;
-          if (smem > kSmBlock) continue;
-          // the shared memory keeps the blocks an SM can hold within its TMEM columns, so an
-          // allocation never waits
-          const int floor_smem = kSmPerSM / (kTmemCols / cols + 1) - 1024 + 16;
-          if (smem < floor_smem) smem = floor_smem;
-          const int occ = std::min(kTmemCols / cols, kSmPerSM / (smem + 2560));
-          // a model in SM clocks: an MMA of M = 128, K = 16 reads 4 KB of A and 32 nt_n bytes of B
-          // at 128 B per clock or computes nt_n / 2 clocks (both measured); a weight copy takes
-          // about 1500 clocks of latency and 24 B per clock and SM; the first planes, the gaps
-          // between passes with one box buffer and the epilogue are hidden only by the SM's other
-          // blocks
-          const double one = std::max(32.0 + ts.nt_n / 4.0, ts.nt_n / 2.0);
-          const double mma = 27.0 * (ts.G / 2) * planes * one;                    // tensor pipe
-          const double chain = 27.0 * (ts.G / 2) * std::max(planes * one, 110.0);  // issue of one warp
-          const double trip = 27.0 * npass / taps * (1500.0 + copy / 24.0) / (ring - 1);
-          const double body = std::max(chain, trip);
-          const double extra = 2500.0 + box / 30.0 * (nbox == 1 ? npass : 1) * 0.5 + 12.0 * planes * ts.nt_n;
-          const double blocks = (double)tiles_xy * ((D + planes - 1) / planes) * ts.ntiles;
-          const double waves = std::ceil(blocks / (kSms * (double)occ));
-          const double l2 = occ * 27.0 * ts.G * 16 * ts.nt_n / 24.0;  // weights of all blocks of the SM
-          const double cost = waves * std::max(std::max(occ * mma, l2), body + extra);
-          if (best == 0 || cost < best) {
-            best = cost;
-            ts.planes = planes;
-            ts.nbox = nbox;
-            ts.taps = taps;
-            ts.ring = ring;
-            ts.cols = cols;
-            ts.smem = smem;
-            *out = ts;
+    for (int nacc : {2, 1})
+      for (int nbox = 1; nbox <= kMaxBox; nbox++)
+        for (int taps : {9, 3, 1})
+          for (int ring = 2; ring <= kRingB; ring++) {
+            if (nacc * planes * ts.nt_n > kTmemCols) continue;
+            const int cols = pow2_cols(nacc * planes * ts.nt_n);
+            const int box = kGroupBytes * gp * (planes + 2), copy = taps * ts.nt_n * gp * 16;
+            int smem = nbox * box + ring * copy;
+            if (smem > kSmBlock) continue;
+            // the shared memory keeps the blocks an SM can hold within its TMEM columns, so an
+            // allocation never waits
+            const int floor_smem = kSmPerSM / (kTmemCols / cols + 1) - 1024 + 16;
+            if (smem < floor_smem) smem = floor_smem;
+            const int occ = std::min({kTmemCols / cols, kSmPerSM / (smem + 2560), 65536 / (kTileThreads * 64)});
+            const int64_t tiles = tiles_xy * ((D + planes - 1) / planes) * ts.ntiles;
+            // a model in SM clocks: an MMA of M = 128, K = 16 reads 4 KB of A and 32 nt_n bytes of B
+            // at 128 B per clock or computes nt_n / 2 clocks, and its issue takes about 110 clocks of
+            // its warp (all measured); a weight copy takes about 1500 clocks of latency and 24 B per
+            // clock and SM; the epilogue, about 60 clocks per column, runs beside the next tile's MMAs
+            // with two accumulator sets; a box's load runs beside the MMAs before it with two buffers;
+            // else only the SM's other blocks hide them
+            const double one = std::max(32.0 + ts.nt_n / 4.0, ts.nt_n / 2.0);
+            const double mma = 27.0 * (ts.G / 2) * planes * one;                     // tensor pipe
+            const double chain = 27.0 * (ts.G / 2) * std::max(planes * one, 110.0);  // issue of one warp
+            const double trip = 27.0 * npass / taps * (1500.0 + copy / 24.0) / (ring - 1);
+            const double body = std::max(chain, trip);
+            const double load = 1500.0 + box / 30.0 * 0.5, epi = 500.0 + 60.0 * planes * ts.nt_n;
+            const double l2 = 27.0 * ts.G * 16 * ts.nt_n / 24.0;
+            const double turns = std::ceil(tiles / (kSms * (double)occ));               // tiles per block
+            const double share = std::min((double)occ, std::ceil(tiles / (double)kSms));  // blocks on an SM
+            // one block's time per tile, or the SM's pipes shared by its blocks
+            const double each = std::max(body + (nbox == 1 ? npass * load : 0.0), share * std::max(mma, l2));
+            const double cost = (nbox == 1 ? 0.0 : load) +
+                                (nacc == 2 ? turns * std::max(each, epi) + epi : turns * (each + epi));
+            if (best == 0 || cost < best) {
+              best = cost;
+              ts.planes = planes;
+              ts.nacc = nacc;
+              ts.nbox = nbox;
+              ts.taps = taps;
+              ts.ring = ring;
+              ts.cols = cols;
+              ts.smem = smem;
+              ts.tiles = tiles;
+              ts.grid = (int)std::min<int64_t>(tiles, (int64_t)kSms * occ);
+              *out = ts;
+            }
           }
-        }
   return best > 0;
 }
 
@@ -584,8 +637,7 @@ cudaError_t run_tile(const uint16_t *w, const float *b, int n_rows, int n_red, i
     tile_pack_kernel<<<blocks_x((int64_t)pack_elems, 256, 4096), 256, 0, s>>>(w, n_rows, n_red, cop, BWD, ts.nt_n, ts.gp,
                                                                               ts.npass, ts.ntiles, wp);
     prepare(src, ts.G);
-    tile_conv_kernel<BWD><<<dim3((unsigned)tiles_xy, (unsigned)((D + ts.planes - 1) / ts.planes), (unsigned)ts.ntiles),
-                            kTileThreads, ts.smem, s>>>(tm, wp, b, n_rows, ts, D, H, W, relu, y);
+    tile_conv_kernel<BWD><<<ts.grid, kTileThreads, ts.smem, s>>>(tm, wp, b, n_rows, ts, D, H, W, relu, y);
     e = cudaGetLastError();
   }
   const cudaError_t f = cudaFreeAsync(buf, s);
