@@ -188,7 +188,7 @@ __device__ __forceinline__ float2 stage2(const StageArgs &a, float2 x, float2 y,
   if constexpr (MODE == 0) return r;
   if constexpr (MODE == 1) return pfma(bc(a.cdt), r, y);
   if constexpr (MODE == 2) return pfma(bc(a.cdt), r, x);
-  return pfma(bc(1.f / 3.f), padd(x, y), pmul(bc(a.cdt), r));
+  return pfma(bc(a.cdt), r, pmul(padd(x, y), bc(1.f / 3.f)));  // the third rounded by itself, as in fwi_internal.h
 }
 // the step-start values of three variables from field f on, loaded together: a.out may be a.X, so
 // the compiler keeps these loads behind the stores of the variables before, and each group waits
