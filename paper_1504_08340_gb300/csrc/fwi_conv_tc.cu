@@ -176,42 +176,45 @@ __device__ __forceinline__ uint4 pack8(const uint16_t h[8]) {
                     (uint32_t)h[4] | (uint32_t)h[5] << 16, (uint32_t)h[6] | (uint32_t)h[7] << 16);
 }
 
-// src[g][p][e] = x[8 g + e][p] (zero for channels >= cin)
-__global__ void __launch_bounds__(256) to_group_major(const uint16_t *__restrict__ x, int64_t nv, int cin,
-                                                      uint16_t *__restrict__ src) {
-  const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  const int g = blockIdx.y;
-  if (p >= nv) return;
-  const uint16_t *q = x + 8 * g * nv + p;
-  uint32_t v[4] = {0u, 0u, 0u, 0u};
+// The copies that a convolution needs before its MMAs are one launch: its blocks share out the
+// source's and the weights' (or the gradient's) part. At 17 x 33 x 33 voxels, where each of them
+// takes 2 to 4 us, launches of their own took 8 % of a training sample (1000 against 920 us).
+
+// src[g][p][e] = x[8 g + e][p] (zero for channels >= cin), g = block / nx
+__device__ __forceinline__ void group_major_block(const uint16_t *__restrict__ x, int64_t nv, int cin,
+                                                  uint16_t *__restrict__ src, int block, int nx) {
+  const int g = block / nx;
   const int n = cin - 8 * g;
+  for (int64_t p = (int64_t)(block - g * nx) * 256 + threadIdx.x; p < nv; p += (int64_t)nx * 256) {
+    const uint16_t *q = x + 8 * g * nv + p;
+    uint32_t v[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-  for (int e = 0; e < 8; e++)
-    if (e < n) v[e >> 1] |= (uint32_t)__ldg(q + e * nv) << (16 * (e & 1));
-  *reinterpret_cast<uint4 *>(src + ((int64_t)g * nv + p) * 8) = make_uint4(v[0], v[1], v[2], v[3]);
+    for (int e = 0; e < 8; e++)
+      if (e < n) v[e >> 1] |= (uint32_t)__ldg(q + e * nv) << (16 * (e & 1));
+    *reinterpret_cast<uint4 *>(src + ((int64_t)g * nv + p) * 8) = make_uint4(v[0], v[1], v[2], v[3]);
+  }
 }
 
 // the split gradient in group-major form: channel s cop + co of src is part s of dy[co], cop
 // the channels rounded up to 8; zero for co >= cout and for groups past 3 cop / 8. A thread
-// reads 8 channels of a voxel once and writes their three parts.
-__global__ void split_group_major(const float *__restrict__ dy, int64_t nv, int cout, int cop, int G,
-                                  uint16_t *__restrict__ src) {
-  const int gq = cop / 8;
-  for (int g = blockIdx.y; g < gq; g += gridDim.y)
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nv; p += (int64_t)gridDim.x * blockDim.x) {
-      uint16_t h[3][8];
+// reads 8 channels of a voxel once and writes their three parts. g = block / nx of cop / 8.
+__device__ __forceinline__ void split_group_block(const float *__restrict__ dy, int64_t nv, int cout, int cop, int G,
+                                                  uint16_t *__restrict__ src, int block, int nx) {
+  const int gq = cop / 8, g = block / nx;
+  for (int64_t p = (int64_t)(block - g * nx) * 256 + threadIdx.x; p < nv; p += (int64_t)nx * 256) {
+    uint16_t h[3][8];
 #pragma unroll
-      for (int e = 0; e < 8; e++) {
-        uint16_t t[3];
-        split3(8 * g + e < cout ? __ldg(dy + (int64_t)(8 * g + e) * nv + p) : 0.f, t);
+    for (int e = 0; e < 8; e++) {
+      uint16_t t[3];
+      split3(8 * g + e < cout ? __ldg(dy + (int64_t)(8 * g + e) * nv + p) : 0.f, t);
 #pragma unroll
-        for (int s = 0; s < 3; s++) h[s][e] = t[s];
-      }
-#pragma unroll
-      for (int s = 0; s < 3; s++) *reinterpret_cast<uint4 *>(src + ((int64_t)(s * gq + g) * nv + p) * 8) = pack8(h[s]);
-      if (g == 0)
-        for (int z = 3 * gq; z < G; z++) *reinterpret_cast<uint4 *>(src + ((int64_t)z * nv + p) * 8) = make_uint4(0u, 0u, 0u, 0u);
+      for (int s = 0; s < 3; s++) h[s][e] = t[s];
     }
+#pragma unroll
+    for (int s = 0; s < 3; s++) *reinterpret_cast<uint4 *>(src + ((int64_t)(s * gq + g) * nv + p) * 8) = pack8(h[s]);
+    if (g == 0)
+      for (int z = 3 * gq; z < G; z++) *reinterpret_cast<uint4 *>(src + ((int64_t)z * nv + p) * 8) = make_uint4(0u, 0u, 0u, 0u);
+  }
 }
 
 // cuTensorMapEncodeTiled from the driver, looked up once through the runtime
@@ -280,31 +283,42 @@ struct TileShape {
 };
 
 // weight chunks: for N tile nt, pass ps, tap t: nt_n x (gp x 8) K-major, core (kg, ng) at
-// kg * (nt_n / 8) * 128 + ng * 128. Source channel c = 8 (ps gp + kg) + kk; forward: w[n][c][t];
-// backward: c = s cop + co, w[co][n][t]
-__global__ void tile_pack_kernel(const uint16_t *__restrict__ w, int n_rows, int n_red, int cop, bool bwd, int nt_n,
-                                 int gp, int npass, int ntiles, uint16_t *__restrict__ out) {
-  const int64_t chunk = (int64_t)nt_n * gp * 8;
-  const int64_t total = (int64_t)ntiles * npass * 27 * chunk;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int q = (int)(i / chunk);  // (tile, pass, tap)
-    const int e = (int)(i % chunk);
-    const int kk = e & 7, row = (e >> 3) & 7, r = e >> 6;
-    const int ng = r % (nt_n / 8), kg = r / (nt_n / 8);
-    const int t = q % 27, ps = q / 27 % npass, nt = q / 27 / npass;
-    const int n = nt * nt_n + ng * 8 + row;
-    const int c = 8 * (ps * gp + kg) + kk;
-    uint16_t v = 0;
-    if (n < n_rows) {
-      if (!bwd) {
-        if (c < n_red) v = w[((int64_t)n * n_red + c) * 27 + t];
+// kg * (nt_n / 8) * 128 + ng * 128, i.e. 16 bytes (8 source channels) per (kg, n) in order.
+// Source channel c = 8 (ps gp + kg) + kk; forward: w[n][c][t]; backward: c = s cop + co, w[co][n][t]
+template <bool BWD>
+__device__ __forceinline__ void pack_block(const uint16_t *__restrict__ w, int n_rows, int n_red, int cop, const TileShape &ts,
+                                           uint16_t *__restrict__ out, int block, int nblocks) {
+  const int64_t total = (int64_t)ts.ntiles * ts.npass * 27 * ts.gp * ts.nt_n;
+  for (int64_t i = (int64_t)block * 256 + threadIdx.x; i < total; i += (int64_t)nblocks * 256) {
+    const int r = (int)(i / ts.nt_n), q = r / ts.gp;  // (tile, pass, tap, kg), (tile, pass, tap)
+    const int kg = r - q * ts.gp, t = q % 27, ps = q / 27 % ts.npass, nt = q / 27 / ts.npass;
+    const int n = nt * ts.nt_n + (int)(i - (int64_t)r * ts.nt_n), c0 = 8 * (ps * ts.gp + kg);
+    uint16_t h[8];
+#pragma unroll
+    for (int kk = 0; kk < 8; kk++) {
+      const int c = c0 + kk;
+      if (!BWD) {
+        h[kk] = n < n_rows && c < n_red ? __ldg(w + ((int64_t)n * n_red + c) * 27 + t) : (uint16_t)0;
       } else {
-        const int part = c / cop, co = c % cop;
-        if (part < 3 && co < n_red) v = w[((int64_t)co * n_rows + n) * 27 + t];
+        const int part = c / cop, co = c - part * cop;
+        h[kk] = n < n_rows && part < 3 && co < n_red ? __ldg(w + ((int64_t)co * n_rows + n) * 27 + t) : (uint16_t)0;
       }
     }
-    out[i] = v;
+    *reinterpret_cast<uint4 *>(out + i * 8) = pack8(h);
   }
+}
+
+// the copies of a forward (x) or backward-data (dy) convolution: blocks below nsrc the source,
+// the others the weights
+template <bool BWD>
+__global__ void __launch_bounds__(256) tile_prep_kernel(const void *__restrict__ in, int64_t nv, int n_red, int cop,
+                                                        const uint16_t *__restrict__ w, int n_rows, TileShape ts,
+                                                        uint16_t *__restrict__ src, uint16_t *__restrict__ wp, int nx,
+                                                        int nsrc) {
+  const int b = blockIdx.x;
+  if (b >= nsrc) pack_block<BWD>(w, n_rows, n_red, cop, ts, wp, b - nsrc, gridDim.x - nsrc);
+  else if (BWD) split_group_block(static_cast<const float *>(in), nv, n_red, cop, ts.G, src, b, nx);
+  else group_major_block(static_cast<const uint16_t *>(in), nv, n_red, src, b, nx);
 }
 
 template <bool BWD>
@@ -613,11 +627,11 @@ unsigned blocks_x(int64_t n, int threads, int64_t most) {
 
 size_t align256(size_t n) { return (n + 255) / 256 * 256; }
 
-// the tile form over a group-major source that `prepare` fills; n_rows GEMM output channels,
-// n_red real source channels (forward: cin; backward: cout, with cop = the part stride)
-template <bool BWD, class Prepare>
-cudaError_t run_tile(const uint16_t *w, const float *b, int n_rows, int n_red, int cop, int groups, int D, int H, int W,
-                     int relu, void *y, cudaStream_t s, Prepare prepare) {
+// the tile form of the forward (x) or backward-data (dy) convolution of `in`; n_rows GEMM output
+// channels, n_red real source channels (forward: cin; backward: cout, with cop = the part stride)
+template <bool BWD>
+cudaError_t run_tile(const void *in, const uint16_t *w, const float *b, int n_rows, int n_red, int cop, int groups, int D,
+                     int H, int W, int relu, void *y, cudaStream_t s) {
   const int64_t nv = (int64_t)D * H * W;
   const int64_t tiles_xy = (int64_t)((W + kTX - 1) / kTX) * ((H + kTY - 1) / kTY);
   TileShape ts;
@@ -634,9 +648,9 @@ cudaError_t run_tile(const uint16_t *w, const float *b, int n_rows, int n_red, i
   CUtensorMap tm;
   e = box_map(&tm, src, D, H, W, ts.G, ts.gp);
   if (e == cudaSuccess) {
-    tile_pack_kernel<<<blocks_x((int64_t)pack_elems, 256, 4096), 256, 0, s>>>(w, n_rows, n_red, cop, BWD, ts.nt_n, ts.gp,
-                                                                              ts.npass, ts.ntiles, wp);
-    prepare(src, ts.G);
+    const unsigned nx = blocks_x(nv, 256, 65536), nsrc = nx * (unsigned)(BWD ? cop / 8 : ts.G);
+    const unsigned npack = blocks_x((int64_t)pack_elems / 8, 256, 4096);
+    tile_prep_kernel<BWD><<<nsrc + npack, 256, 0, s>>>(in, nv, n_red, cop, w, n_rows, ts, src, wp, (int)nx, (int)nsrc);
     tile_conv_kernel<BWD><<<ts.grid, kTileThreads, ts.smem, s>>>(tm, wp, b, n_rows, ts, D, H, W, relu, y);
     e = cudaGetLastError();
   }
@@ -671,10 +685,9 @@ constexpr int kWorkSlice = 2048;    // voxels per slice the size of `work` is co
 // (channel mt cm + c), per voxel tile and tile row; zero outside the grid and past cout. A
 // block turns one tile of up to 32 channels through shared memory, so that both its reads
 // (8 voxels of a row) and its writes (16 bytes of consecutive channels) are contiguous.
-__global__ void __launch_bounds__(256) split_tiles(const float *__restrict__ dy, int cout, int cm, int ntx, int nty, int D,
-                                                   int H, int W, uint16_t *__restrict__ dyt) {
+__device__ __forceinline__ void split_tile_block(const float *__restrict__ dy, int cout, int cm, int ntx, int nty, int ntile,
+                                                 int D, int H, int W, uint16_t *__restrict__ dyt, int tile, int mt, int c0) {
   __shared__ float st[32][kM + 1];
-  const int tile = blockIdx.x, mt = blockIdx.z, c0 = blockIdx.y * 32;  // channel chunk of the M tile
   const int x0 = tile % ntx * kTX, y0 = tile / ntx % nty * kTY, z = tile / ntx / nty;
   const int nc = min(32, cm - c0);
   for (int i = threadIdx.x; i < nc * kM; i += 256) {
@@ -682,7 +695,7 @@ __global__ void __launch_bounds__(256) split_tiles(const float *__restrict__ dy,
     st[c][v] = (co < cout && x < W && y < H) ? __ldg(dy + (((int64_t)co * D + z) * H + y) * W + x) : 0.f;
   }
   __syncthreads();
-  const int64_t base = ((int64_t)mt * gridDim.x + tile) * kTY * (3 * cm);
+  const int64_t base = ((int64_t)mt * ntile + tile) * kTY * (3 * cm);
   for (int i = threadIdx.x; i < 32 * kTY; i += 256) {
     const int c = i & 31, y = i >> 5;
     if (c >= nc) continue;
@@ -707,6 +720,32 @@ struct WgShape {
   int slices, per;         // slices, tiles per slice
   int ring, smem;
 };
+
+// x alone, for grids where the two copies' own launches cost nothing: wgrad_prep_kernel's shared
+// memory leaves its x blocks fewer on an SM (65 x 129 x 129 voxels: 332 against 327 us a call)
+__global__ void __launch_bounds__(256) group_major_kernel(const uint16_t *__restrict__ x, int64_t nv, int cin,
+                                                          uint16_t *__restrict__ src, int nx) {
+  group_major_block(x, nv, cin, src, blockIdx.x, nx);
+}
+constexpr int64_t kPrepVoxels = 1 << 18;  // voxels up to which the two copies are one launch
+
+// the copies of a weight gradient: blocks below nsrc x, the others the gradient tiles
+__global__ void __launch_bounds__(256) wgrad_prep_kernel(const float *__restrict__ dy, const uint16_t *__restrict__ x,
+                                                         int64_t nv, int cin, int cout, WgShape g, int D, int H, int W,
+                                                         uint16_t *__restrict__ src, uint16_t *__restrict__ dyt, int nx,
+                                                         int nsrc) {
+  const int b = blockIdx.x;
+  if (b < nsrc) {
+    group_major_block(x, nv, cin, src, b, nx);
+    return;
+  }
+  const int chunks = (g.cm + 31) / 32;  // of 32 channels of an M tile
+  for (int64_t i = b - nsrc; i < (int64_t)g.tiles * chunks * g.mt; i += gridDim.x - nsrc) {
+    const int r = (int)(i / g.tiles);
+    __syncthreads();  // the tile before has been read
+    split_tile_block(dy, cout, g.cm, g.ntx, g.nty, g.tiles, D, H, W, dyt, (int)(i % g.tiles), r / chunks, r % chunks * 32);
+  }
+}
 
 template <int T>
 __global__ void __launch_bounds__(32 * (5 + T), 1)
@@ -896,20 +935,13 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float *__restri
 
 cudaError_t conv3d_forward_tc(const uint16_t *x, const uint16_t *w, const float *b, int cin, int cout, int D, int H,
                               int W, int relu, uint16_t *y, cudaStream_t s) {
-  const int64_t nv = (int64_t)D * H * W;
-  return run_tile<false>(w, b, cout, cin, 0, (cin + 7) / 8, D, H, W, relu, y, s, [&](uint16_t *src, int G) {
-    to_group_major<<<dim3((unsigned)((nv + 255) / 256), (unsigned)G), 256, 0, s>>>(x, nv, cin, src);
-  });
+  return run_tile<false>(x, w, b, cout, cin, 8, (cin + 7) / 8, D, H, W, relu, y, s);
 }
 
 cudaError_t conv3d_backward_data_tc(const float *dy, const uint16_t *w, int cin, int cout, int D, int H, int W,
                                     float *dx, cudaStream_t s) {
   const int cop = (cout + 7) / 8 * 8;
-  const int64_t nv = (int64_t)D * H * W;
-  return run_tile<true>(w, nullptr, cin, cout, cop, 3 * cop / 8, D, H, W, 0, dx, s, [&](uint16_t *src, int G) {
-    split_group_major<<<dim3(blocks_x(nv, 256, 65536), (unsigned)std::min(cop / 8, 65535)), 256, 0, s>>>(dy, nv, cout,
-                                                                                                        cop, G, src);
-  });
+  return run_tile<true>(dy, w, nullptr, cin, cout, cop, 3 * cop / 8, D, H, W, 0, dx, s);
 }
 
 // floats the caller's scratch holds: one 128-row-padded im2col row set per 2048 voxels and
@@ -969,9 +1001,12 @@ cudaError_t conv3d_backward_weight_tc(const float *dy, const uint16_t *x, int ci
   CUtensorMap tm;
   e = box_map(&tm, src, D, H, W, g.G, g.nt_n / 8);
   if (e == cudaSuccess) {
-    to_group_major<<<dim3((unsigned)((nv + 255) / 256), (unsigned)g.G), 256, 0, s>>>(x, nv, cin, src);
-    split_tiles<<<dim3((unsigned)tiles, (unsigned)((g.cm + 31) / 32), (unsigned)g.mt), 256, 0, s>>>(dy, cout, g.cm, g.ntx,
-                                                                                                  g.nty, D, H, W, dyt);
+    const unsigned nx = blocks_x(nv, 256, 65536), nsrc = nx * (unsigned)g.G;
+    const unsigned ntl = blocks_x((int64_t)g.tiles * ((g.cm + 31) / 32) * g.mt, 1, 1 << 30);
+    const bool apart = nv > kPrepVoxels;
+    if (apart) group_major_kernel<<<nsrc, 256, 0, s>>>(x, nv, cin, src, (int)nx);
+    wgrad_prep_kernel<<<(apart ? 0 : nsrc) + ntl, 256, 0, s>>>(dy, x, nv, cin, cout, g, D, H, W, src, dyt, (int)nx,
+                                                              apart ? 0 : (int)nsrc);
     kernel<<<dim3((unsigned)combos, (unsigned)g.slices), 32 * (5 + g.T), g.smem, s>>>(tm, dyt, g, D, cin, cout, part);
     wgrad_reduce_kernel<<<blocks_x((int64_t)cout * (27 * (int64_t)cin + 1), 32, 65536), 256, 0, s>>>(part, g.slices, cin,
                                                                                                   cout, dw, db);
