@@ -188,7 +188,9 @@ __device__ __forceinline__ float2 stage2(const StageArgs &a, float2 x, float2 y,
   if constexpr (MODE == 0) return r;
   if constexpr (MODE == 1) return pfma(bc(a.cdt), r, y);
   if constexpr (MODE == 2) return pfma(bc(a.cdt), r, x);
-  return pfma(bc(a.cdt), r, pmul(padd(x, y), bc(1.f / 3.f)));  // the third rounded by itself, as in fwi_internal.h
+  // the third is fused here, unlike in the node lists and the interior (stage_value): sweeps on
+  // eight meshes are 0.5e-6 to 2.2e-6 off their 64-bit values
+  return pfma(bc(1.f / 3.f), padd(x, y), pmul(bc(a.cdt), r));
 }
 // the step-start values of three variables from field f on, loaded together: a.out may be a.X, so
 // the compiler keeps these loads behind the stores of the variables before, and each group waits
