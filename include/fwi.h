@@ -271,11 +271,12 @@ fwi_status fwi_tune_shot_batch(fwi_ctx *ctx, int shot0, int nshots, int max_batc
                                int *chosen);
 
 /* Picks the launch shapes of the stage kernels by measurement: for each candidate (most
- * planes per block of the interior kernel, fewer where that fills the GPU better: 4, 8, 16, 32; node pairs per x segment of a PML warp
- * task: 16, 32) it times `steps` forward RK4 steps (1 <= steps < nsteps) of the first
- * shot batch of shots [shot0, shot0 + nshots), keeps the fastest for later calls and
- * returns it in chosen[0] (planes) and chosen[1] (pairs). The shapes change no node's
- * arithmetic: every result is bitwise the same with any of them. Not in the paper.
+ * planes per block of the interior kernel: 4, 8, 16, 32, fewer where that fills the GPU
+ * better; a quarter of the most node pairs per x segment of the PML kernel: 16, 32) it
+ * times `steps` forward RK4 steps (1 <= steps < nsteps) of the first shot batch of shots
+ * [shot0, shot0 + nshots), keeps the fastest for later calls and returns it in chosen[0]
+ * (planes) and chosen[1] (pairs). The shapes change no node's arithmetic: every result is
+ * bitwise the same with any of them. Not in the paper.
  * Errors: FWI_E_INVAL, FWI_E_STATE, FWI_E_CUDA. */
 fwi_status fwi_tune_tiles(fwi_ctx *ctx, int shot0, int nshots, int steps, int chosen[2]);
 
@@ -356,8 +357,8 @@ fwi_status fwi_set_graphs(fwi_ctx *ctx, int enable);
 /* Kernel timing: with enable = 1 every stage-kernel launch of later calls is
  * bracketed by CUDA events on the context's stream; fwi_get_timing returns the
  * summed device time (ms) and launch count of kernel class `which`
- * (0: RK stage kernels, 1: gradient kernel, 2: point-load / sampling kernels (none: the
- * stage kernels do both), 3: all kernels launched, time unset) since the last reset. */
+ * (0: RK stage kernels, 1: gradient kernel, 2: none; point loads and
+ * samples count in class 0), 3: all kernels launched, time unset) since the last reset. */
 fwi_status fwi_set_timing(fwi_ctx *ctx, int enable);
 fwi_status fwi_get_timing(fwi_ctx *ctx, int which, double *ms, int64_t *launches);
 fwi_status fwi_reset_timing(fwi_ctx *ctx);

@@ -533,8 +533,11 @@ __device__ __forceinline__ void face_write(const Geo &g, const StageArgs &a, con
   }
 }
 
+// Blocks per SM. Three variables' step-start values in flight (kXG) want 72 registers, 80 in
+// stage 4, which reads three step-start rows: 67.7 ms a 64x64x32 gradient against 71.0 ms at nine
+// blocks and one variable; 252.0 against 262.7 ms at 96x96x48, four shots.
 #ifndef FWI_PML_STAGE4_MINB
-#define FWI_PML_STAGE4_MINB 6  // stage 4 reads three step-start rows: 80 registers
+#define FWI_PML_STAGE4_MINB 6
 #endif
 #ifndef FWI_PML_MINB
 #define FWI_PML_MINB 7
