@@ -264,8 +264,9 @@ cudaError_t box_map(CUtensorMap *tm, uint16_t *src, int D, int H, int W, int G, 
 // any N); the epilogue's stores (8 voxels of a row per channel) overlap it only across the
 // blocks of an SM. Several planes share each weight copy and two of three halo planes: with
 // one plane a block, 28 -> 28 channels moved 90 KB through L2 per 128 voxels, 27 KB now.
-// Measured at 65 x 129 x 129 voxels: forward 28 -> 28 226 -> 142 us, backward data 28 -> 84
-// 1359 -> 546 us (one thread issuing for one plane a block before).
+// Measured at 65 x 129 x 129 voxels, whole calls with their copies: forward 28 -> 28 262 -> 143
+// us, backward data 28 -> 84 1600 -> 519 us (one thread issuing for one plane a block before).
+// ncu at 32 -> 32, forward: 112 us, tensor pipe 27 % (11 % before), 36 M warp instructions (87 M).
 constexpr int kTileThreads = 288;
 constexpr int kRingB = 4;      // most weight copies in flight
 constexpr int kMaxPlanes = 4;  // output planes of a block
