@@ -261,8 +261,8 @@ cudaError_t box_map(CUtensorMap *tm, uint16_t *src, int D, int H, int W, int G, 
 // the MMAs of plane p, and the four chains keep the tensor pipe fed. Warp 4 copies, warps 5 to 8 write the results.
 //
 // Bound: in the MMA phase the operands' shared-memory reads (M = 128, K = 16: 4 KB of A for
-// any N); the epilogue's stores (8 voxels of a row per channel) overlap it only across the
-// blocks of an SM. Several planes share each weight copy and two of three halo planes: with
+// any N); the epilogue's stores (8 voxels of a row per channel) overlap it across the blocks
+// of an SM and, with two accumulator sets, beside the next tile's MMAs. Several planes share each weight copy and two of three halo planes: with
 // one plane a block, 28 -> 28 channels moved 90 KB through L2 per 128 voxels, 27 KB now.
 // Measured at 65 x 129 x 129 voxels, whole calls with their copies: forward 28 -> 28 262 -> 143
 // us, backward data 28 -> 84 1600 -> 519 us (one thread issuing for one plane a block before).
