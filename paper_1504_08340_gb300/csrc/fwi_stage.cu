@@ -74,21 +74,34 @@ __device__ __forceinline__ Ax make_ax(int c, int n, int lo, int hi) {
 
 __device__ __forceinline__ int nrd(const Ax &a) { return (int)a.r0 + (a.ns == 2 ? (int)a.r1 : 0); }
 
+// A value of the stage input. RO: nothing writes it while the kernel runs (a launch per stage), so
+// it may come through the read-only path. The blocks of the persistent sweep write the next
+// stages' inputs within the launch, for which that path is not defined: there the loads are plain
+// ones, ordered by the grid barrier. Its buffers are picked by the stage, so the compiler is told
+// that they are in global memory (8x8x4 elements, a 100-step sweep: 7.18 ms as generic loads, 6.92 so).
+template <bool RO>
+__device__ __forceinline__ float ldy(const float *p) {
+  if constexpr (RO) return __ldg(p);
+  __builtin_assume(__isGlobal(p));
+  return *p;
+}
+
 // element-wise derivative (times h) of field f at index i along stride s, side type t
-__device__ __forceinline__ float dst(const float *__restrict__ f, int64_t i, int64_t s, int t) {
-  if (t == kC) return __ldg(f + i + s) - __ldg(f + i - s);
-  if (t == kL) return __ldg(f + i - 2 * s) - 4.f * __ldg(f + i - s) + 3.f * __ldg(f + i);
-  return -3.f * __ldg(f + i) + 4.f * __ldg(f + i + s) - __ldg(f + i + 2 * s);
+template <bool RO>
+__device__ __forceinline__ float dst(const float *f, int64_t i, int64_t s, int t) {
+  if (t == kC) return ldy<RO>(f + i + s) - ldy<RO>(f + i - s);
+  if (t == kL) return ldy<RO>(f + i - 2 * s) - 4.f * ldy<RO>(f + i - s) + 3.f * ldy<RO>(f + i);
+  return -3.f * ldy<RO>(f + i) + 4.f * ldy<RO>(f + i + s) - ldy<RO>(f + i + 2 * s);
 }
 
 // sum over the sides of `a` that are interior elements (all sides when all_sides)
-__device__ __forceinline__ float dsum(const float *__restrict__ f, int64_t i, int64_t s, const Ax &a,
-                                      bool all_sides) {
+template <bool RO>
+__device__ __forceinline__ float dsum(const float *f, int64_t i, int64_t s, const Ax &a, bool all_sides) {
   if (a.ns == 2 && (all_sides || (a.r0 && a.r1)))  // L + R in one 4-point stencil
-    return __ldg(f + i - 2 * s) - 4.f * __ldg(f + i - s) + 4.f * __ldg(f + i + s) - __ldg(f + i + 2 * s);
+    return ldy<RO>(f + i - 2 * s) - 4.f * ldy<RO>(f + i - s) + 4.f * ldy<RO>(f + i + s) - ldy<RO>(f + i + 2 * s);
   float v = 0.f;
-  if (all_sides || a.r0) v += dst(f, i, s, a.t0);
-  if (a.ns == 2 && !all_sides && a.r1) v += dst(f, i, s, a.t1);
+  if (all_sides || a.r0) v += dst<RO>(f, i, s, a.t0);
+  if (a.ns == 2 && !all_sides && a.r1) v += dst<RO>(f, i, s, a.t1);
   return v;
 }
 
@@ -118,20 +131,20 @@ __device__ __forceinline__ void write_hist(const Geo &g, const StageArgs &a, int
 // derivative along k (the set of interior elements is a product of side sets),
 //   sum sigma_jj = lam (nk nl d_j u_j + nl S_k u_k + nk S_l u_l) + 2 mu nk nl d_j u_j
 //   sum sigma_kj = mu (nk nl d_j u_k + nl S_k u_j),  sum sigma_lj = mu (nk nl d_j u_l + nk S_l u_j)
-template <int j>
-__device__ __forceinline__ void interior_line_point(const Geo &g, const float *__restrict__ U, int64_t q,
+template <bool RO, int j>
+__device__ __forceinline__ void interior_line_point(const Geo &g, const float *U, int64_t q,
                                                     const int64_t st[3], const int cq[3], int pt, const Ax ax[3],
                                                     float nk, float nl, bool all_sides, float &sj_, float &sk_,
                                                     float &sl_) {
   constexpr int k = (j + 1) % 3, l = (j + 2) % 3;
   const int64_t S = g.stride;
-  const float dj_j = dst(U + j * S, q, st[j], pt);
-  const float dj_k = dst(U + k * S, q, st[j], pt);
-  const float dj_l = dst(U + l * S, q, st[j], pt);
-  const float Sk_k = dsum(U + k * S, q, st[k], ax[k], all_sides);
-  const float Sk_j = dsum(U + j * S, q, st[k], ax[k], all_sides);
-  const float Sl_l = dsum(U + l * S, q, st[l], ax[l], all_sides);
-  const float Sl_j = dsum(U + j * S, q, st[l], ax[l], all_sides);
+  const float dj_j = dst<RO>(U + j * S, q, st[j], pt);
+  const float dj_k = dst<RO>(U + k * S, q, st[j], pt);
+  const float dj_l = dst<RO>(U + l * S, q, st[j], pt);
+  const float Sk_k = dsum<RO>(U + k * S, q, st[k], ax[k], all_sides);
+  const float Sk_j = dsum<RO>(U + j * S, q, st[k], ax[k], all_sides);
+  const float Sl_l = dsum<RO>(U + l * S, q, st[l], ax[l], all_sides);
+  const float Sl_j = dsum<RO>(U + j * S, q, st[l], ax[l], all_sides);
   const float lam = __ldg(g.lam_n + q), mu = __ldg(g.mu_n + q);
   const float n2 = nk * nl;
   sj_ = lam * (n2 * dj_j + nl * Sk_k + nk * Sl_l) + 2.f * mu * n2 * dj_j;
@@ -140,8 +153,8 @@ __device__ __forceinline__ void interior_line_point(const Geo &g, const float *_
 }
 
 // interior-element force (times 3 h^2 / (W detJ)) at a node, contribution of axis j
-template <int j>
-__device__ __forceinline__ void interior_force_axis(const Geo &g, const float *__restrict__ U, int64_t node,
+template <bool RO, int j>
+__device__ __forceinline__ void interior_force_axis(const Geo &g, const float *U, int64_t node,
                                                     const int c3[3], const int64_t st[3], const Ax ax[3],
                                                     bool all_sides, float f[3]) {
   constexpr int k = (j + 1) % 3, l = (j + 2) % 3;
@@ -164,7 +177,7 @@ __device__ __forceinline__ void interior_force_axis(const Geo &g, const float *_
       int cq[3] = {c3[0], c3[1], c3[2]};
       cq[j] += off;
       float a, b, c;
-      interior_line_point<j>(g, U, node + off * st[j], st, cq, point_type(p), ax, nk, nl, all_sides, a, b, c);
+      interior_line_point<RO, j>(g, U, node + off * st[j], st, cq, point_type(p), ax, nk, nl, all_sides, a, b, c);
       acc_j += cf * a;
       acc_k += cf * b;
       acc_l += cf * c;
@@ -179,8 +192,8 @@ __device__ __forceinline__ void interior_force_axis(const Geo &g, const float *_
 // line quadrature of the j-column of Sdot Le + S Lp + Sbar Lw (forward) or of the
 // same with tau(T) = mu (T + diag T) + lambda tr(T) I in place of S (adjoint).
 // Lambda_jj does not depend on x_j, so it is the node's value along the whole line.
-template <bool ADJ, int j>
-__device__ __forceinline__ void pml_force_axis(const Geo &g, const float *__restrict__ Y, int64_t node,
+template <bool RO, bool ADJ, int j>
+__device__ __forceinline__ void pml_force_axis(const Geo &g, const float *Y, int64_t node,
                                                const int c3[3], const int64_t st[3], const Ax ax[3], const float Le[3],
                                                const float Lp[3], const float Lw[3], float f[3]) {
   constexpr int k = (j + 1) % 3, l = (j + 2) % 3;
@@ -207,19 +220,19 @@ __device__ __forceinline__ void pml_force_axis(const Geo &g, const float *__rest
 #pragma unroll
         for (int lv = 0; lv < 3; lv++) {
           const float *b = Y + (int64_t)(9 * lv + 3) * S;
-          vj += Lv[lv] * __ldg(b + sym(j, j) * S + q);
-          vk += Lv[lv] * __ldg(b + sym(k, j) * S + q);
-          vl += Lv[lv] * __ldg(b + sym(l, j) * S + q);
+          vj += Lv[lv] * ldy<RO>(b + sym(j, j) * S + q);
+          vk += Lv[lv] * ldy<RO>(b + sym(k, j) * S + q);
+          vl += Lv[lv] * ldy<RO>(b + sym(l, j) * S + q);
         }
       } else {
         const float lam = __ldg(g.lam_n + q), mu = __ldg(g.mu_n + q);
 #pragma unroll
         for (int lv = 0; lv < 3; lv++) {
           const float *b = Y + (int64_t)(9 * lv + 3) * S;
-          const float tjj = __ldg(b + j * S + q), tkk = __ldg(b + k * S + q), tll = __ldg(b + l * S + q);
+          const float tjj = ldy<RO>(b + j * S + q), tkk = ldy<RO>(b + k * S + q), tll = ldy<RO>(b + l * S + q);
           vj += Lv[lv] * (2.f * mu * tjj + lam * (tjj + tkk + tll));
-          vk += Lv[lv] * (mu * __ldg(b + sym(k, j) * S + q));
-          vl += Lv[lv] * (mu * __ldg(b + sym(l, j) * S + q));
+          vk += Lv[lv] * (mu * ldy<RO>(b + sym(k, j) * S + q));
+          vl += Lv[lv] * (mu * ldy<RO>(b + sym(l, j) * S + q));
         }
       }
       qj += cf * vj;
@@ -238,8 +251,8 @@ __device__ __forceinline__ void pml_force_axis(const Geo &g, const float *__rest
 
 // S rows: column j of H = sum over PML elements of the element-wise derivatives of
 // udot (x Le_jj), u (x Lp_jj) and ubar (x Lw_jj) at the node
-template <int j>
-__device__ __forceinline__ void pml_strain_axis(const Geo &g, const float *__restrict__ Y, int64_t node,
+template <bool RO, int j>
+__device__ __forceinline__ void pml_strain_axis(const Geo &g, const float *Y, int64_t node,
                                                 const int64_t st[3], const Ax ax[3], const float Le[3],
                                                 const float Lp[3], const float Lw[3], float H[3][3]) {
   constexpr int k = (j + 1) % 3, l = (j + 2) % 3;
@@ -253,12 +266,12 @@ __device__ __forceinline__ void pml_strain_axis(const Geo &g, const float *__res
     const int cpml = ax[k].ns * ax[l].ns - (rdj ? nrd(ax[k]) * nrd(ax[l]) : 0);
     if (cpml == 0) continue;
     const float c = (float)cpml;
-    h0 += c * (Le[j] * dst(Y + 18 * S, node, st[j], t) + Lp[j] * dst(Y + 9 * S, node, st[j], t) +
-               Lw[j] * dst(Y, node, st[j], t));
-    h1 += c * (Le[j] * dst(Y + 19 * S, node, st[j], t) + Lp[j] * dst(Y + 10 * S, node, st[j], t) +
-               Lw[j] * dst(Y + S, node, st[j], t));
-    h2 += c * (Le[j] * dst(Y + 20 * S, node, st[j], t) + Lp[j] * dst(Y + 11 * S, node, st[j], t) +
-               Lw[j] * dst(Y + 2 * S, node, st[j], t));
+    h0 += c * (Le[j] * dst<RO>(Y + 18 * S, node, st[j], t) + Lp[j] * dst<RO>(Y + 9 * S, node, st[j], t) +
+               Lw[j] * dst<RO>(Y, node, st[j], t));
+    h1 += c * (Le[j] * dst<RO>(Y + 19 * S, node, st[j], t) + Lp[j] * dst<RO>(Y + 10 * S, node, st[j], t) +
+               Lw[j] * dst<RO>(Y + S, node, st[j], t));
+    h2 += c * (Le[j] * dst<RO>(Y + 20 * S, node, st[j], t) + Lp[j] * dst<RO>(Y + 11 * S, node, st[j], t) +
+               Lw[j] * dst<RO>(Y + 2 * S, node, st[j], t));
   }
   H[0][j] = h0;
   H[1][j] = h1;
@@ -323,40 +336,40 @@ struct ShellShared {
 };
 
 // axis-J terms of the node: of the interior elements (rd) and of the PML elements (pm)
-template <bool ADJ, int J>
+template <bool RO, bool ADJ, int J>
 __device__ __forceinline__ void shell_axis(const Geo &g, const StageArgs &a, const NodeCtx &n, ShellShared &sh, int lane,
                                            bool rd, bool pm) {
-  const float *__restrict__ Y = a.Y;
+  const float *Y = a.Y;
   const int64_t S = g.stride;
   if (rd && !n.dir) {
     float fr[3] = {0.f, 0.f, 0.f};
-    interior_force_axis<J>(g, Y + 9 * S, n.node, n.c3, n.st, n.ax, false, fr);
+    interior_force_axis<RO, J>(g, Y + 9 * S, n.node, n.c3, n.st, n.ax, false, fr);
 #pragma unroll
     for (int c = 0; c < 3; c++) sh.fr[J][c][lane] = fr[c];
   }
   if (pm && !n.dir) {
     float fp[3] = {0.f, 0.f, 0.f};
-    if (n.pml) pml_force_axis<ADJ, J>(g, Y, n.node, n.c3, n.st, n.ax, n.Le, n.Lp, n.Lw, fp);
+    if (n.pml) pml_force_axis<RO, ADJ, J>(g, Y, n.node, n.c3, n.st, n.ax, n.Le, n.Lp, n.Lw, fp);
 #pragma unroll
     for (int c = 0; c < 3; c++) sh.fp[J][c][lane] = fp[c];
   }
   if (pm && n.pml) {
     float H[3][3];
-    pml_strain_axis<J>(g, Y, n.node, n.st, n.ax, n.Le, n.Lp, n.Lw, H);
+    pml_strain_axis<RO, J>(g, Y, n.node, n.st, n.ax, n.Le, n.Lp, n.Lw, H);
 #pragma unroll
     for (int i = 0; i < 3; i++) sh.H[i][J][lane] = H[i][J];
   }
 }
 
 // first phase of warp w of W
-template <bool ADJ, int W>
+template <bool RO, bool ADJ, int W>
 __device__ __forceinline__ void shell_terms(const Geo &g, const StageArgs &a, const NodeCtx &n, ShellShared &sh, int lane,
                                             int w) {
   const int j = w % 3;
   const bool rd = W == 3 || w < 3, pm = W == 3 || w >= 3;
-  if (j == 0) shell_axis<ADJ, 0>(g, a, n, sh, lane, rd, pm);
-  else if (j == 1) shell_axis<ADJ, 1>(g, a, n, sh, lane, rd, pm);
-  else shell_axis<ADJ, 2>(g, a, n, sh, lane, rd, pm);
+  if (j == 0) shell_axis<RO, ADJ, 0>(g, a, n, sh, lane, rd, pm);
+  else if (j == 1) shell_axis<RO, ADJ, 1>(g, a, n, sh, lane, rd, pm);
+  else shell_axis<RO, ADJ, 2>(g, a, n, sh, lane, rd, pm);
 }
 
 // u-row force of component c
@@ -368,12 +381,22 @@ __device__ __forceinline__ float shell_force(const Geo &g, const ShellShared &sh
   return f[0] + f[1] + f[2];
 }
 
+// a variable's own stage-input values, its three levels; loaded before any of the node's stores,
+// which the plain loads of the persistent sweep could not pass
+struct OwnInput {
+  float v[3];
+};
+template <bool RO>
+__device__ __forceinline__ OwnInput load_input(const StageArgs &a, int64_t i0, int64_t nine) {
+  return OwnInput{{ldy<RO>(a.Y + i0), ldy<RO>(a.Y + i0 + nine), ldy<RO>(a.Y + i0 + 2 * nine)}};
+}
+
 // stress component c (order xx yy zz yz xz xy) of the node: its three levels
 template <bool ADJ>
 __device__ __forceinline__ void shell_stress(const Geo &g, const StageArgs &a, const NodeCtx &n,
-                                             const ShellShared &sh, int lane, int c, const StepStart &x) {
+                                             const ShellShared &sh, int lane, int c, const StepStart &x,
+                                             const OwnInput &y) {
   const int64_t S = g.stride;
-  const float *__restrict__ Y = a.Y;
   const int64_t i0 = (int64_t)(3 + c) * S + n.node, i1 = (int64_t)(12 + c) * S + n.node,
                 i2 = (int64_t)(21 + c) * S + n.node;
   if (!n.pml) {
@@ -396,7 +419,7 @@ __device__ __forceinline__ void shell_stress(const Geo &g, const StageArgs &a, c
     const float lam = __ldg(g.lam_n + n.node), mu = __ldg(g.mu_n + n.node);
     src = c < 3 ? __fmaf_rn(lam, P(0) + P(1) + P(2), __fmul_rn(2.f * mu, src)) : __fmul_rn(mu, src);
   }
-  const float s0 = __ldg(Y + i0), s1 = __ldg(Y + i1), s2 = __ldg(Y + i2);
+  const float s0 = y.v[0], s1 = y.v[1], s2 = y.v[2];
   __stcs(a.out + i0, stage_value(a, x.v[0], s0, s1));
   __stcs(a.out + i1, stage_value(a, x.v[1], s1, s2));
   __stcs(a.out + i2, stage_value(a, x.v[2], s2, __fmul_rn(__fmaf_rn(-n.cd, s0, __fmaf_rn(-n.cc, s1, __fmaf_rn(-n.cb, s2, src))), n.inv_a)));
@@ -405,9 +428,9 @@ __device__ __forceinline__ void shell_stress(const Geo &g, const StageArgs &a, c
 // displacement component c of the node: its three levels
 template <bool PTS>
 __device__ __forceinline__ void shell_disp(const Geo &g, const StageArgs &a, const Points &q, int shot, const NodeCtx &n,
-                                           const ShellShared &sh, int lane, int c, const StepStart &x) {
+                                           const ShellShared &sh, int lane, int c, const StepStart &x,
+                                           const OwnInput &y) {
   const int64_t S = g.stride;
-  const float *__restrict__ Y = a.Y;
   const int64_t i0 = (int64_t)c * S + n.node, i1 = (int64_t)(9 + c) * S + n.node, i2 = (int64_t)(18 + c) * S + n.node;
   if (n.dir) {
     if (a.stage == 0) {
@@ -419,7 +442,7 @@ __device__ __forceinline__ void shell_disp(const Geo &g, const StageArgs &a, con
   }
   const float fsum = shell_force(g, sh, c, lane);
   const float inv_m = n.inv_a / (g.rho * (float)n.nel);
-  const float u0 = __ldg(Y + i0), u1 = __ldg(Y + i1), u2 = __ldg(Y + i2);
+  const float u0 = y.v[0], u1 = y.v[1], u2 = y.v[2];
   const float decay = __fmaf_rn(n.cd, u0, __fmaf_rn(n.cc, u1, __fmul_rn(n.cb, u2)));
   const float acc = -__fmaf_rn(decay, n.inv_a, __fmul_rn(fsum, inv_m));
   if (n.pml || a.stage == 0) __stcs(a.out + i0, stage_value(a, x.v[0], u0, n.pml ? u1 : 0.f));
@@ -432,19 +455,33 @@ __device__ __forceinline__ void shell_disp(const Geo &g, const StageArgs &a, con
 }
 
 // second phase of warp w of W: displacement component w (w < 3), stress components w, w + W, ...
+template <int W>
+struct ShellOwn {
+  StepStart xu, xs[6 / W];
+  OwnInput yu, ys[6 / W];
+};
+template <bool RO, int W>
+__device__ __forceinline__ ShellOwn<W> shell_load(const Geo &g, const StageArgs &a, const NodeCtx &n, int w) {
+  const int64_t S = g.stride;
+  ShellOwn<W> o{};
+  if (w < 3 && !n.dir) {
+    o.xu = load_start(a, w * S + n.node, 9 * S);
+    o.yu = load_input<RO>(a, w * S + n.node, 9 * S);
+  }
+#pragma unroll
+  for (int h = 0; h < 6 / W; h++)
+    if (n.pml) {
+      o.xs[h] = load_start(a, (3 + w + h * W) * S + n.node, 9 * S);
+      o.ys[h] = load_input<RO>(a, (3 + w + h * W) * S + n.node, 9 * S);
+    }
+  return o;
+}
 template <bool ADJ, int W, bool PTS>
 __device__ __forceinline__ void shell_write(const Geo &g, const StageArgs &a, const Points &q, int shot, const NodeCtx &n,
-                                            const ShellShared &sh, int lane, int w) {
-  constexpr int NS = 6 / W;
-  const int64_t S = g.stride;
-  StepStart xu{}, xs[NS];
-  if (w < 3 && !n.dir) xu = load_start(a, w * S + n.node, 9 * S);
+                                            const ShellShared &sh, int lane, int w, const ShellOwn<W> &o) {
+  if (w < 3) shell_disp<PTS>(g, a, q, shot, n, sh, lane, w, o.xu, o.yu);
 #pragma unroll
-  for (int h = 0; h < NS; h++)
-    if (n.pml) xs[h] = load_start(a, (3 + w + h * W) * S + n.node, 9 * S);
-  if (w < 3) shell_disp<PTS>(g, a, q, shot, n, sh, lane, w, xu);
-#pragma unroll
-  for (int h = 0; h < NS; h++) shell_stress<ADJ>(g, a, n, sh, lane, w + h * W, xs[h]);
+  for (int h = 0; h < 6 / W; h++) shell_stress<ADJ>(g, a, n, sh, lane, w + h * W, o.xs[h], o.ys[h]);
 }
 
 template <bool ADJ, int W, bool PTS>
@@ -461,10 +498,10 @@ __global__ void __launch_bounds__(W *kShellNodes, 24 / W) shell_kernel(Geo g, St
     const int node = g.shell[i];
     const int I = node % g.px, r = node / g.px;
     n = node_ctx(g, I, r % g.n[1], r / g.n[1]);
-    shell_terms<ADJ, W>(g, a, n, sh, lane, w);
+    shell_terms<true, ADJ, W>(g, a, n, sh, lane, w);
   }
   __syncthreads();
-  if (live) shell_write<ADJ, W, PTS>(g, a, q, shot, n, sh, lane, w);
+  if (live) shell_write<ADJ, W, PTS>(g, a, q, shot, n, sh, lane, w, shell_load<true, W>(g, a, n, w));
 }
 
 // ---- persistent forward sweep (see PersistArgs)
@@ -503,8 +540,9 @@ __device__ bool grid_barrier(const PersistArgs &p, unsigned expected) {
 }
 
 // six warps a block: the sweep is meant for meshes of about one wave of blocks, where a stage
-// takes one node chunk's chain of loads (8x8x4 elements, a 100-step sweep: 7.07 ms; with three
-// warps and 4 blocks an SM 8.09 ms, with six warps and 2 blocks 8.71 ms)
+// takes one node chunk's chain of loads (8x8x4 elements, a 100-step sweep, measured with read-only
+// loads: 7.07 ms; with three warps and 4 blocks an SM 8.09 ms, with six warps and 2 blocks 8.71
+// ms; 6.92 ms now). The second phase's own operands are loaded before the block's barrier.
 constexpr int kPersistWarps = 6;
 __global__ void __launch_bounds__(kPersistWarps *kShellNodes, 3) persistent_forward_kernel(Geo g, PersistArgs p) {
   __shared__ ShellShared sh;
@@ -536,14 +574,16 @@ __global__ void __launch_bounds__(kPersistWarps *kShellNodes, 3) persistent_forw
         const int i = (ch % nch) * kShellNodes + lane;
         const bool live = i < p.nall && node_ok(g, kSitePersist, p.nodes[i]);
         NodeCtx n;
+        ShellOwn<kPersistWarps> own{};
         if (live) {
           const int node = p.nodes[i];
           const int I = node % g.px, r = node / g.px;
           n = node_ctx(g, I, r % g.n[1], r / g.n[1]);
-          shell_terms<false, kPersistWarps>(g, a, n, sh, lane, w);
+          shell_terms<false, false, kPersistWarps>(g, a, n, sh, lane, w);
+          own = shell_load<false, kPersistWarps>(g, a, n, w);
         }
         __syncthreads();
-        if (live) shell_write<false, kPersistWarps, true>(g, a, q, b, n, sh, lane, w);
+        if (live) shell_write<false, kPersistWarps, true>(g, a, q, b, n, sh, lane, w, own);
         __syncthreads();
       }
       if (!grid_barrier(p, expected)) return;
