@@ -349,6 +349,10 @@ fwi_status check_status(fwi_ctx *c) {
 }
 
 fwi_status stage(fwi_ctx *c, bool adj, const fwi::StageArgs &a, const fwi::Points &q, bool pml_points) {
+  // the one thing that can refuse a stage, before anything of it is launched
+  fwi::PlaneMap map;
+  if (!fwi::plane_map(c->geo, a, &map))
+    return fail(c, FWI_E_CUDA, "no tensor map for the stage input (not 16-byte aligned, or no driver entry)");
   cudaEvent_t e0;
   time_begin(c, &e0);
   // fork: interior and interface/face kernels on the side streams, bulk PML here
@@ -359,9 +363,7 @@ fwi_status stage(fwi_ctx *c, bool adj, const fwi::StageArgs &a, const fwi::Point
   // elements with 2 PML elements, two shots: a gradient in 54.7 ms with the interior first, 32.3 last)
   int nk = fwi::launch_shell(c->geo, a, q, adj, c->side[1]) + fwi::launch_pml_face(c->geo, a, q, adj, c->side[1]) +
            fwi::launch_pml(c->geo, a, adj, c->stream);
-  const int ni = fwi::launch_interior(c->geo, a, q, c->side[0]);
-  if (ni < 0) return fail(c, FWI_E_CUDA, "no tensor map for the stage input (not 16-byte aligned, or no driver entry)");
-  nk += ni;
+  nk += fwi::launch_interior(c->geo, a, q, map, c->side[0]);
   for (int i = 0; i < kSides; i++) {
     CUDA_TRY(c, cudaEventRecord(c->ev_join[i], c->side[i]));
     CUDA_TRY(c, cudaStreamWaitEvent(c->stream, c->ev_join[i], 0));

@@ -404,12 +404,22 @@ EncodeTiled encode_tiled() {
   return fn;
 }
 
+bool has_interior(const Geo &g) {
+  return g.box_hi[0] >= g.box_lo[0] && g.box_hi[1] >= g.box_lo[1] && g.box_hi[2] >= g.box_lo[2];
+}
+
+}  // namespace
+
 // tensor map of the stage input Y of nshot shots as a 4-D FP32 tensor: x (the row pitch px),
 // y (NJ rows), z (NK planes), f (27 nshot fields, `stride` floats apart; shot b's field c is
 // 27 b + c, as the shots' state sets are 27 stride floats apart). Boxes are 72 x 12 x 1 x 3;
 // elements outside the tensor read as zero (the row padding x >= NI holds zeros in every
 // state buffer, so a box reads zero wherever the node grid ends).
-bool plane_map(const Geo &g, const StageArgs &a, CUtensorMap *tm) {
+bool plane_map(const Geo &g, const StageArgs &a, PlaneMap *out) {
+  static_assert(sizeof(PlaneMap) == sizeof(CUtensorMap) && alignof(PlaneMap) >= alignof(CUtensorMap), "PlaneMap");
+  std::memset(out, 0, sizeof(*out));
+  if (!has_interior(g)) return true;  // no launch, no map
+  CUtensorMap *const tm = reinterpret_cast<CUtensorMap *>(out);
   const EncodeTiled enc = encode_tiled();
   if (!enc || ((uintptr_t)a.Y & 15) != 0 || (a.nshot > 1 && a.sstride != (int64_t)kFields * g.stride)) return false;
   const cuuint64_t dims[4] = {(cuuint64_t)g.px, (cuuint64_t)g.n[1], (cuuint64_t)g.n[2],
@@ -422,8 +432,6 @@ bool plane_map(const Geo &g, const StageArgs &a, CUtensorMap *tm) {
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-}  // namespace
-
 cudaError_t prepare_interior() {
   for (auto kernel : {interior_kernel<0, false>, interior_kernel<1, false>, interior_kernel<2, false>,
                       interior_kernel<3, false>, interior_kernel<1, true>, interior_kernel<2, true>, interior_kernel<3, true>}) {
@@ -433,9 +441,9 @@ cudaError_t prepare_interior() {
   return cudaSuccess;
 }
 
-int launch_interior(const Geo &g0, const StageArgs &a, const Points &q, cudaStream_t s) {
+int launch_interior(const Geo &g0, const StageArgs &a, const Points &q, const PlaneMap &map, cudaStream_t s) {
   Geo g = g0;
-  if (g.box_hi[0] < g.box_lo[0] || g.box_hi[1] < g.box_lo[1] || g.box_hi[2] < g.box_lo[2]) return 0;
+  if (!has_interior(g)) return 0;
   const int nx = g.box_hi[0] - (g.box_lo[0] - 1) + 1;
   const int tx = (nx + 2 * kTP - 1) / (2 * kTP), ty = (g.box_hi[1] - g.box_lo[1] + kTY) / kTY;
   // a ring fill costs about 1.5 planes: 5 planes of copies against 4.5 us per computed plane
@@ -443,8 +451,7 @@ int launch_interior(const Geo &g0, const StageArgs &a, const Points &q, cudaStre
   const dim3 grd(tx, ty,
                  (g.box_hi[2] - g.box_lo[2] + g.int_kc) / g.int_kc * a.nshot);
   CUtensorMap tm;
-  std::memset(&tm, 0, sizeof(tm));
-  if (!plane_map(g, a, &tm)) return -1;
+  std::memcpy(&tm, &map, sizeof(tm));
   const bool pts = q.fused && q.k0 <= g.box_hi[2];
   const auto kernel = a.stage == 0   ? interior_kernel<0, false>
                       : a.stage == 1 ? (pts ? interior_kernel<1, true> : interior_kernel<1, false>)

@@ -210,15 +210,20 @@ __device__ __forceinline__ bool node_ok(const Geo &g, int site, long long node) 
 // One RK4 stage is four kernels writing disjoint node sets; they read the same
 // input and may run concurrently on different streams. Each launcher returns the
 // number of kernels it launched:
-//  launch_interior: nodes all of whose elements are interior (fwi_interior.cu); -1 if
-//                   the tensor map of the stage input could not be encoded (Y not
-//                   16-byte aligned, or the driver entry point missing);
+//  launch_interior: nodes all of whose elements are interior (fwi_interior.cu), with the tensor
+//                   map of the stage input from plane_map. plane_map is false when it could not
+//                   be encoded (Y not 16-byte aligned, or the driver entry point missing): the
+//                   one way a stage can be refused, so it comes before the first launch;
 //  launch_pml:      nodes all of whose elements are PML, off the outer faces (fwi_pml.cu);
 //  launch_shell:    the interface shell (fwi_stage.cu);
 //  launch_pml_face: the PML nodes on the outer faces of the grid (fwi_pml.cu).
 // launch_points: points_kernel over the sources and receivers (only those on launch_pml's
 // nodes when q.fused), after the stage's kernels.
-int launch_interior(const Geo &g, const StageArgs &a, const Points &q, cudaStream_t s);
+struct alignas(128) PlaneMap {  // a CUtensorMap
+  unsigned char bytes[128];
+};
+bool plane_map(const Geo &g, const StageArgs &a, PlaneMap *tm);
+int launch_interior(const Geo &g, const StageArgs &a, const Points &q, const PlaneMap &tm, cudaStream_t s);
 int launch_pml(const Geo &g, const StageArgs &a, bool adjoint, cudaStream_t s);
 int launch_points(const Geo &g, const StageArgs &a, const Points &q, const int64_t *rec_node, cudaStream_t s);
 int launch_pml_face(const Geo &g, const StageArgs &a, const Points &q, bool adjoint, cudaStream_t s);
