@@ -138,6 +138,12 @@ __device__ __forceinline__ void tmem_ld16(uint32_t r[16], unsigned a) {
       : "r"(a));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
+// max(f, 0) that keeps a NaN (fmaxf would return 0, and a tile given up would look like zeros)
+__device__ __forceinline__ float relu_nan(float f) {
+  float r;
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(r) : "f"(f));
+  return r;
+}
 // 16 columns of this thread's TMEM lane
 __device__ __forceinline__ void tmem_st16(unsigned a, const uint4 v[4]) {
   asm volatile(
@@ -515,7 +521,7 @@ __global__ void __launch_bounds__(kTileThreads, 2)
               v[j] = ok ? __uint_as_float(r[j]) : __uint_as_float(0x7FC00000u);
             } else {
               float f = __uint_as_float(r[j]) + sbias[c0 + j];
-              if (relu) f = fmaxf(f, 0.f);
+              if (relu) f = relu_nan(f);
               v[j] = ok ? __bfloat16_as_ushort(__float2bfloat16_rn(f)) : (uint16_t)0x7FC0;
             }
           }
