@@ -686,14 +686,16 @@ constexpr int kWgAccCols = 368;    // accumulator columns: 368 + 16 (bias) = 384
 constexpr int kWgMaxRing = 8;      // most stages in flight
 constexpr int kWgRows = 42;        // gradient channels per M tile (3 parts: 126 rows)
 constexpr int kWgSlice = 48;       // most tiles per slice: 6144 voxels, 384 sums per accumulator
+constexpr int kWgThin = 8;         // times as many on grids of one or two rows (one of a tile's 8 MMAs is not zero)
 constexpr int kWorkSlice = 2048;    // voxels per slice the size of `work` is counted by
 
 // dyt[mt][tile][y][r][8 x]: the split gradient of the rows r = part cm + c of M tile mt
-// (channel mt cm + c), per voxel tile and tile row; zero outside the grid and past cout. A
-// block turns one tile of up to 32 channels through shared memory, so that both its reads
+// (channel mt cm + c), per voxel tile (the ncopy tiles from `first` on) and tile row; zero outside
+// the grid and past cout. A block turns one tile of up to 32 channels through shared memory, so that both its reads
 // (8 voxels of a row) and its writes (16 bytes of consecutive channels) are contiguous.
-__device__ __forceinline__ void split_tile_block(const float *__restrict__ dy, int cout, int cm, int ntx, int nty, int ntile,
-                                                 int D, int H, int W, uint16_t *__restrict__ dyt, int tile, int mt, int c0) {
+__device__ __forceinline__ void split_tile_block(const float *__restrict__ dy, int cout, int cm, int ntx, int nty, int first,
+                                                 int ncopy, int D, int H, int W, uint16_t *__restrict__ dyt, int tile,
+                                                 int mt, int c0) {
   __shared__ float st[32][kM + 1];
   const int x0 = tile % ntx * kTX, y0 = tile / ntx % nty * kTY, z = tile / ntx / nty;
   const int nc = min(32, cm - c0);
@@ -702,7 +704,7 @@ __device__ __forceinline__ void split_tile_block(const float *__restrict__ dy, i
     st[c][v] = (co < cout && x < W && y < H) ? __ldg(dy + (((int64_t)co * D + z) * H + y) * W + x) : 0.f;
   }
   __syncthreads();
-  const int64_t base = ((int64_t)mt * ntile + tile) * kTY * (3 * cm);
+  const int64_t base = ((int64_t)mt * ncopy + (tile - first)) * kTY * (3 * cm);
   for (int i = threadIdx.x; i < 32 * kTY; i += 256) {
     const int c = i & 31, y = i >> 5;
     if (c >= nc) continue;
@@ -725,6 +727,8 @@ struct WgShape {
   int cm, mt;              // gradient channels per M tile, M tiles
   int G, ntx, nty, tiles;  // source groups, voxel tiles
   int slices, per;         // slices, tiles per slice
+  int slice0;              // first slice of the launch
+  int first, ncopy;        // first tile and tiles of its slices, those in the copy of the gradient
   int ring, smem;
 };
 
@@ -747,10 +751,11 @@ __global__ void __launch_bounds__(256) wgrad_prep_kernel(const float *__restrict
     return;
   }
   const int chunks = (g.cm + 31) / 32;  // of 32 channels of an M tile
-  for (int64_t i = b - nsrc; i < (int64_t)g.tiles * chunks * g.mt; i += gridDim.x - nsrc) {
-    const int r = (int)(i / g.tiles);
+  for (int64_t i = b - nsrc; i < (int64_t)g.ncopy * chunks * g.mt; i += gridDim.x - nsrc) {
+    const int r = (int)(i / g.ncopy);
     __syncthreads();  // the tile before has been read
-    split_tile_block(dy, cout, g.cm, g.ntx, g.nty, g.tiles, D, H, W, dyt, (int)(i % g.tiles), r / chunks, r % chunks * 32);
+    split_tile_block(dy, cout, g.cm, g.ntx, g.nty, g.first, g.ncopy, D, H, W, dyt, g.first + (int)(i % g.ncopy), r / chunks,
+                     r % chunks * 32);
   }
 }
 
@@ -767,7 +772,7 @@ __global__ void __launch_bounds__(32 * (5 + T), 1)
   // the blocks of one slice are neighbours in the grid: its voxels are read while L2 holds them
   constexpr int ngrp = 27 / T;
   const int grp = blockIdx.x % ngrp, nt = blockIdx.x / ngrp % g.ntile, mt = blockIdx.x / ngrp / g.ntile;
-  const int slice = blockIdx.y;
+  const int slice = g.slice0 + blockIdx.y;
   const int tap0 = grp * T, kz = tap0 / 9, ky0 = tap0 / 3 % 3;
   const bool bias = tap0 / 9 == 1 && (T == 9 || ky0 == 1) && nt == 0;
   const int R = 3 * g.cm, plane = g.ntx * g.nty;
@@ -824,7 +829,7 @@ __global__ void __launch_bounds__(32 * (5 + T), 1)
     }
     if (!ok) atomicExch(&okslot, 0);
   } else if (warp == 4 && one) {  // copies
-    const uint16_t *src = dyt + ((int64_t)mt * g.tiles + t0) * (a_bytes / 2);
+    const uint16_t *src = dyt + ((int64_t)mt * g.ncopy + (t0 - g.first)) * (a_bytes / 2);
     bool ok = true;
     int i = 0;
     for (; i < n; i++) {
@@ -971,7 +976,7 @@ cudaError_t conv3d_backward_weight_tc(const float *dy, const uint16_t *x, int ci
   g.ntx = (W + kTX - 1) / kTX;
   g.nty = (H + kTY - 1) / kTY;
   const int64_t tiles = (int64_t)g.ntx * g.nty * D;
-  if (tiles > 0x7fffffff / 64) return cudaErrorInvalidValue;
+  if ((nv + kWorkSlice - 1) / kWorkSlice > 65535) return cudaErrorInvalidValue;  // the limit the size of `work` assumes
   g.tiles = (int)tiles;
   g.mt = (cout + kWgRows - 1) / kWgRows;
   g.cm = (cout + g.mt - 1) / g.mt;
@@ -984,12 +989,12 @@ cudaError_t conv3d_backward_weight_tc(const float *dy, const uint16_t *x, int ci
   const int combos = 27 / g.T * g.ntile * g.mt;
   // one block per SM (all its TMEM): as many slices as fill whole waves of the SMs, at most
   // kWgSlice tiles each, and on small grids at least two tiles
-  const int64_t waves = ((int64_t)combos * ((tiles + kWgSlice - 1) / kWgSlice) + kSms - 1) / kSms;
+  const int cap = H <= 2 ? kWgThin * kWgSlice : kWgSlice;
+  const int64_t waves = ((int64_t)combos * ((tiles + cap - 1) / cap) + kSms - 1) / kSms;
   int64_t slices = std::max<int64_t>(1, waves * kSms / combos);
-  slices = std::max<int64_t>(std::min(slices, (tiles + 1) / 2), (tiles + kWgSlice - 1) / kWgSlice);
+  slices = std::max<int64_t>(std::min(slices, (tiles + 1) / 2), (tiles + cap - 1) / cap);
   g.per = (int)((tiles + slices - 1) / slices);
   g.slices = (int)((tiles + g.per - 1) / g.per);
-  if ((nv + kWorkSlice - 1) / kWorkSlice > 65535) return cudaErrorInvalidValue;  // as the size of `work` assumes
   const int stage = (g.nt_n / 8 * kGroupBytes + 3 * g.cm * kTY * 16 + 127) / 128 * 128;
   g.ring = std::min(kWgMaxRing, kSmBlock / stage);
   g.smem = std::max({g.ring * stage, kM * (g.T * g.nt_n + 17) * 4, kSmPerSM / 2});  // one block per SM, as its TMEM is one block's
@@ -997,7 +1002,13 @@ cudaError_t conv3d_backward_weight_tc(const float *dy, const uint16_t *x, int ci
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmBlock);
   if (e != cudaSuccess) return e;
   const size_t src_bytes = align256((size_t)g.G * nv * 16);
-  const size_t dyt_bytes = align256((size_t)g.mt * tiles * kTY * 3 * g.cm * 16);
+  // The copy of the gradient holds whole tiles: on thin grids many times the gradient's size. It
+  // is at most about twice that of a grid of full tiles, and the slices take turns with it.
+  const int64_t tile_bytes = (int64_t)g.mt * kTY * 3 * g.cm * 16;
+  const int64_t most_bytes = std::max<int64_t>(2 * tile_bytes * (nv / kM), 256 << 20);
+  int64_t turn = std::min(g.slices, 65535);  // slices of a launch: its grid's y
+  if (tile_bytes * tiles > most_bytes) turn = std::max<int64_t>(1, std::min(turn, most_bytes / (tile_bytes * g.per)));
+  const size_t dyt_bytes = align256((size_t)(tile_bytes * std::min(tiles, turn * g.per)));
   const int64_t part_floats = (int64_t)g.slices * cout * (27 * (int64_t)cin + 1);
   const bool own = part_floats > conv3d_backward_weight_tc_work(cin, cout, D, H, W);
   unsigned char *buf = nullptr;
@@ -1009,12 +1020,18 @@ cudaError_t conv3d_backward_weight_tc(const float *dy, const uint16_t *x, int ci
   e = box_map(&tm, src, D, H, W, g.G, g.nt_n / 8);
   if (e == cudaSuccess) {
     const unsigned nx = blocks_x(nv, 256, 65536), nsrc = nx * (unsigned)g.G;
-    const unsigned ntl = blocks_x((int64_t)g.tiles * ((g.cm + 31) / 32) * g.mt, 1, 1 << 30);
     const bool apart = nv > kPrepVoxels;
     if (apart) group_major_kernel<<<nsrc, 256, 0, s>>>(x, nv, cin, src, (int)nx);
-    wgrad_prep_kernel<<<(apart ? 0 : nsrc) + ntl, 256, 0, s>>>(dy, x, nv, cin, cout, g, D, H, W, src, dyt, (int)nx,
-                                                              apart ? 0 : (int)nsrc);
-    kernel<<<dim3((unsigned)combos, (unsigned)g.slices), 32 * (5 + g.T), g.smem, s>>>(tm, dyt, g, D, cin, cout, part);
+    for (int64_t sl = 0; sl < g.slices; sl += turn) {
+      const int ns = (int)std::min<int64_t>(turn, g.slices - sl);
+      g.slice0 = (int)sl;
+      g.first = (int)(sl * g.per);
+      g.ncopy = (int)std::min<int64_t>((int64_t)ns * g.per, tiles - g.first);
+      const unsigned ntl = blocks_x((int64_t)g.ncopy * ((g.cm + 31) / 32) * g.mt, 1, 1 << 30);
+      const unsigned nx_here = apart || sl > 0 ? 0 : nsrc;
+      wgrad_prep_kernel<<<nx_here + ntl, 256, 0, s>>>(dy, x, nv, cin, cout, g, D, H, W, src, dyt, (int)nx, (int)nx_here);
+      kernel<<<dim3((unsigned)combos, (unsigned)ns), 32 * (5 + g.T), g.smem, s>>>(tm, dyt, g, D, cin, cout, part);
+    }
     wgrad_reduce_kernel<<<blocks_x((int64_t)cout * (27 * (int64_t)cin + 1), 32, 65536), 256, 0, s>>>(part, g.slices, cin,
                                                                                                   cout, dw, db);
     e = cudaGetLastError();
