@@ -357,8 +357,9 @@ fwi_status fwi_set_graphs(fwi_ctx *ctx, int enable);
 /* Kernel timing: with enable = 1 every stage-kernel launch of later calls is
  * bracketed by CUDA events on the context's stream; fwi_get_timing returns the
  * summed device time (ms) and launch count of kernel class `which`
- * (0: RK stage kernels, 1: gradient kernel, 2: none; point loads and
- * samples count in class 0), 3: all kernels launched, time unset) since the last reset. */
+ * (0: RK stage kernels, 1: gradient kernel, 2: point-load / sampling kernels, of the stages
+ * whose own kernels do not apply the points: more than 8 million nodes in the batch, or points
+ * inside the PML; 3: all kernels launched, time unset) since the last reset. */
 fwi_status fwi_set_timing(fwi_ctx *ctx, int enable);
 fwi_status fwi_get_timing(fwi_ctx *ctx, int which, double *ms, int64_t *launches);
 fwi_status fwi_reset_timing(fwi_ctx *ctx);

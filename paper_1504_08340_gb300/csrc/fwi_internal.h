@@ -225,7 +225,7 @@ struct alignas(128) PlaneMap {  // a CUtensorMap
 bool plane_map(const Geo &g, const StageArgs &a, PlaneMap *tm);
 int launch_interior(const Geo &g, const StageArgs &a, const Points &q, const PlaneMap &tm, cudaStream_t s);
 int launch_pml(const Geo &g, const StageArgs &a, bool adjoint, cudaStream_t s);
-int launch_points(const Geo &g, const StageArgs &a, const Points &q, const int64_t *rec_node, cudaStream_t s);
+void launch_points(const Geo &g, const StageArgs &a, const Points &q, const int64_t *rec_node, cudaStream_t s);
 int launch_pml_face(const Geo &g, const StageArgs &a, const Points &q, bool adjoint, cudaStream_t s);
 int launch_shell(const Geo &g, const StageArgs &a, const Points &q, bool adjoint, cudaStream_t s);
 // raises the interior kernel's shared-memory limit on the current device

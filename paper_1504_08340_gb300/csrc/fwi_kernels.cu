@@ -222,9 +222,8 @@ inline unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + thre
 
 }  // namespace
 
-int launch_points(const Geo &g, const StageArgs &a, const Points &q, const int64_t *rec_node, cudaStream_t s) {
+void launch_points(const Geo &g, const StageArgs &a, const Points &q, const int64_t *rec_node, cudaStream_t s) {
   points_kernel<<<blocks_for((int64_t)a.nshot * (q.nrec + 1), 128), 128, 0, s>>>(g, a, q, rec_node);
-  return 1;
 }
 
 void launch_rec_map(const int64_t *node, int nrec, int *rec_of, int64_t rec0, int64_t rec_n, cudaStream_t s) {
