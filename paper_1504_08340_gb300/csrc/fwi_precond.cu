@@ -91,25 +91,28 @@ struct Cells {
 };
 
 // blockIdx.y walks the (channel, z) planes of the output and the threads its voxels (y, x) in
-// order, so an index costs one 32-bit division and consecutive threads write consecutive
-// voxels. Bound by HBM; one flat 64-bit index per value had taken three 64-bit divisions
-// (upsampling 56 channels to 65 x 129 x 129: 443 us, 75 us this way, 20 us of traffic).
+// order; on planes of at most kT / 2 voxels (SMALL) threadIdx.y walks planes too. An index costs one 32-bit
+// division and consecutive threads write consecutive voxels. Bound by HBM; one flat 64-bit index
+// per value had taken three 64-bit divisions (upsampling 56 channels to 65 x 129 x 129: 322 us, 66 us
+// this way, 20 us of traffic), and a block per plane wastes its threads on small planes (pooling
+// 64 channels of 4096 x 4 x 4: 76 us).
 
 // f(c, z, y, x, i) for this thread's voxels of a [C][D][H][W] grid, i the voxel's offset in the plane
-template <class F>
+template <bool SMALL, class F>
 __device__ __forceinline__ void for_voxels(int C, int D, int H, int W, F f) {
   const int64_t planes = (int64_t)C * D;
   const int64_t n = (int64_t)H * W;
-  for (int64_t cz = blockIdx.y; cz < planes; cz += gridDim.y) {
+  const unsigned tx = SMALL ? blockDim.x : kT, ty = SMALL ? blockDim.y : 1;
+  for (int64_t cz = (int64_t)blockIdx.y * ty + (SMALL ? threadIdx.y : 0); cz < planes; cz += (int64_t)gridDim.y * ty) {
     const int c = (int)(cz / D), z = (int)(cz - (int64_t)c * D);
     if (n <= 0x7fffffff) {
 #pragma unroll 4
-      for (unsigned i = blockIdx.x * kT + threadIdx.x; i < (unsigned)n; i += gridDim.x * kT) {
+      for (unsigned i = blockIdx.x * tx + threadIdx.x; i < (unsigned)n; i += gridDim.x * tx) {
         const unsigned y = i / (unsigned)W;
         f(c, z, (int)y, (int)(i - y * W), (int64_t)i);
       }
     } else {
-      for (int64_t i = (int64_t)blockIdx.x * kT + threadIdx.x; i < n; i += (int64_t)gridDim.x * kT)
+      for (int64_t i = (int64_t)blockIdx.x * tx + threadIdx.x; i < n; i += (int64_t)gridDim.x * tx)
         f(c, z, (int)(i / W), (int)(i % W), i);
     }
   }
@@ -132,18 +135,20 @@ __device__ __forceinline__ float cell_sum(const T *__restrict__ r, const Cells &
 }
 
 // y[c][q] = mean of x[c][p] over the fine voxels p of coarse cell q (FP32 sum, rounded to BF16)
+template <bool SMALL>
 __global__ void __launch_bounds__(kT) pool2_fwd_kernel(const uint16_t *__restrict__ x, int C, Cells g,
                                                        uint16_t *__restrict__ y) {
-  for_voxels(C, g.Dc, g.Hc, g.Wc, [&](int c, int q0, int q1, int q2, int64_t i) {
+  for_voxels<SMALL>(C, g.Dc, g.Hc, g.Wc, [&](int c, int q0, int q1, int q2, int64_t i) {
     const float s = cell_sum(x + (((int64_t)c * g.D + 2 * q0) * g.H + 2 * q1) * g.W + 2 * q2, g, q0, q1, q2, bf2f);
     y[((int64_t)c * g.Dc + q0) * g.Hc * g.Wc + i] = f2bf(s / (float)g.count(q0, q1, q2));
   });
 }
 
 // dx[c][p] (+)= dy[c][cell(p)] / count(cell(p))
+template <bool SMALL>
 __global__ void __launch_bounds__(kT) pool2_bwd_kernel(const float *__restrict__ dy, int C, Cells g, int acc,
                                                        float *__restrict__ dx) {
-  for_voxels(C, g.D, g.H, g.W, [&](int c, int z, int y, int x, int64_t i) {
+  for_voxels<SMALL>(C, g.D, g.H, g.W, [&](int c, int z, int y, int x, int64_t i) {
     const int q0 = z >> 1, q1 = y >> 1, q2 = x >> 1;
     const float v = dy[(((int64_t)c * g.Dc + q0) * g.Hc + q1) * g.Wc + q2] / (float)g.count(q0, q1, q2);
     float *o = dx + ((int64_t)c * g.D + z) * g.H * g.W + i;
@@ -153,9 +158,10 @@ __global__ void __launch_bounds__(kT) pool2_bwd_kernel(const float *__restrict__
 
 // y[c][p] = x[c][cell(p)] (nearest neighbour); a thread owns one x of a coarse row and writes
 // it to the up to four fine rows of that row's cells
+template <bool SMALL>
 __global__ void __launch_bounds__(kT) up2_fwd_kernel(const uint16_t *__restrict__ x, int C, Cells g,
                                                      uint16_t *__restrict__ y) {
-  for_voxels(C, g.Dc, g.Hc, g.W, [&](int c, int q0, int q1, int xx, int64_t) {
+  for_voxels<SMALL>(C, g.Dc, g.Hc, g.W, [&](int c, int q0, int q1, int xx, int64_t) {
     const uint16_t v = __ldg(x + (((int64_t)c * g.Dc + q0) * g.Hc + q1) * g.Wc + (xx >> 1));
     uint16_t *o = y + (((int64_t)c * g.D + 2 * q0) * g.H + 2 * q1) * g.W + xx;
     const bool bz = 2 * q0 + 1 < g.D, by = 2 * q1 + 1 < g.H;
@@ -168,9 +174,10 @@ __global__ void __launch_bounds__(kT) up2_fwd_kernel(const uint16_t *__restrict_
 }
 
 // dx[c][q] (+)= sum of dy[c][p] over the fine voxels p of cell q, in a fixed order
+template <bool SMALL>
 __global__ void __launch_bounds__(kT) up2_bwd_kernel(const float *__restrict__ dy, int C, Cells g, int acc,
                                                      float *__restrict__ dx) {
-  for_voxels(C, g.Dc, g.Hc, g.Wc, [&](int c, int q0, int q1, int q2, int64_t i) {
+  for_voxels<SMALL>(C, g.Dc, g.Hc, g.Wc, [&](int c, int q0, int q1, int q2, int64_t i) {
     const float s = cell_sum(dy + (((int64_t)c * g.D + 2 * q0) * g.H + 2 * q1) * g.W + 2 * q2, g, q0, q1, q2,
                              [](float v) { return v; });
     float *o = dx + ((int64_t)c * g.Dc + q0) * g.Hc * g.Wc + i;
@@ -178,10 +185,17 @@ __global__ void __launch_bounds__(kT) up2_bwd_kernel(const float *__restrict__ d
   });
 }
 
-// grid of for_voxels over C x D planes of H x W voxels: four voxels a thread
-dim3 plane_grid(int C, int D, int H, int W) {
-  const int64_t planes = (int64_t)C * D, b = ((int64_t)H * W + 4 * kT - 1) / (4 * kT);
-  return dim3((unsigned)(b < 65536 ? b : 65536), (unsigned)(planes < 65535 ? planes : 65535));
+// launch of for_voxels over C x D planes of H x W voxels: four voxels a thread on large planes
+struct PlaneLaunch {
+  dim3 grid, block;
+};
+PlaneLaunch plane_launch(int C, int D, int H, int W) {
+  const int64_t n = (int64_t)H * W, b = (n + 4 * kT - 1) / (4 * kT);
+  int tx = kT;
+  while (tx > 1 && tx / 2 >= n) tx /= 2;  // the voxels of a small plane, rounded up
+  const int ty = kT / tx;
+  const int64_t rows = ((int64_t)C * D + ty - 1) / ty;
+  return {dim3((unsigned)(b < 65536 ? b : 65536), (unsigned)(rows < 65535 ? rows : 65535)), dim3(tx, ty)};
 }
 
 Cells cells(int D, int H, int W) { return Cells{D, H, W, (D + 1) / 2, (H + 1) / 2, (W + 1) / 2}; }
@@ -264,19 +278,26 @@ fwi_status fwi_nn_adam(float *master, uint16_t *w, const float *g, float *m, flo
 fwi_status fwi_nn_pool2_forward(const uint16_t *x, int C, int D, int H, int W, uint16_t *y, void *stream) {
   if (!x || !y || !sizes_ok(C, 1, D, H, W)) return FWI_E_INVAL;
   const Cells g = cells(D, H, W);
-  pool2_fwd_kernel<<<plane_grid(C, g.Dc, g.Hc, g.Wc), kT, 0, (cudaStream_t)stream>>>(x, C, g, y);
+  const PlaneLaunch l = plane_launch(C, g.Dc, g.Hc, g.Wc);
+  const auto kernel = l.block.y > 1 ? pool2_fwd_kernel<true> : pool2_fwd_kernel<false>;
+  kernel<<<l.grid, l.block, 0, (cudaStream_t)stream>>>(x, C, g, y);
   return launched();
 }
 
 fwi_status fwi_nn_pool2_backward(const float *dy, int C, int D, int H, int W, int accumulate, float *dx, void *stream) {
   if (!dy || !dx || !sizes_ok(C, 1, D, H, W)) return FWI_E_INVAL;
-  pool2_bwd_kernel<<<plane_grid(C, D, H, W), kT, 0, (cudaStream_t)stream>>>(dy, C, cells(D, H, W), accumulate != 0, dx);
+  const PlaneLaunch l = plane_launch(C, D, H, W);
+  const auto kernel = l.block.y > 1 ? pool2_bwd_kernel<true> : pool2_bwd_kernel<false>;
+  kernel<<<l.grid, l.block, 0, (cudaStream_t)stream>>>(dy, C, cells(D, H, W), accumulate != 0, dx);
   return launched();
 }
 
 fwi_status fwi_nn_upsample2_forward(const uint16_t *x, int C, int D, int H, int W, uint16_t *y, void *stream) {
   if (!x || !y || !sizes_ok(C, 1, D, H, W)) return FWI_E_INVAL;
-  up2_fwd_kernel<<<plane_grid(C, (D + 1) / 2, (H + 1) / 2, W), kT, 0, (cudaStream_t)stream>>>(x, C, cells(D, H, W), y);
+  const Cells g = cells(D, H, W);
+  const PlaneLaunch l = plane_launch(C, g.Dc, g.Hc, W);
+  const auto kernel = l.block.y > 1 ? up2_fwd_kernel<true> : up2_fwd_kernel<false>;
+  kernel<<<l.grid, l.block, 0, (cudaStream_t)stream>>>(x, C, g, y);
   return launched();
 }
 
@@ -284,7 +305,9 @@ fwi_status fwi_nn_upsample2_backward(const float *dy, int C, int D, int H, int W
                                      void *stream) {
   if (!dy || !dx || !sizes_ok(C, 1, D, H, W)) return FWI_E_INVAL;
   const Cells g = cells(D, H, W);
-  up2_bwd_kernel<<<plane_grid(C, g.Dc, g.Hc, g.Wc), kT, 0, (cudaStream_t)stream>>>(dy, C, g, accumulate != 0, dx);
+  const PlaneLaunch l = plane_launch(C, g.Dc, g.Hc, g.Wc);
+  const auto kernel = l.block.y > 1 ? up2_bwd_kernel<true> : up2_bwd_kernel<false>;
+  kernel<<<l.grid, l.block, 0, (cudaStream_t)stream>>>(dy, C, g, accumulate != 0, dx);
   return launched();
 }
 
