@@ -219,7 +219,7 @@ __device__ __forceinline__ float stage_value(const StageArgs &a, float x, float 
   if constexpr (MODE == 0) return rate;
   if constexpr (MODE == 1) return __fmaf_rn(a.cdt, rate, yv);
   if constexpr (MODE == 2) return __fmaf_rn(a.cdt, rate, x);
-  return __fmaf_rn(a.cdt, rate, __fmul_rn(x + yv, 1.f / 3.f));  // the third rounded by itself, as in fwi_internal.h
+  return stage4(x + yv, a.cdt, rate);
 }
 
 // write the stage outputs of one interior node

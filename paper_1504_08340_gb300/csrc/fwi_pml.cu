@@ -188,9 +188,8 @@ __device__ __forceinline__ float2 stage2(const StageArgs &a, float2 x, float2 y,
   if constexpr (MODE == 0) return r;
   if constexpr (MODE == 1) return pfma(bc(a.cdt), r, y);
   if constexpr (MODE == 2) return pfma(bc(a.cdt), r, x);
-  // the third is fused here, unlike in the node lists and the interior (stage_value): sweeps on
-  // eight meshes are 0.5e-6 to 2.2e-6 off their 64-bit values
-  return pfma(bc(1.f / 3.f), padd(x, y), pmul(bc(a.cdt), r));
+  const float2 s = padd(x, y), q = pmul(s, bc(1.f / 3.f));  // as stage4
+  return pfma(bc(a.cdt), r, pfma(pfma(bc(-3.f), q, s), bc(1.f / 3.f), q));
 }
 // the step-start values of three variables from field f on, loaded together: a.out may be a.X, so
 // the compiler keeps these loads behind the stores of the variables before, and each group waits
