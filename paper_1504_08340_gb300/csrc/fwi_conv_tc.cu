@@ -277,6 +277,11 @@ constexpr int kTileThreads = 288;
 constexpr int kRingB = 4;      // most weight copies in flight
 constexpr int kMaxPlanes = 4;  // output planes of a block
 constexpr int kMaxBox = 2;     // box buffers (passes in flight)
+// blocks of 288 threads that an SM's registers hold, forward and backward data: the kernel's launch
+// bound, and what tile_shape counts with. With three assumed for the forward, which takes 85
+// registers, a grid had 456 blocks of which 304 ran, then 152 alone with a third of the tiles:
+// 8 -> 16 channels at 65 x 129 x 129 voxels 193 us, 97 with two; 28 -> 2 at 33 x 65 x 65 36.9 and 31.3.
+constexpr int kTileBlocks[2] = {2, 3};
 
 struct TileShape {
   int nt_n, ntiles;  // GEMM output channels per block, N tiles
@@ -329,7 +334,7 @@ __global__ void __launch_bounds__(256) tile_prep_kernel(const void *__restrict__
 }
 
 template <bool BWD>
-__global__ void __launch_bounds__(kTileThreads, 2)
+__global__ void __launch_bounds__(kTileThreads, kTileBlocks[BWD])
     tile_conv_kernel(const __grid_constant__ CUtensorMap tm, const uint16_t *__restrict__ wpack,
                      const float *__restrict__ bias, int n_out, TileShape ts, int D, int H, int W, int relu,
                      void *__restrict__ yout) {
@@ -554,9 +559,9 @@ int pow2_cols(int n) {
   return c;
 }
 
-// shapes of the tile form for n_rows output channels and `groups` channel groups; false when
-// no shape fits
-bool tile_shape(int n_rows, int groups, int64_t tiles_xy, int D, TileShape *out) {
+// shapes of the tile form for n_rows output channels and `groups` channel groups, on an SM whose
+// registers hold reg_blocks blocks; false when no shape fits
+bool tile_shape(int n_rows, int groups, int64_t tiles_xy, int D, int reg_blocks, TileShape *out) {
   const int n16 = (n_rows + 15) / 16 * 16;
   TileShape ts{};
   ts.nt_n = n16 < kMaxN ? n16 : kMaxN;
@@ -589,7 +594,7 @@ bool tile_shape(int n_rows, int groups, int64_t tiles_xy, int D, TileShape *out)
             // allocation never waits
             const int floor_smem = kSmPerSM / (kTmemCols / cols + 1) - 1024 + 16;
             if (smem < floor_smem) smem = floor_smem;
-            const int occ = std::min({kTmemCols / cols, kSmPerSM / (smem + 2560), 65536 / (kTileThreads * 64)});
+            const int occ = std::min({kTmemCols / cols, kSmPerSM / (smem + 2560), reg_blocks});
             const int64_t tiles = tiles_xy * ((D + planes - 1) / planes) * ts.ntiles;
             // a model in SM clocks: an MMA of M = 128, K = 16 reads 4 KB of A and 32 nt_n bytes of B
             // at 128 B per clock or computes nt_n / 2 clocks, and its issue takes about 110 clocks of
@@ -642,7 +647,7 @@ cudaError_t run_tile(const void *in, const uint16_t *w, const float *b, int n_ro
   const int64_t nv = (int64_t)D * H * W;
   const int64_t tiles_xy = (int64_t)((W + kTX - 1) / kTX) * ((H + kTY - 1) / kTY);
   TileShape ts;
-  if (tiles_xy > 0x7fffffff || D > 65535 || !tile_shape(n_rows, groups, tiles_xy, D, &ts) || ts.ntiles > 65535)
+  if (tiles_xy > 0x7fffffff || D > 65535 || !tile_shape(n_rows, groups, tiles_xy, D, kTileBlocks[BWD], &ts) || ts.ntiles > 65535)
     return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(tile_conv_kernel<BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmBlock);
   if (e != cudaSuccess) return e;

@@ -55,3 +55,27 @@ def test_block_walks_over_channel_tiles(many, few, shape):
     dw_ref, db_ref = P.conv3d_backward_weight(dy.astype(np.float64), xv)
     assert rel_l2(dw.cpu().numpy(), dw_ref) < 1e-5
     assert rel_l2(db.cpu().numpy(), db_ref) < 1e-5
+
+
+def test_fewer_channels_take_no_longer():
+    # 8 -> 16 channels are a seventh of the work of 28 -> 28. With a grid of more blocks than the GPU holds
+    # at once, each owning its share of the tiles, they took a third longer.
+    lib = _lib()
+    shape = (65, 129, 129)
+
+    def best(cin, cout):
+        x = torch.zeros((cin, *shape), dtype=torch.bfloat16, device="cuda")
+        w = torch.zeros((cout, cin, 27), dtype=torch.bfloat16, device="cuda")
+        y = torch.empty((cout, *shape), dtype=torch.bfloat16, device="cuda")
+        ms = []
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(10):
+                assert lib.fwi_nn_conv3d_forward(_p(x), _p(w), None, cin, cout, *shape, 1, _p(y), _s()) == 0
+            b.record()
+            b.synchronize()
+            ms.append(a.elapsed_time(b))
+        return min(ms)
+
+    assert best(8, 16) < best(28, 28)
