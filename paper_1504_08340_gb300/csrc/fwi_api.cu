@@ -360,7 +360,7 @@ fwi_status stage(fwi_ctx *c, bool adj, const fwi::StageArgs &a, const fwi::Point
   for (int i = 0; i < kSides; i++) CUDA_TRY(c, cudaStreamWaitEvent(c->side[i], c->ev_fork, 0));
   // the interior last: its blocks, launched first, fill the SMs' registers and shared memory and
   // the others, which take longer on small meshes, start behind them (a graph's replay, 19x38x5
-  // elements with 2 PML elements, two shots: a gradient in 54.7 ms with the interior first, 32.3 last)
+  // elements with 2 PML elements, two shots: a gradient in 52.8 ms with the interior first, 33.1 last)
   int nk = fwi::launch_shell(c->geo, a, q, adj, c->side[1]) + fwi::launch_pml_face(c->geo, a, q, adj, c->side[1]) +
            fwi::launch_pml(c->geo, a, adj, c->stream);
   nk += fwi::launch_interior(c->geo, a, q, map, c->side[0]);
@@ -380,9 +380,10 @@ fwi_status stage(fwi_ctx *c, bool adj, const fwi::StageArgs &a, const fwi::Point
   return FWI_OK;
 }
 
-// nodes of all shots of a launch up to which the stage kernels apply the points (see Points;
-// at 2.4 M nodes, 64x64x32, fused 75.0 against 75.8 ms, at 25 M, four shots of 96x96x48, 277.1
-// against 274.9 ms)
+// nodes of all shots of a launch up to which the stage kernels apply the points (see Points).
+// Gradients with the points fused / in their own kernel: 2.4 M nodes (64x64x32) 25.06 / 25.29 ms, 3.2 M
+// (16 shots of 16x16x8) 32.39 / 32.59, 7.3 M 66.52 / 66.55, 9.7 M 85.88 / 85.79, 12.7 M (two shots of
+// 96x96x48) 110.75 / 110.35
 constexpr int64_t kFusedNodes = 8000000;
 
 // the sources of the shots from shot0 on as load 1
@@ -731,6 +732,8 @@ fwi_status fwi_create(const fwi_config *cfg, fwi_ctx **out) {
   g.stride = (px * nJ * nK + 63) / 64 * 64;
   g.inv_h = (float)(1.0 / cfg->h);
   g.rho = (float)cfg->rho;
+  // most planes per block of the interior kernel; 32, 16, 8 and 4 as launched now: 64x64x32 gradient with four
+  // shots 163.1, 164.9, 165.3, 166.0 ms, 96x96x48 forward with eight 160.0, 160.3, 160.5, 159.9
   g.int_kc = 32;
   g.pml_seg = 32;
   g.inv_rho_h = (float)(1.0 / (cfg->rho * cfg->h));

@@ -17,8 +17,9 @@
 // the no-swizzle canonical layouts (8 rows of 16 bytes stored contiguously; LBO is the
 // byte stride between core matrices along K and SBO along M or N, in K-major and MN-major
 // operands). So the taps are shifted views of the box: no thread gathers anything. One
-// thread issues the tcgen05.mma and commits them to mbarriers, one the copies; the
-// epilogue reads the accumulators with tcgen05.ld.
+// elected lane per warp issues tcgen05.mma and commits them to mbarriers, a warp per plane
+// (forward, data) or per tap (weight gradient); another issues the copies; the epilogue reads
+// the accumulators with tcgen05.ld.
 //
 // Every mbarrier wait is bounded (about a second). A block whose wait gives up waits
 // (bounded) for what it issued, writes NaN to its outputs (so the caller's loss turns
@@ -33,13 +34,14 @@
 #include <type_traits>
 
 #include "fwi_conv_tc.h"
+#include "fwi_internal.h"  // kSms
 
 namespace fwi_tc {
 namespace {
 
+using fwi::kSms;
 constexpr int kM = 128;           // MMA M: the voxels of a tile, or the gradient rows of the weight gradient
 constexpr int kMaxN = 256;        // output channels per block (MMA N <= 256)
-constexpr int kSms = 152;
 constexpr int kSmPerSM = 233472;  // shared memory of an SM (228 KB); 1 KB more is reserved per block
 constexpr int kSmBlock = 230400;  // dynamic shared memory a block can have beside 2 KB of static
 constexpr int kTmemCols = 512;    // TMEM columns of an SM
@@ -738,12 +740,15 @@ struct WgShape {
 };
 
 // x alone, for grids where the two copies' own launches cost nothing: wgrad_prep_kernel's shared
-// memory leaves its x blocks fewer on an SM (65 x 129 x 129 voxels: 332 against 327 us a call)
+// memory leaves its x blocks fewer on an SM
 __global__ void __launch_bounds__(256) group_major_kernel(const uint16_t *__restrict__ x, int64_t nv, int cin,
                                                           uint16_t *__restrict__ src, int nx) {
   group_major_block(x, nv, cin, src, blockIdx.x, nx);
 }
-constexpr int64_t kPrepVoxels = 1 << 18;  // voxels up to which the two copies are one launch
+// Voxels up to which the two copies are one launch. One launch against two, 28 and 56 channels: 17 x 33 x
+// 33 voxels 31.6 / 33.7 and 45.7 / 48.7 us a call, 49 x 97 x 97 (461 thousand) 157.0 / 160.9 and 475.0 /
+// 477.0, 65 x 129 x 129 (1.08 million) 338.4 / 339.7 and 1023.4 / 1021.9.
+constexpr int64_t kPrepVoxels = 1 << 18;
 
 // the copies of a weight gradient: blocks below nsrc x, the others the gradient tiles
 __global__ void __launch_bounds__(256) wgrad_prep_kernel(const float *__restrict__ dy, const uint16_t *__restrict__ x,

@@ -19,7 +19,7 @@ constexpr int kLevelFields = 9;
 // of range is read or written; the call then returns FWI_E_BOUNDS. In the normal build
 // guard() is the constant true and the checks compile away.
 enum BoundsSite {
-  kSiteShell = 1, kSiteFace = 2, kSitePml = 3, kSiteInterior = 4, kSitePoint = 5, kSiteSample = 6,
+  kSiteShell = 1, kSiteFace = 2, kSitePml = 3, kSiteInterior = 4, kSitePoint = 5,
   kSiteGradient = 7, kSiteSnapshot = 8, kSitePersist = 9
 };
 #ifdef FWI_BOUNDS_CHECK
@@ -127,7 +127,7 @@ inline int chunk_planes(int64_t tiles, int planes, int slots, int most, double s
   }
   return best;
 }
-constexpr int kSms = 152;
+constexpr int kSms = 152;  // SMs of the GPU
 
 // the buffers of shot `shot` of the batch
 __host__ __device__ inline StageArgs shot_args(StageArgs a, int shot) {

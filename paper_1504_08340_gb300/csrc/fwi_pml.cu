@@ -664,8 +664,9 @@ static Region pml_region(const Geo &g) {
     r.nseg[b] = (r.P[b] + kSegWarps * g.pml_seg - 1) / (kSegWarps * g.pml_seg);
     r.per[b] = (r.P[b] + r.nseg[b] - 1) / r.nseg[b];
     // packed rows keep every lane busy, but a warp's row loads then break at row ends: worth it
-    // below kPackBelow of 32 lanes (18 of 32 lanes, 16x16x8 elements: a gradient in 36.7 ms
-    // unpacked, 30.6 ms packed; 29 of 32, 96x96x48, four shots: 276.0 against 279.5 ms)
+    // below kPackBelow of 32 lanes. Forward sweeps of 40 x 20 elements in (y, z), the rows across the
+    // grid unpacked / packed, 4 PML elements: 18 pairs 10.57 / 10.29 ms, 22 12.77 / 12.39, 26 12.66 / 12.64, 28
+    // 12.49 / 12.62, 30 14.92 / 14.80, 31 14.99 / 15.07; 10 PML elements: 26 16.73 / 16.42, 28 17.08 / 16.52, 30 19.93 / 20.2
     r.packed[b] = r.per[b] < kPackBelow || r.per[b] > 32;
     int per_plane = 0;
     for (int c = 0; c < 2; c++) {
