@@ -748,7 +748,7 @@ __global__ void __launch_bounds__(256) group_major_kernel(const uint16_t *__rest
 // Voxels up to which the two copies are one launch. One launch against two, 28 and 56 channels: 17 x 33 x
 // 33 voxels 31.6 / 33.7 and 45.7 / 48.7 us a call, 49 x 97 x 97 (461 thousand) 157.0 / 160.9 and 475.0 /
 // 477.0, 65 x 129 x 129 (1.08 million) 338.4 / 339.7 and 1023.4 / 1021.9.
-constexpr int64_t kPrepVoxels = 1 << 18;
+constexpr int64_t kPrepVoxels = 1 << 20;
 
 // the copies of a weight gradient: blocks below nsrc x, the others the gradient tiles
 __global__ void __launch_bounds__(256) wgrad_prep_kernel(const float *__restrict__ dy, const uint16_t *__restrict__ x,
