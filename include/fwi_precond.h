@@ -69,8 +69,9 @@ int64_t fwi_nn_conv3d_backward_weight_work(int cin, int cout, int D, int H, int 
  * per slice of at most 6144 voxels the products of dy, taken as three BF16 parts per value
  * (so they keep FP32 accuracy; each part has its own FP32 sum), with the shifted tiles of x,
  * the parts' sums into `work`, then the slices added in order. Copies of x (group-major) and
- * of the split dy (tile-ordered), and on small grids the partial sums, are allocated and freed
- * in stream order. A non-finite x makes the taps that use it non-finite, and no others.
+ * of the split dy (tile-ordered), and on small or thin grids the partial sums, are allocated
+ * and freed in stream order. A non-finite x makes the taps that use it non-finite, and no
+ * others. FWI_E_INVAL for grids of more than 65535 * 2048 voxels.
  * dy: FP32 [cout][D][H][W]; x: BF16 [cin][D][H][W]; dw: FP32 [cout][cin][27];
  * db: FP32 [cout] or null; work: FP32 scratch (fwi_nn_conv3d_backward_weight_work). */
 fwi_status fwi_nn_conv3d_backward_weight(const float *dy, const uint16_t *x, int cin, int cout, int D, int H, int W,
