@@ -20,7 +20,7 @@
 #include "../../include/fwi.h"
 #include "fwi_internal.h"
 
-// Side streams of a stage: interior; interface shell, then outer-face nodes. With the faces on a
+// Side streams of a stage: bulk PML; interface shell, then outer-face nodes. With the faces on a
 // third, a 16x16x8 sweep of 2000 steps replays in 257 ms instead of 272, but instantiating its
 // graph, in which every kernel of a stage then waits for four, takes 0.47 s instead of 0.20, and
 // direct launches are slower too (37x23x18 gradient 77.8 against 74.7 ms).
@@ -111,7 +111,8 @@ struct fwi_ctx {
   int bar_extra = 0;
   int *d_all = nullptr, *d_rec_of = nullptr;  // every node; node -> receiver index, or -1 (see Points)
   unsigned *d_bar = nullptr;
-  int *d_status = nullptr;                    // FWI_E_TIMEOUT when a bounded device wait gave up
+  int *d_status = nullptr;                    // [0]: FWI_E_TIMEOUT when a bounded device wait gave up
+  bool side_used = false;                     // the side streams have had work (see stage)
 
   bool timing = false;
   std::vector<cudaEvent_t> ev_free;
@@ -353,17 +354,29 @@ fwi_status stage(fwi_ctx *c, bool adj, const fwi::StageArgs &a, const fwi::Point
   fwi::PlaneMap map;
   if (!fwi::plane_map(c->geo, a, &map))
     return fail(c, FWI_E_CUDA, "no tensor map for the stage input (not 16-byte aligned, or no driver entry)");
+  // A stream gets its hardware queue at its first work. Where the first stage's launches gave them,
+  // a process's first context ran the slower of two ways (37x23x18 elements launched directly: 83 ms,
+  // 73.8 with the queues taken here, in this order). Contexts that only replay graphs take none:
+  // with idle queues beside them, their replays were 2 % slower (16x16x8 29.0 against 28.5 ms).
+  if (!c->side_used && c->stream != c->cap) {
+    for (int i = 0; i < kSides; i++) CUDA_TRY(c, cudaMemsetAsync(c->d_status + 1, 0, sizeof(int), c->side[i]));
+    c->side_used = true;
+  }
   cudaEvent_t e0;
   time_begin(c, &e0);
-  // fork: interior and interface/face kernels on the side streams, bulk PML here
+  // fork: PML and interface/face kernels on the side streams, interior here
   CUDA_TRY(c, cudaEventRecord(c->ev_fork, c->stream));
   for (int i = 0; i < kSides; i++) CUDA_TRY(c, cudaStreamWaitEvent(c->side[i], c->ev_fork, 0));
-  // the interior last: its blocks, launched first, fill the SMs' registers and shared memory and
-  // the others, which take longer on small meshes, start behind them (a graph's replay, 19x38x5
-  // elements with 2 PML elements, two shots: a gradient in 52.8 ms with the interior first, 33.1 last)
+  // the interior last, and on the stream of lowest priority: its blocks, when they come first, fill
+  // the SMs' registers and shared memory and the others, which take longer on small meshes, start
+  // behind them (a graph's replay, 19x38x5 elements with 2 PML elements, two shots: a gradient in
+  // 52.8 ms with the interior first, 33.1 last). Launched directly, the order alone leaves the
+  // start to the streams' hardware queues, and a pass had one of two speeds: 37x23x18 elements 74.5 or
+  // 89 ms, with the priorities and the queues taken as above 73.8 from pass to pass; 16x16x8 31.5 or
+  // 39, now 31.7; 50x40x20 with 4 PML elements 28.5 or 34, now 29.6
   int nk = fwi::launch_shell(c->geo, a, q, adj, c->side[1]) + fwi::launch_pml_face(c->geo, a, q, adj, c->side[1]) +
-           fwi::launch_pml(c->geo, a, adj, c->stream);
-  nk += fwi::launch_interior(c->geo, a, q, map, c->side[0]);
+           fwi::launch_pml(c->geo, a, adj, c->side[0]);
+  nk += fwi::launch_interior(c->geo, a, q, map, c->stream);
   for (int i = 0; i < kSides; i++) {
     CUDA_TRY(c, cudaEventRecord(c->ev_join[i], c->side[i]));
     CUDA_TRY(c, cudaStreamWaitEvent(c->stream, c->ev_join[i], 0));
@@ -775,8 +788,10 @@ fwi_status fwi_create(const fwi_config *cfg, fwi_ctx **out) {
     }
   }
   fwi_status st = FWI_OK;
+  int least = 0, greatest = 0;  // priorities: the side streams before the interior kernel's (see stage)
+  if (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess) st = fail(c, FWI_E_CUDA, "stream setup failed");
   for (int i = 0; i < kSides && st == FWI_OK; i++)
-    if (cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking) != cudaSuccess ||
+    if (cudaStreamCreateWithPriority(&c->side[i], cudaStreamNonBlocking, greatest) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_join[i], cudaEventDisableTiming) != cudaSuccess)
       st = fail(c, FWI_E_CUDA, "stream setup failed");
   if (st == FWI_OK && cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess)
@@ -856,8 +871,8 @@ fwi_status fwi_create(const fwi_config *cfg, fwi_ctx **out) {
     st = fail(c, FWI_E_CUDA, "error word clear failed");
 #endif
   g.oob = c->d_oob;
-  if (st == FWI_OK) st = dalloc(c, &c->d_status, 1);
-  if (st == FWI_OK && cudaMemset(c->d_status, 0, sizeof(int)) != cudaSuccess)
+  if (st == FWI_OK) st = dalloc(c, &c->d_status, 2);
+  if (st == FWI_OK && cudaMemset(c->d_status, 0, 2 * sizeof(int)) != cudaSuccess)
     st = fail(c, FWI_E_CUDA, "status word clear failed");
   g.status = c->d_status;
   g.wait_cycles = (long long)(1000.0 * 1e-3 * 2.2e9);  // about a second
