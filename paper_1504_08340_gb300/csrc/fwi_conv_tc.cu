@@ -279,10 +279,10 @@ constexpr int kTileThreads = 288;
 constexpr int kRingB = 4;      // most weight copies in flight
 constexpr int kMaxPlanes = 4;  // output planes of a block
 constexpr int kMaxBox = 2;     // box buffers (passes in flight)
-// blocks of 288 threads that an SM's registers hold, forward and backward data: the kernel's launch
-// bound, and what tile_shape counts with. With three assumed for the forward, which takes 85
-// registers, a grid had 456 blocks of which 304 ran, then 152 alone with a third of the tiles:
-// 8 -> 16 channels at 65 x 129 x 129 voxels 193 us, 97 with two; 28 -> 2 at 33 x 65 x 65 36.9 and 31.3.
+// blocks of 288 threads that an SM's registers hold, forward (85 registers a thread) and backward data
+// (72; held to 66 by a launch bound of three blocks it is up to 2.5 % slower). With three assumed for
+// the forward, a grid had 456 blocks of which 304 ran, then 152 alone with a third of the tiles: 8 -> 16
+// channels at 65 x 129 x 129 voxels 193 us, 97 with two; 28 -> 2 at 33 x 65 x 65 36.9 and 31.3.
 constexpr int kTileBlocks[2] = {2, 3};
 
 struct TileShape {
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(256) tile_prep_kernel(const void *__restrict__
 }
 
 template <bool BWD>
-__global__ void __launch_bounds__(kTileThreads, kTileBlocks[BWD])
+__global__ void __launch_bounds__(kTileThreads, 2)
     tile_conv_kernel(const __grid_constant__ CUtensorMap tm, const uint16_t *__restrict__ wpack,
                      const float *__restrict__ bias, int n_out, TileShape ts, int D, int H, int W, int relu,
                      void *__restrict__ yout) {
