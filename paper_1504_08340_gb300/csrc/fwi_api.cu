@@ -366,7 +366,8 @@ fwi_status stage(fwi_ctx *c, bool adj, const fwi::StageArgs &a, const fwi::Point
   time_begin(c, &e0);
   // fork: PML and interface/face kernels on the side streams, interior here
   CUDA_TRY(c, cudaEventRecord(c->ev_fork, c->stream));
-  for (int i = 0; i < kSides; i++) CUDA_TRY(c, cudaStreamWaitEvent(c->side[i], c->ev_fork, 0));
+  const int first = c->cfg.npml > 0 ? 0 : 1;  // without a PML the first has no kernel
+  for (int i = first; i < kSides; i++) CUDA_TRY(c, cudaStreamWaitEvent(c->side[i], c->ev_fork, 0));
   // the interior last, and on the stream of lowest priority: its blocks, when they come first, fill
   // the SMs' registers and shared memory and the others, which take longer on small meshes, start
   // behind them (a graph's replay, 19x38x5 elements with 2 PML elements, two shots: a gradient in
@@ -377,7 +378,7 @@ fwi_status stage(fwi_ctx *c, bool adj, const fwi::StageArgs &a, const fwi::Point
   int nk = fwi::launch_shell(c->geo, a, q, adj, c->side[1]) + fwi::launch_pml_face(c->geo, a, q, adj, c->side[1]) +
            fwi::launch_pml(c->geo, a, adj, c->side[0]);
   nk += fwi::launch_interior(c->geo, a, q, map, c->stream);
-  for (int i = 0; i < kSides; i++) {
+  for (int i = first; i < kSides; i++) {
     CUDA_TRY(c, cudaEventRecord(c->ev_join[i], c->side[i]));
     CUDA_TRY(c, cudaStreamWaitEvent(c->stream, c->ev_join[i], 0));
   }
